@@ -239,7 +239,7 @@ dwt2d_status check_buffers(const dwt2d_plan_s* p, const void* src, int64_t sp, c
 
 // Warps of a streaming kernel resident per SM (their register budgets).
 int resident_per_sm(bool fwd, int nl, int q1, int scheme) {
-    if (fwd) return q1 <= 2 ? 16 : (nl <= 2 ? 12 : 8);
+    if (fwd) return nl >= 3 ? 8 : (q1 >= 4 && scheme == SCH_NONSEP ? 12 : 16);
     return q1 <= 2 ? (scheme == SCH_NONSEP ? 12 : 16) : 12;
 }
 
@@ -774,13 +774,13 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     // per SM (3 waves of 16) for CDF 9/7 and at 44 for LeGall 5/3 (its
     // shorter halo) with 2 columns per lane, at 24 (2 waves of 12) with 4;
     // the small later ones at one wave
-    const int fwl = opt(o.fwd_warps_per_sm_large, wavelet == DWT2D_CDF97 ? 48 : 44);
+    const int fwl = opt(o.fwd_warps_per_sm_large, wavelet == DWT2D_CDF97 ? 48 : 64);
     p->fwd_warps_large = (tuning && tuning->warps_per_sm > 0) || fwl < 0 ? 0 : sms * fwl;
-    const int fwl4 = opt(o.fwd_warps_per_sm_large, 24);
+    const int fwl4 = opt(o.fwd_warps_per_sm_large, 32);
     p->fwd_warps_large4 = (tuning && tuning->warps_per_sm > 0) || fwl4 < 0 ? 0 : sms * fwl4;
     p->large_segq = opt(o.large_segment, 16);
     // the finest inverse launch: 64 warps per SM (4 waves of 16)
-    const int iwl = opt(o.inv_warps_per_sm_large, 64);
+    const int iwl = opt(o.inv_warps_per_sm_large, half ? 32 : (wavelet == DWT2D_CDF97 ? 64 : 80));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;
     p->fwd_q1 = o.fwd_cols_per_lane;  // 0: automatic
     p->pdl = opt(o.programmatic_launch, 1) > 0;
@@ -790,7 +790,7 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     // lane, 4 at 4) and 2 % (inverse, 4) faster at 8192^2
     p->fwd_short = o.fwd_short_tail < 0 ? 0 : opt(o.fwd_short_tail, 3);
     p->fwd_short4 = o.fwd_short_tail < 0 ? 0 : opt(o.fwd_short_tail, 4);
-    p->inv_short = o.inv_short_tail < 0 ? 0 : opt(o.inv_short_tail, 4);
+    p->inv_short = o.inv_short_tail < 0 ? 0 : opt(o.inv_short_tail, wavelet == DWT2D_CDF97 ? 4 : 3);
     p->host_bands = opt(o.host_bands, 8);
     p->host_pipeline = opt(o.host_pipeline, 1) > 0;
     p->inv_q1 = o.inv_cols_per_lane == 4 ? 4 : 2;

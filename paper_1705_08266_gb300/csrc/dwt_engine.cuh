@@ -29,6 +29,25 @@ namespace dwt {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// How much of the border an instantiation handles.  kInner: none, and both
+// axes are active, so the coefficients are compile-time constants.  kEdgeRows:
+// rows at the top and the bottom and inactive axes; columns past the border
+// hold mirrored data, so that they need no code (the lifting steps are
+// symmetric bit for bit: a mirrored signal stays mirrored).  kEdgeAll: columns
+// too, by a select at every neighbour (kernels that load bands directly).
+enum Border { kInner = 0, kEdgeRows = 1, kEdgeAll = 2 };
+
+// Whole-sample symmetric extension of an axis of n samples: the sample that
+// position x (possibly outside) takes.
+__device__ __forceinline__ int reflect(int x, int n) {
+    if (n == 1) return 0;
+    while (x < 0 || x >= n) {
+        x = x < 0 ? -x : x;
+        x = x >= n ? 2 * (n - 1) - x : x;
+    }
+    return x;
+}
+
 template <class T, int Q>
 struct Quads {
     T c[4][Q];  // c[component][column within lane]
@@ -231,10 +250,7 @@ struct LevelCtx {
     float s[4];      // scale of LL, HL, LH, HH (forward) or its inverse (inverse)
 };
 
-__device__ __forceinline__ LevelCtx make_ctx(int g0, int Q, int h, int w, int lane_lo,
-                                             int lane_hi, const float* s) {
-    (void)lane_lo;
-    (void)lane_hi;
+__device__ __forceinline__ LevelCtx make_ctx(int g0, int Q, int h, int w, const float* s) {
     LevelCtx x;
     const int ne_c = (w + 1) >> 1, no_c = w >> 1;
     x.right = x.left = x.odd = 0u;
@@ -267,27 +283,35 @@ __device__ __forceinline__ T shfl_up(T v) {
     return __shfl_up_sync(kFull, v, 1);
 }
 
-// R[j] = v at column j+1, mirrored at the right border (EDGE) or not (interior).
-template <bool EDGE, class T, int Q>
-__device__ __forceinline__ void right_nb(const T (&v)[Q], T (&R)[Q], unsigned m) {
-    const T n = shfl_dn(v[0]);
+// R[j] = v at column j+1, mirrored at the right border (kEdgeAll) or not;
+// n: the next lane's first value.
+template <int E, class T, int Q>
+__device__ __forceinline__ void right_of(const T (&v)[Q], T n, T (&R)[Q], unsigned m) {
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
         const T nb = (j + 1 < Q) ? v[j + 1] : n;
-        if (EDGE) R[j] = ((m >> j) & 1u) ? nb : v[j];
+        if (E == kEdgeAll) R[j] = ((m >> j) & 1u) ? nb : v[j];
         else R[j] = nb;
     }
 }
-// L[j] = v at column j-1, mirrored at the left border (EDGE) or not (interior).
-template <bool EDGE, class T, int Q>
-__device__ __forceinline__ void left_nb(const T (&v)[Q], T (&L)[Q], unsigned m) {
-    const T p = shfl_up(v[Q - 1]);
+template <int E, class T, int Q>
+__device__ __forceinline__ void right_nb(const T (&v)[Q], T (&R)[Q], unsigned m) {
+    right_of<E>(v, shfl_dn(v[0]), R, m);
+}
+// L[j] = v at column j-1, mirrored at the left border (kEdgeAll) or not;
+// p: the lane before's last value.
+template <int E, class T, int Q>
+__device__ __forceinline__ void left_of(const T (&v)[Q], T p, T (&L)[Q], unsigned m) {
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
         const T nb = (j > 0) ? v[j - 1] : p;
-        if (EDGE) L[j] = ((m >> j) & 1u) ? nb : v[j];
+        if (E == kEdgeAll) L[j] = ((m >> j) & 1u) ? nb : v[j];
         else L[j] = nb;
     }
+}
+template <int E, class T, int Q>
+__device__ __forceinline__ void left_nb(const T (&v)[Q], T (&L)[Q], unsigned m) {
+    left_of<E>(v, shfl_up(v[Q - 1]), L, m);
 }
 // Columns without odd samples take the odd sample of the column before.
 template <class T, int Q>
@@ -363,9 +387,7 @@ enum Kind { K_NONE = 0, K_DOWN = 1, K_UP = 2 };
 
 // ------------------------------------------------------------------ ops ----
 // Every op names its vertical dependency (kind) and whether it needs the own
-// odd samples mirrored horizontally before it runs (kHsub).  EDGE = false is
-// the interior form: no border substitution and both axes active, so the
-// coefficients are compile-time constants.
+// odd samples mirrored horizontally before it runs (kHsub).
 
 template <int ID, int SIGN>
 struct Coef;
@@ -378,186 +400,186 @@ struct Coef<2, SIGN> { static constexpr float v = SIGN * kGamma; };
 template <int SIGN>
 struct Coef<3, SIGN> { static constexpr float v = SIGN * kDelta; };
 
-template <bool EDGE>
-__device__ __forceinline__ float hcoef(float c, const LevelCtx& x) { return EDGE ? c * x.hf : c; }
-template <bool EDGE>
-__device__ __forceinline__ float vcoef(float c, const LevelCtx& x) { return EDGE ? c * x.vf : c; }
-template <bool EDGE>
-__device__ __forceinline__ bool hact(const LevelCtx& x) { return EDGE ? x.ha : true; }
-template <bool EDGE>
-__device__ __forceinline__ bool vact(const LevelCtx& x) { return EDGE ? x.va : true; }
+template <int E>
+__device__ __forceinline__ float hcoef(float c, const LevelCtx& x) { return E != kInner ? c * x.hf : c; }
+template <int E>
+__device__ __forceinline__ float vcoef(float c, const LevelCtx& x) { return E != kInner ? c * x.vf : c; }
+template <int E>
+__device__ __forceinline__ bool hact(const LevelCtx& x) { return E != kInner ? x.ha : true; }
+template <int E>
+__device__ __forceinline__ bool vact(const LevelCtx& x) { return E != kInner ? x.va : true; }
 
-// float, separable (Sec. 2 matrices)
-template <int ID, int SIGN, int PK>
+// float, separable (Sec. 2 matrices).  The vertical steps run as packed pairs
+// (c0, c1) / (c2, c3) of a quadruple, the horizontal ones scalar.
+template <int ID, int SIGN>
 struct OpFTH {
     static constexpr int kind = K_NONE;
-    template <bool EDGE, int Q>
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<float, Q>& a, const LevelCtx& x) {
         float c0r[Q], c2r[Q];
-        right_nb<EDGE>(a.c[0], c0r, x.right);
-        right_nb<EDGE>(a.c[2], c2r, x.right);
-        const float p = hcoef<EDGE>(Coef<ID, SIGN>::v, x);
-        if constexpr (PK != 0 && Q % 2 == 0) {
+        right_nb<E>(a.c[0], c0r, x.right);
+        right_nb<E>(a.c[2], c2r, x.right);
+        const float p = hcoef<E>(Coef<ID, SIGN>::v, x);
 #pragma unroll
-            for (int j = 0; j < Q / 2; ++j) {
-                float2 c1 = pk<PK, Q>(a.c[1], j), c3 = pk<PK, Q>(a.c[3], j);
-                f_TH(c1, c3, pk<PK, Q>(a.c[0], j), pk<PK, Q>(c0r, j), pk<PK, Q>(a.c[2], j), pk<PK, Q>(c2r, j), p);
-                unpk<PK, Q>(c1, a.c[1], j);
-                unpk<PK, Q>(c3, a.c[3], j);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < Q; ++j) f_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], p);
-        }
+        for (int j = 0; j < Q; ++j) f_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], p);
     }
 };
-template <int ID, int SIGN, int PK>
+template <int ID, int SIGN>
 struct OpFTV {
     static constexpr int kind = K_DOWN;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = false;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<float, Q>& a, const float (&n0)[Q],
-                                                 const float (&n1)[Q], const LevelCtx& x) {
-        const float p = vcoef<EDGE>(Coef<ID, SIGN>::v, x);
-        if constexpr (PK != 0 && Q % 2 == 0) {
+                                                 const float (&n1)[Q], float, float,
+                                                 const LevelCtx& x) {
+        const float p = vcoef<E>(Coef<ID, SIGN>::v, x);
 #pragma unroll
-            for (int j = 0; j < Q / 2; ++j) {
-                float2 c2 = pk<PK, Q>(a.c[2], j), c3 = pk<PK, Q>(a.c[3], j);
-                f_TV(c2, c3, pk<PK, Q>(a.c[0], j), pk<PK, Q>(n0, j), pk<PK, Q>(a.c[1], j), pk<PK, Q>(n1, j), p);
-                unpk<PK, Q>(c2, a.c[2], j);
-                unpk<PK, Q>(c3, a.c[3], j);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < Q; ++j) f_TV(a.c[2][j], a.c[3][j], a.c[0][j], n0[j], a.c[1][j], n1[j], p);
-        }
+        for (int j = 0; j < Q; ++j)
+            v_part<true>(a.c[2][j], a.c[3][j], a.c[0][j], a.c[1][j], n0[j], n1[j], p);
     }
 };
-template <int ID, int SIGN, int PK>
+template <int ID, int SIGN>
 struct OpFSH {
     static constexpr int kind = K_NONE;
-    template <bool EDGE, int Q>
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<float, Q>& a, const LevelCtx& x) {
-        if (EDGE && x.need_hsub) {
+        if (E == kEdgeAll && x.need_hsub) {
             subst_odd(a.c[1], x.odd);
             subst_odd(a.c[3], x.odd);
         }
         float c1l[Q], c3l[Q];
-        left_nb<EDGE>(a.c[1], c1l, x.left);
-        left_nb<EDGE>(a.c[3], c3l, x.left);
-        const float u = hcoef<EDGE>(Coef<ID, SIGN>::v, x);
-        if constexpr (PK != 0 && Q % 2 == 0) {
+        left_nb<E>(a.c[1], c1l, x.left);
+        left_nb<E>(a.c[3], c3l, x.left);
+        const float u = hcoef<E>(Coef<ID, SIGN>::v, x);
 #pragma unroll
-            for (int j = 0; j < Q / 2; ++j) {
-                float2 c0 = pk<PK, Q>(a.c[0], j), c2 = pk<PK, Q>(a.c[2], j);
-                f_SH(c0, c2, pk<PK, Q>(a.c[1], j), pk<PK, Q>(c1l, j), pk<PK, Q>(a.c[3], j), pk<PK, Q>(c3l, j), u);
-                unpk<PK, Q>(c0, a.c[0], j);
-                unpk<PK, Q>(c2, a.c[2], j);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < Q; ++j) f_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], u);
-        }
+        for (int j = 0; j < Q; ++j) f_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], u);
     }
 };
-template <int ID, int SIGN, int PK>
+// PACK: 0 scalar (the last step of a chain, whose results go to other places
+// than the pair), 1 packed
+template <int ID, int SIGN, bool PACK>
 struct OpFSV {
     static constexpr int kind = K_UP;
     static constexpr bool kHsub = false;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = false;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<float, Q>& a, const float (&up2)[Q],
-                                                 const float (&up3)[Q], const LevelCtx& x) {
-        const float u = vcoef<EDGE>(Coef<ID, SIGN>::v, x);
-        if constexpr (PK != 0 && Q % 2 == 0) {
+                                                 const float (&up3)[Q], float, float,
+                                                 const LevelCtx& x) {
+        const float u = vcoef<E>(Coef<ID, SIGN>::v, x);
 #pragma unroll
-            for (int j = 0; j < Q / 2; ++j) {
-                float2 c0 = pk<PK, Q>(a.c[0], j), c1 = pk<PK, Q>(a.c[1], j);
-                f_SV(c0, c1, pk<PK, Q>(a.c[2], j), pk<PK, Q>(up2, j), pk<PK, Q>(a.c[3], j), pk<PK, Q>(up3, j), u);
-                unpk<PK, Q>(c0, a.c[0], j);
-                unpk<PK, Q>(c1, a.c[1], j);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < Q; ++j) f_SV(a.c[0][j], a.c[1][j], a.c[2][j], up2[j], a.c[3][j], up3[j], u);
-        }
+        for (int j = 0; j < Q; ++j)
+            v_part<PACK>(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], up2[j], up3[j], u);
     }
 };
 
-// float, non-separable (Sec. 3; RED = reduced form)
-template <int ID, int SIGN, bool RED, int PK>
+// float, non-separable, plain form (Sec. 3), on column pairs (PK = 1
+// adjacent, 2 strided; 0 scalar)
+template <int ID, int SIGN, int PK>
 struct OpFT {
     static constexpr int kind = K_DOWN;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = true;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<float, Q>& a, const float (&n0)[Q],
-                                                 const float (&n1)[Q], const LevelCtx& x) {
+                                                 const float (&n1)[Q], float c0n, float n0n,
+                                                 const LevelCtx& x) {
         float c0r[Q], c2r[Q], n0r[Q];
-        right_nb<EDGE>(a.c[0], c0r, x.right);
-        right_nb<EDGE>(a.c[2], c2r, x.right);
-        right_nb<EDGE>(n0, n0r, x.right);
-        const float ph = hcoef<EDGE>(Coef<ID, SIGN>::v, x), pv = vcoef<EDGE>(Coef<ID, SIGN>::v, x);
+        right_of<E>(a.c[0], c0n, c0r, x.right);
+        right_nb<E>(a.c[2], c2r, x.right);
+        right_of<E>(n0, n0n, n0r, x.right);
+        const float ph = hcoef<E>(Coef<ID, SIGN>::v, x), pv = vcoef<E>(Coef<ID, SIGN>::v, x);
         if constexpr (PK != 0 && Q % 2 == 0) {
 #pragma unroll
             for (int j = 0; j < Q / 2; ++j) {
                 float2 c1 = pk<PK, Q>(a.c[1], j), c2 = pk<PK, Q>(a.c[2], j), c3 = pk<PK, Q>(a.c[3], j);
-                if (RED)
-                    f_T_red(c1, c2, c3, pk<PK, Q>(a.c[0], j), pk<PK, Q>(c0r, j), pk<PK, Q>(c2r, j), pk<PK, Q>(n0, j), pk<PK, Q>(n1, j),
-                            pk<PK, Q>(n0r, j), ph, pv);
-                else
-                    f_T_plain(c1, c2, c3, pk<PK, Q>(a.c[0], j), pk<PK, Q>(c0r, j), pk<PK, Q>(c2r, j), pk<PK, Q>(n0, j), pk<PK, Q>(n1, j),
-                              pk<PK, Q>(n0r, j), ph, pv);
+                f_T_plain(c1, c2, c3, pk<PK, Q>(a.c[0], j), pk<PK, Q>(c0r, j), pk<PK, Q>(c2r, j),
+                          pk<PK, Q>(n0, j), pk<PK, Q>(n1, j), pk<PK, Q>(n0r, j), ph, pv);
                 unpk<PK, Q>(c1, a.c[1], j);
                 unpk<PK, Q>(c2, a.c[2], j);
                 unpk<PK, Q>(c3, a.c[3], j);
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                if (RED)
-                    f_T_red(a.c[1][j], a.c[2][j], a.c[3][j], a.c[0][j], c0r[j], c2r[j], n0[j], n1[j],
-                            n0r[j], ph, pv);
-                else
-                    f_T_plain(a.c[1][j], a.c[2][j], a.c[3][j], a.c[0][j], c0r[j], c2r[j], n0[j], n1[j],
-                              n0r[j], ph, pv);
-            }
+            for (int j = 0; j < Q; ++j)
+                f_T_plain(a.c[1][j], a.c[2][j], a.c[3][j], a.c[0][j], c0r[j], c2r[j], n0[j], n1[j], n0r[j],
+                          ph, pv);
         }
     }
 };
-template <int ID, int SIGN, bool RED, int PK>
+template <int ID, int SIGN, int PK>
 struct OpFS {
     static constexpr int kind = K_UP;
     static constexpr bool kHsub = true;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = true;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<float, Q>& a, const float (&up2)[Q],
-                                                 const float (&up3)[Q], const LevelCtx& x) {
+                                                 const float (&up3)[Q], float c3p, float u3p,
+                                                 const LevelCtx& x) {
         float c1l[Q], c3l[Q], u3l[Q];
-        left_nb<EDGE>(a.c[1], c1l, x.left);
-        left_nb<EDGE>(a.c[3], c3l, x.left);
-        left_nb<EDGE>(up3, u3l, x.left);
-        const float uh = hcoef<EDGE>(Coef<ID, SIGN>::v, x), uv = vcoef<EDGE>(Coef<ID, SIGN>::v, x);
+        left_nb<E>(a.c[1], c1l, x.left);
+        left_of<E>(a.c[3], c3p, c3l, x.left);
+        left_of<E>(up3, u3p, u3l, x.left);
+        const float uh = hcoef<E>(Coef<ID, SIGN>::v, x), uv = vcoef<E>(Coef<ID, SIGN>::v, x);
         if constexpr (PK != 0 && Q % 2 == 0) {
 #pragma unroll
             for (int j = 0; j < Q / 2; ++j) {
                 float2 c0 = pk<PK, Q>(a.c[0], j), c1 = pk<PK, Q>(a.c[1], j), c2 = pk<PK, Q>(a.c[2], j);
-                if (RED)
-                    f_S_red(c0, c1, c2, pk<PK, Q>(a.c[3], j), pk<PK, Q>(c1l, j), pk<PK, Q>(c3l, j), pk<PK, Q>(up2, j), pk<PK, Q>(up3, j),
-                            pk<PK, Q>(u3l, j), uh, uv);
-                else
-                    f_S_plain(c0, c1, c2, pk<PK, Q>(a.c[3], j), pk<PK, Q>(c1l, j), pk<PK, Q>(c3l, j), pk<PK, Q>(up2, j),
-                              pk<PK, Q>(up3, j), pk<PK, Q>(u3l, j), uh, uv);
+                f_S_plain(c0, c1, c2, pk<PK, Q>(a.c[3], j), pk<PK, Q>(c1l, j), pk<PK, Q>(c3l, j),
+                          pk<PK, Q>(up2, j), pk<PK, Q>(up3, j), pk<PK, Q>(u3l, j), uh, uv);
                 unpk<PK, Q>(c0, a.c[0], j);
                 unpk<PK, Q>(c1, a.c[1], j);
                 unpk<PK, Q>(c2, a.c[2], j);
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                if (RED)
-                    f_S_red(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], c1l[j], c3l[j], up2[j],
-                            up3[j], u3l[j], uh, uv);
-                else
-                    f_S_plain(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], c1l[j], c3l[j], up2[j],
-                              up3[j], u3l[j], uh, uv);
-            }
+            for (int j = 0; j < Q; ++j)
+                f_S_plain(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], c1l[j], c3l[j], up2[j], up3[j], u3l[j],
+                          uh, uv);
         }
+    }
+};
+
+// float, non-separable, reduced form: one spatial step of 8 multiply-adds per
+// quadruple.  The vertical part runs first, on whole quadruples (pairs); the
+// horizontal part then reads the neighbour's result of it by shuffle instead
+// of recomputing it (the ph pv n0r term of the split P0 + P1).
+template <int ID, int SIGN, bool PACK>
+struct OpRT {
+    static constexpr int kind = K_DOWN;
+    static constexpr bool kShare = false;
+    template <int E, int Q>
+    __device__ __forceinline__ static void apply(Quads<float, Q>& a, const float (&n0)[Q],
+                                                 const float (&n1)[Q], float, float,
+                                                 const LevelCtx& x) {
+        const float ph = hcoef<E>(Coef<ID, SIGN>::v, x), pv = vcoef<E>(Coef<ID, SIGN>::v, x);
+        float c0r[Q], c2r[Q];
+        right_nb<E>(a.c[0], c0r, x.right);
+#pragma unroll
+        for (int j = 0; j < Q; ++j)
+            v_part<PACK>(a.c[2][j], a.c[3][j], a.c[0][j], a.c[1][j], n0[j], n1[j], pv);
+        right_nb<E>(a.c[2], c2r, x.right);
+#pragma unroll
+        for (int j = 0; j < Q; ++j) f_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], ph);
+    }
+};
+template <int ID, int SIGN, bool PACK>
+struct OpRS {
+    static constexpr int kind = K_UP;
+    static constexpr bool kHsub = true;
+    static constexpr bool kShare = false;
+    template <int E, int Q>
+    __device__ __forceinline__ static void apply(Quads<float, Q>& a, const float (&up2)[Q],
+                                                 const float (&up3)[Q], float, float,
+                                                 const LevelCtx& x) {
+        const float uh = hcoef<E>(Coef<ID, SIGN>::v, x), uv = vcoef<E>(Coef<ID, SIGN>::v, x);
+        float c1l[Q], c3l[Q];
+        left_nb<E>(a.c[3], c3l, x.left);
+#pragma unroll
+        for (int j = 0; j < Q; ++j)
+            v_part<PACK>(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], up2[j], up3[j], uv);
+        left_nb<E>(a.c[1], c1l, x.left);
+#pragma unroll
+        for (int j = 0; j < Q; ++j) f_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], uh);
     }
 };
 
@@ -565,54 +587,56 @@ struct OpFS {
 template <int SIGN>
 struct OpITH {
     static constexpr int kind = K_NONE;
-    template <bool EDGE, int Q>
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<int, Q>& a, const LevelCtx& x) {
         int c0r[Q], c2r[Q];
-        right_nb<EDGE>(a.c[0], c0r, x.right);
-        right_nb<EDGE>(a.c[2], c2r, x.right);
+        right_nb<E>(a.c[0], c0r, x.right);
+        right_nb<E>(a.c[2], c2r, x.right);
 #pragma unroll
         for (int j = 0; j < Q; ++j)
-            i_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], hact<EDGE>(x), SIGN);
+            i_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], hact<E>(x), SIGN);
     }
 };
 template <int SIGN>
 struct OpITV {
     static constexpr int kind = K_DOWN;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = false;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<int, Q>& a, const int (&n0)[Q],
-                                                 const int (&n1)[Q], const LevelCtx& x) {
+                                                 const int (&n1)[Q], int, int, const LevelCtx& x) {
 #pragma unroll
         for (int j = 0; j < Q; ++j)
-            i_TV(a.c[2][j], a.c[3][j], a.c[0][j], n0[j], a.c[1][j], n1[j], vact<EDGE>(x), SIGN);
+            i_TV(a.c[2][j], a.c[3][j], a.c[0][j], n0[j], a.c[1][j], n1[j], vact<E>(x), SIGN);
     }
 };
 template <int SIGN>
 struct OpISH {
     static constexpr int kind = K_NONE;
-    template <bool EDGE, int Q>
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<int, Q>& a, const LevelCtx& x) {
-        if (EDGE && x.need_hsub) {
+        if (E == kEdgeAll && x.need_hsub) {
             subst_odd(a.c[1], x.odd);
             subst_odd(a.c[3], x.odd);
         }
         int c1l[Q], c3l[Q];
-        left_nb<EDGE>(a.c[1], c1l, x.left);
-        left_nb<EDGE>(a.c[3], c3l, x.left);
+        left_nb<E>(a.c[1], c1l, x.left);
+        left_nb<E>(a.c[3], c3l, x.left);
 #pragma unroll
         for (int j = 0; j < Q; ++j)
-            i_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], hact<EDGE>(x), SIGN);
+            i_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], hact<E>(x), SIGN);
     }
 };
 template <int SIGN>
 struct OpISV {
     static constexpr int kind = K_UP;
     static constexpr bool kHsub = false;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = false;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<int, Q>& a, const int (&up2)[Q],
-                                                 const int (&up3)[Q], const LevelCtx& x) {
+                                                 const int (&up3)[Q], int, int, const LevelCtx& x) {
 #pragma unroll
         for (int j = 0; j < Q; ++j)
-            i_SV(a.c[0][j], a.c[1][j], a.c[2][j], up2[j], a.c[3][j], up3[j], vact<EDGE>(x), SIGN);
+            i_SV(a.c[0][j], a.c[1][j], a.c[2][j], up2[j], a.c[3][j], up3[j], vact<E>(x), SIGN);
     }
 };
 
@@ -620,21 +644,23 @@ struct OpISV {
 template <bool FWD>
 struct OpIT {
     static constexpr int kind = K_DOWN;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = true;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<int, Q>& a, const int (&n0)[Q],
-                                                 const int (&n1)[Q], const LevelCtx& x) {
+                                                 const int (&n1)[Q], int c0n, int n0n,
+                                                 const LevelCtx& x) {
         int c0r[Q], c2r[Q], n0r[Q];
-        right_nb<EDGE>(a.c[0], c0r, x.right);
-        right_nb<EDGE>(a.c[2], c2r, x.right);
-        right_nb<EDGE>(n0, n0r, x.right);
+        right_of<E>(a.c[0], c0n, c0r, x.right);
+        right_nb<E>(a.c[2], c2r, x.right);
+        right_of<E>(n0, n0n, n0r, x.right);
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
             if (FWD)
                 i_T_fwd(a.c[1][j], a.c[2][j], a.c[3][j], a.c[0][j], c0r[j], c2r[j], n0[j], n1[j],
-                        n0r[j], hact<EDGE>(x), vact<EDGE>(x));
+                        n0r[j], hact<E>(x), vact<E>(x));
             else
                 i_T_inv(a.c[1][j], a.c[2][j], a.c[3][j], a.c[0][j], c0r[j], c2r[j], n0[j], n1[j],
-                        n0r[j], hact<EDGE>(x), vact<EDGE>(x));
+                        n0r[j], hact<E>(x), vact<E>(x));
         }
     }
 };
@@ -642,21 +668,23 @@ template <bool FWD>
 struct OpIS {
     static constexpr int kind = K_UP;
     static constexpr bool kHsub = true;
-    template <bool EDGE, int Q>
+    static constexpr bool kShare = true;
+    template <int E, int Q>
     __device__ __forceinline__ static void apply(Quads<int, Q>& a, const int (&up2)[Q],
-                                                 const int (&up3)[Q], const LevelCtx& x) {
+                                                 const int (&up3)[Q], int c3p, int u3p,
+                                                 const LevelCtx& x) {
         int c1l[Q], c3l[Q], u3l[Q];
-        left_nb<EDGE>(a.c[1], c1l, x.left);
-        left_nb<EDGE>(a.c[3], c3l, x.left);
-        left_nb<EDGE>(up3, u3l, x.left);
+        left_nb<E>(a.c[1], c1l, x.left);
+        left_of<E>(a.c[3], c3p, c3l, x.left);
+        left_of<E>(up3, u3p, u3l, x.left);
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
             if (FWD)
                 i_S_fwd(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], c1l[j], c3l[j], up2[j], up3[j],
-                        u3l[j], hact<EDGE>(x), vact<EDGE>(x));
+                        u3l[j], hact<E>(x), vact<E>(x));
             else
                 i_S_inv(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], c1l[j], c3l[j], up2[j], up3[j],
-                        u3l[j], hact<EDGE>(x), vact<EDGE>(x));
+                        u3l[j], hact<E>(x), vact<E>(x));
         }
     }
 };
@@ -671,55 +699,77 @@ struct Block {
     Quads<T, Q> r[RB];
 };
 
-template <class T, int Q, int KIND>
+// SHARE: the stage reads a neighbour lane's value of two rows (its own and the
+// lower / upper one); a row's value is exchanged once and kept for the row
+// that reads it next.
+template <class T, int Q, int KIND, bool SHARE>
 struct StageState {};
-template <class T, int Q>
-struct StageState<T, Q, K_DOWN> {
+template <class T, int Q, bool SHARE>
+struct StageState<T, Q, K_DOWN, SHARE> {
     Quads<T, Q> saved;  // the last input row of the previous block (pre-step)
+    T c0n;              // its c0 in the next lane's first column
 };
-template <class T, int Q>
-struct StageState<T, Q, K_UP> {
+template <class T, int Q, bool SHARE>
+struct StageState<T, Q, K_UP, SHARE> {
     T p2[Q], p3[Q];  // odd-row components of the previous block's last row (pre-step, mirrored)
+    T c3p;           // its c3 in the previous lane's last column
 };
 
-template <bool EDGE, class T, int Q, int RB, class Op>
-__device__ __forceinline__ void run_stage(StageState<T, Q, K_NONE>&, Block<T, Q, RB>& b, int&,
+template <class Op>
+__host__ __device__ constexpr bool op_share() {
+    if constexpr (Op::kind == K_NONE) return false;
+    else return Op::kShare;
+}
+
+template <int E, class T, int Q, int RB, class Op>
+__device__ __forceinline__ void run_stage(StageState<T, Q, K_NONE, false>&, Block<T, Q, RB>& b, int&,
                                           const LevelCtx& x) {
 #pragma unroll
-    for (int j = 0; j < RB; ++j) Op::template apply<EDGE>(b.r[j], x);
+    for (int j = 0; j < RB; ++j) Op::template apply<E>(b.r[j], x);
 }
 
 // A predict reading the lower row.  Input rows [r0, r0 + RB); output rows
 // [r0 - 1, r0 + RB - 1): row r0 - 1 (kept from the last block) completes now and
 // the last input row waits for the next block.
-template <bool EDGE, class T, int Q, int RB, class Op>
-__device__ __forceinline__ void run_stage(StageState<T, Q, K_DOWN>& st, Block<T, Q, RB>& b, int& r0,
-                                          const LevelCtx& x) {
-    const Quads<T, Q> keep = b.r[RB - 1];
+template <int E, class T, int Q, int RB, class Op, bool SHARE>
+__device__ __forceinline__ void run_stage(StageState<T, Q, K_DOWN, SHARE>& st, Block<T, Q, RB>& b,
+                                          int& r0, const LevelCtx& x) {
+    T sh[RB];
+    if constexpr (SHARE) {
 #pragma unroll
-    for (int j = RB - 1; j >= 0; --j) {
-        Quads<T, Q> o = (j > 0) ? b.r[j - 1] : st.saved;  // output row r0 - 1 + j
-        T n0[Q], n1[Q];                                     // its lower row, pre-step
+        for (int j = 0; j < RB; ++j) sh[j] = shfl_dn(b.r[j].c[0][0]);
+    }
+    Quads<T, Q> o = st.saved;  // output row r0 - 1 + j
+    T on{};
+    if constexpr (SHARE) on = st.c0n;
+#pragma unroll
+    for (int j = 0; j < RB; ++j) {
+        const Quads<T, Q> next = b.r[j];
+        T n0[Q], n1[Q], nn{};  // its lower row, pre-step
         // the lower row is past the last even row: mirror (the row itself)
-        const bool real = !EDGE || (r0 + j) < x.ne_r;
+        const bool real = E == kInner || (r0 + j) < x.ne_r;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            n0[i] = real ? b.r[j].c[0][i] : o.c[0][i];
-            n1[i] = real ? b.r[j].c[1][i] : o.c[1][i];
+            n0[i] = real ? next.c[0][i] : o.c[0][i];
+            n1[i] = real ? next.c[1][i] : o.c[1][i];
         }
-        Op::template apply<EDGE>(o, n0, n1, x);
+        if constexpr (SHARE) nn = real ? sh[j] : on;
+        Op::template apply<E>(o, n0, n1, on, nn, x);
         b.r[j] = o;
+        o = next;
+        if constexpr (SHARE) on = sh[j];
     }
-    st.saved = keep;
+    st.saved = o;
+    if constexpr (SHARE) st.c0n = on;
     r0 -= 1;
 }
 
 // An update reading the upper row.  Input and output rows [r0, r0 + RB).
-template <bool EDGE, class T, int Q, int RB, class Op>
-__device__ __forceinline__ void run_stage(StageState<T, Q, K_UP>& st, Block<T, Q, RB>& b, int& r0,
-                                          const LevelCtx& x) {
-    if (EDGE) {
-        if (Op::kHsub && x.need_hsub) {
+template <int E, class T, int Q, int RB, class Op, bool SHARE>
+__device__ __forceinline__ void run_stage(StageState<T, Q, K_UP, SHARE>& st, Block<T, Q, RB>& b,
+                                          int& r0, const LevelCtx& x) {
+    if (E != kInner) {
+        if (E == kEdgeAll && Op::kHsub && x.need_hsub) {
 #pragma unroll
             for (int j = 0; j < RB; ++j) {
                 subst_odd(b.r[j].c[1], x.odd);
@@ -739,12 +789,16 @@ __device__ __forceinline__ void run_stage(StageState<T, Q, K_UP>& st, Block<T, Q
             }
         }
     }
-    T n2[Q], n3[Q];
+    T n2[Q], n3[Q], sh[RB];
     copy_arr(n2, b.r[RB - 1].c[2]);
     copy_arr(n3, b.r[RB - 1].c[3]);
+    if constexpr (SHARE) {
 #pragma unroll
-    for (int j = RB - 1; j >= 0; --j) {  // downwards: the upper row is still pre-step
-        T up2[Q], up3[Q];
+        for (int j = 0; j < RB; ++j) sh[j] = shfl_up(b.r[j].c[3][Q - 1]);
+    }
+#pragma unroll
+    for (int j = RB - 1; j >= 0; --j) {  // upwards: the upper row is still pre-step
+        T up2[Q], up3[Q], un{}, cn{};
         if (j > 0) {
             copy_arr(up2, b.r[j - 1].c[2]);
             copy_arr(up3, b.r[j - 1].c[3]);
@@ -752,49 +806,58 @@ __device__ __forceinline__ void run_stage(StageState<T, Q, K_UP>& st, Block<T, Q
             copy_arr(up2, st.p2);
             copy_arr(up3, st.p3);
         }
-        if (EDGE && r0 + j == 0) {  // image top: the upper row is the row itself
+        if constexpr (SHARE) {
+            cn = sh[j];
+            un = j > 0 ? sh[j > 0 ? j - 1 : 0] : st.c3p;
+        }
+        if (E != kInner && r0 + j == 0) {  // image top: the upper row is the row itself
             copy_arr(up2, b.r[j].c[2]);
             copy_arr(up3, b.r[j].c[3]);
+            un = cn;
         }
-        Op::template apply<EDGE>(b.r[j], up2, up3, x);
+        Op::template apply<E>(b.r[j], up2, up3, cn, un, x);
     }
     copy_arr(st.p2, n2);
     copy_arr(st.p3, n3);
+    if constexpr (SHARE) st.c3p = sh[RB - 1];
 }
 
 template <class T, int Q, class... Ops>
 struct Chain {
     static constexpr int LAG = 0;
     __device__ __forceinline__ void init() {}
-    template <bool EDGE, int RB>
+    template <int E, int RB>
     __device__ __forceinline__ void push(Block<T, Q, RB>&, int&, const LevelCtx&) {}
 };
 template <class T, int Q, class Op, class... Rest>
 struct Chain<T, Q, Op, Rest...> {
-    StageState<T, Q, Op::kind> st;
+    static constexpr bool SHARE = op_share<Op>();
+    StageState<T, Q, Op::kind, SHARE> st;
     Chain<T, Q, Rest...> rest;
     static constexpr int LAG = (Op::kind == K_DOWN ? 1 : 0) + Chain<T, Q, Rest...>::LAG;
     __device__ __forceinline__ void init() {
         zero(st);
         rest.init();
     }
-    template <bool EDGE, int RB>
+    template <int E, int RB>
     __device__ __forceinline__ void push(Block<T, Q, RB>& b, int& r0, const LevelCtx& x) {
-        run_stage<EDGE, T, Q, RB, Op>(st, b, r0, x);
-        rest.template push<EDGE, RB>(b, r0, x);
+        run_stage<E, T, Q, RB, Op>(st, b, r0, x);
+        rest.template push<E, RB>(b, r0, x);
     }
 
    private:
-    __device__ __forceinline__ static void zero(StageState<T, Q, K_NONE>&) {}
-    __device__ __forceinline__ static void zero(StageState<T, Q, K_DOWN>& s) {
+    __device__ __forceinline__ static void zero(StageState<T, Q, K_NONE, false>&) {}
+    __device__ __forceinline__ static void zero(StageState<T, Q, K_DOWN, SHARE>& s) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
             for (int j = 0; j < Q; ++j) s.saved.c[k][j] = T(0);
+        s.c0n = T(0);
     }
-    __device__ __forceinline__ static void zero(StageState<T, Q, K_UP>& s) {
+    __device__ __forceinline__ static void zero(StageState<T, Q, K_UP, SHARE>& s) {
 #pragma unroll
         for (int j = 0; j < Q; ++j) s.p2[j] = s.p3[j] = T(0);
+        s.c3p = T(0);
     }
 };
 
@@ -802,56 +865,47 @@ struct Chain<T, Q, Op, Rest...> {
 template <class T, int Q, int SCH, bool FWD>
 struct Pipe;
 
-// CDF 9/7 forward: pairs (alpha, beta), (gamma, delta).  The forward runs the
-// scalar form of the float steps at 2 columns per lane (its register budget of
-// 128 leaves no room for the register pairs) and the packed form at 4
-// (kFwdPack4: 1 adjacent, 2 strided pairs); the inverse runs the packed form
-// on adjacent pairs.  Each was measured faster for its kernel.
-#ifndef DWT_FWD_PACK4
-#define DWT_FWD_PACK4 2
-#endif
-constexpr int kFwdPack4 = DWT_FWD_PACK4;
+// CDF 9/7 forward: pairs (alpha, beta), (gamma, delta).  The reduced form packs
+// the vertical parts of its steps but the last one, whose results are stored
+// or scaled and so leave the pair anyway.  The plain form packs columns
+// (strided pairs) at 4 columns per lane and is scalar at 2.
 template <int Q>
-constexpr int fwd_pk() { return Q >= 4 ? kFwdPack4 : 0; }
+constexpr int fwd_pk() { return Q >= 4 ? 2 : 0; }
 template <int Q>
 struct Pipe<float, Q, SCH_SEP, true> {
-    static constexpr int P = fwd_pk<Q>();
-    using type = Chain<float, Q, OpFTH<0, 1, P>, OpFTV<0, 1, P>, OpFSH<1, 1, P>, OpFSV<1, 1, P>,
-                       OpFTH<2, 1, P>, OpFTV<2, 1, P>, OpFSH<3, 1, P>, OpFSV<3, 1, P>>;
+    using type = Chain<float, Q, OpFTH<0, 1>, OpFTV<0, 1>, OpFSH<1, 1>, OpFSV<1, 1, true>, OpFTH<2, 1>,
+                       OpFTV<2, 1>, OpFSH<3, 1>, OpFSV<3, 1, false>>;
 };
 template <int Q>
 struct Pipe<float, Q, SCH_NONSEP, true> {
     static constexpr int P = fwd_pk<Q>();
-    using type = Chain<float, Q, OpFT<0, 1, false, P>, OpFS<1, 1, false, P>, OpFT<2, 1, false, P>,
-                       OpFS<3, 1, false, P>>;
+    using type = Chain<float, Q, OpFT<0, 1, P>, OpFS<1, 1, P>, OpFT<2, 1, P>,
+                       OpFS<3, 1, P>>;
 };
 template <int Q>
 struct Pipe<float, Q, SCH_RED, true> {
-    static constexpr int P = fwd_pk<Q>();
-    using type = Chain<float, Q, OpFT<0, 1, true, P>, OpFS<1, 1, true, P>, OpFT<2, 1, true, P>,
-                       OpFS<3, 1, true, P>>;
+    using type = Chain<float, Q, OpRT<0, 1, true>, OpRS<1, 1, true>, OpRT<2, 1, true>, OpRS<3, 1, false>>;
 };
-// CDF 9/7 inverse: undo every step in reverse order (packed; strided pairs
-// at 4 columns per lane).
+// CDF 9/7 inverse: undo every step in reverse order.  The bands arrive
+// component by component and the image leaves in pairs, so the first vertical
+// part is scalar and the last one packed.
 template <int Q>
 constexpr int inv_pk() { return Q >= 4 ? 2 : 1; }
 template <int Q>
 struct Pipe<float, Q, SCH_SEP, false> {
-    static constexpr int P = inv_pk<Q>();
-    using type = Chain<float, Q, OpFSV<3, -1, P>, OpFSH<3, -1, P>, OpFTV<2, -1, P>, OpFTH<2, -1, P>,
-                       OpFSV<1, -1, P>, OpFSH<1, -1, P>, OpFTV<0, -1, P>, OpFTH<0, -1, P>>;
+    using type = Chain<float, Q, OpFSV<3, -1, false>, OpFSH<3, -1>, OpFTV<2, -1>, OpFTH<2, -1>,
+                       OpFSV<1, -1, true>, OpFSH<1, -1>, OpFTV<0, -1>, OpFTH<0, -1>>;
 };
 template <int Q>
 struct Pipe<float, Q, SCH_NONSEP, false> {
     static constexpr int P = inv_pk<Q>();
-    using type = Chain<float, Q, OpFS<3, -1, false, P>, OpFT<2, -1, false, P>,
-                       OpFS<1, -1, false, P>, OpFT<0, -1, false, P>>;
+    using type = Chain<float, Q, OpFS<3, -1, P>, OpFT<2, -1, P>,
+                       OpFS<1, -1, P>, OpFT<0, -1, P>>;
 };
 template <int Q>
 struct Pipe<float, Q, SCH_RED, false> {
-    static constexpr int P = inv_pk<Q>();
-    using type = Chain<float, Q, OpFS<3, -1, true, P>, OpFT<2, -1, true, P>,
-                       OpFS<1, -1, true, P>, OpFT<0, -1, true, P>>;
+    using type = Chain<float, Q, OpRS<3, -1, false>, OpRT<2, -1, true>, OpRS<1, -1, true>,
+                       OpRT<0, -1, true>>;
 };
 // LeGall 5/3 (reversible): the reduced scheme keeps the floors on whole 1-D
 // sums and is therefore the same integer dataflow as the non-separable one.
@@ -900,36 +954,36 @@ struct Engine {
     }
     // Push input rows [r0, r0 + RB); on return `b` holds the emitted rows
     // [r0 - LAG, r0 - LAG + RB) (garbage while the pipeline fills).
-    template <bool EDGE, int RB>
+    template <int E, int RB>
     __device__ __forceinline__ void push(Block<T, Q, RB>& b, int r0, const LevelCtx& x) {
         if (!FWD) {
 #pragma unroll
-            for (int j = 0; j < RB; ++j) scale<EDGE>(b.r[j], x);
+            for (int j = 0; j < RB; ++j) scale<E>(b.r[j], x);
         }
-        chain.template push<EDGE, RB>(b, r0, x);
+        chain.template push<E, RB>(b, r0, x);
         if (FWD) {
 #pragma unroll
-            for (int j = 0; j < RB; ++j) scale<EDGE>(b.r[j], x);
+            for (int j = 0; j < RB; ++j) scale<E>(b.r[j], x);
         }
     }
     // One row; returns false while the pipeline is still filling, and sets r to
     // the emitted row.
-    template <bool EDGE>
+    template <int E>
     __device__ __forceinline__ bool push_counted(Quads<T, Q>& a, int& r, const LevelCtx& x) {
         Block<T, Q, 1> b;
         b.r[0] = a;
-        push<EDGE, 1>(b, r, x);
+        push<E, 1>(b, r, x);
         a = b.r[0];
         r -= LAG;
         return ++npush > LAG;
     }
 
    private:
-    template <bool EDGE>
+    template <int E>
     __device__ __forceinline__ static void scale(Quads<int, Q>&, const LevelCtx&) {}
-    template <bool EDGE>
+    template <int E>
     __device__ __forceinline__ static void scale(Quads<float, Q>& a, const LevelCtx& x) {
-        if (EDGE) {
+        if (E != kInner) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
 #pragma unroll

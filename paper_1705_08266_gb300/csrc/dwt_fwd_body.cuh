@@ -21,28 +21,9 @@
 
 namespace dwt {
 
-// Store Q consecutive values at p; `avail` columns remain inside the band.
-// keep: the next launch reads the values back (L2 evict-last).
-template <class S, class T, int Q>
-__device__ __forceinline__ void store_cols(S* p, const T (&v)[Q], int avail, bool vec,
-                                           bool keep = false) {
-    S w[Q];
-#pragma unroll
-    for (int j = 0; j < Q; ++j) w[j] = Storage<S>::st(v[j]);
-    if (!store_ok(p, (avail < Q ? (avail > 0 ? avail : 0) : Q) * (int)sizeof(S))) return;
-    if (vec && avail >= Q) {
-        if (keep) st_vec_keep<S, Q>(p, w);
-        else st_vec<S, Q>(p, w);
-    } else {
-#pragma unroll
-        for (int j = 0; j < Q; ++j)
-            if (j < avail) p[j] = w[j];
-    }
-}
-
-// Border-free store of a lane's Q values at p: every column lies inside its
-// band and p is vector aligned; ok = the lane stores and the row belongs to
-// the work item (one predicate, no branches per column).
+// A whole vector of a lane's Q values at p (vector aligned); ok = the lane
+// stores and the row belongs to the work item.  keep: the next launch reads
+// the values back (L2 evict-last).
 template <class S, class T, int Q>
 __device__ __forceinline__ void st_fast(S* p, const T (&v)[Q], bool ok, bool keep = false) {
     S w[Q];
@@ -54,67 +35,96 @@ __device__ __forceinline__ void st_fast(S* p, const T (&v)[Q], bool ok, bool kee
     }
 }
 
+// The first n of a lane's Q values at p, whose row starts `al` elements past
+// a vector boundary (al < Q, the same for a whole band): aligned vectors, the
+// widest pieces an unaligned band allows, or the columns left at its edge.
+template <class S, class T, int Q>
+__device__ __forceinline__ void st_any(S* p, const T (&v)[Q], int n, int al, bool keep = false) {
+    if (n <= 0) return;
+    S w[Q];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) w[j] = Storage<S>::st(v[j]);
+    if (!store_ok(p, n * (int)sizeof(S))) return;
+    if (n < Q) {
+#pragma unroll
+        for (int j = 0; j < Q; ++j)
+            if (j < n) p[j] = w[j];
+    } else if (al == 0) {
+        if (keep) st_vec_keep<S, Q>(p, w);
+        else st_vec<S, Q>(p, w);
+    } else if constexpr (Q == 4) {
+        if (al == 2) {
+            st_vec<S, 2>(p, *reinterpret_cast<const S(*)[2]>(w));
+            st_vec<S, 2>(p + 2, *reinterpret_cast<const S(*)[2]>(w + 2));
+        } else {
+            p[0] = w[0];
+            st_vec<S, 2>(p + 1, *reinterpret_cast<const S(*)[2]>(w + 1));
+            p[3] = w[3];
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < Q; ++j) p[j] = w[j];
+    }
+}
+
 // Per-level store state of one lane.
 struct StoreGeo {
-    int ne_r, no_r, ne_c, no_c;
-    int g0;            // first quadruple column of this lane
-    int r_lo, r_hi;    // rows of this level that this work item stores
-    bool vec_hl, vec_lh;
+    int ne_r, no_r, ne_c;
+    int g0;          // first quadruple column of this lane
+    int r_lo, r_hi;  // rows of this level that this work item stores
+    int n_e, n_o;    // columns this lane stores of the LL / LH and of the HL / HH bands
+    int al;          // where the HL / HH rows start, in elements past a vector boundary
 };
 
-// Row r's bands at `base` = mallat + r * pitch + g0; dlh = ne_r * pitch.
-template <class S, class T, int Q>
-__device__ __forceinline__ void store_details_at(const Quads<T, Q>& a, int r, const StoreGeo& g,
-                                                 S* base, long long dlh, bool lane_ok) {
-    if (!lane_ok || r < g.r_lo || r >= g.r_hi || r >= g.ne_r) return;
-    store_cols<S, T, Q>(base + g.ne_c, a.c[1], g.no_c - g.g0, g.vec_hl);
-    if (r < g.no_r) {
-        store_cols<S, T, Q>(base + dlh, a.c[2], g.ne_c - g.g0, g.vec_lh);
-        store_cols<S, T, Q>(base + dlh + g.ne_c, a.c[3], g.no_c - g.g0, g.vec_hl);
+// The bands of rows r .. r + R - 1 whose rows the item owns.  WHOLE: every
+// storing lane stores whole aligned vectors and all rows exist; LAST: the LL
+// leaves the chip too.
+template <class S, class T, int Q, int R, bool WHOLE, bool LAST>
+__device__ __forceinline__ void store_rows(const Block<T, Q, R>& b, int r, const StoreGeo& g, S* mallat,
+                                           long long mpitch, S* ll, long long llpitch, bool keep) {
+    S* hl = mallat + (long long)r * mpitch + (g.g0 + g.ne_c);
+    S* lh = hl + ((long long)g.ne_r * mpitch - g.ne_c);
+    S* lrow = ll + (long long)r * llpitch + g.g0;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const bool in = r + k >= g.r_lo && r + k < g.r_hi;
+        if constexpr (WHOLE) {
+            const bool ok = in && g.n_e > 0;
+            st_fast<S, T, Q>(hl, b.r[k].c[1], ok);
+            st_fast<S, T, Q>(lh, b.r[k].c[2], ok);
+            st_fast<S, T, Q>(lh + g.ne_c, b.r[k].c[3], ok);
+            if constexpr (LAST) st_fast<S, T, Q>(lrow, b.r[k].c[0], ok, keep);
+        } else if (in && r + k < g.ne_r) {
+            st_any<S, T, Q>(hl, b.r[k].c[1], g.n_o, g.al);
+            if (r + k < g.no_r) {
+                st_any<S, T, Q>(lh, b.r[k].c[2], g.n_e, 0);
+                st_any<S, T, Q>(lh + g.ne_c, b.r[k].c[3], g.n_o, g.al);
+            }
+            if constexpr (LAST) st_any<S, T, Q>(lrow, b.r[k].c[0], g.n_e, 0, keep);
+        }
+        hl += mpitch;
+        lh += mpitch;
+        if constexpr (LAST) lrow += llpitch;
     }
-}
-
-template <class S, class T, int Q>
-__device__ __forceinline__ void store_details(const Quads<T, Q>& a, int r, const StoreGeo& g,
-                                              S* mallat, long long pitch, bool lane_ok) {
-    if (!lane_ok || r < g.r_lo || r >= g.r_hi || r >= g.ne_r) return;
-    S* row = mallat + (long long)r * pitch;
-    store_cols<S, T, Q>(row + g.ne_c + g.g0, a.c[1], g.no_c - g.g0, g.vec_hl);
-    if (r < g.no_r) {
-        S* row2 = mallat + (long long)(g.ne_r + r) * pitch;
-        store_cols<S, T, Q>(row2 + g.g0, a.c[2], g.ne_c - g.g0, g.vec_lh);
-        store_cols<S, T, Q>(row2 + g.ne_c + g.g0, a.c[3], g.no_c - g.g0, g.vec_hl);
-    }
-}
-
-// Row r's LL at `at` = ll + r * pitch + g0.
-template <class S, class T, int Q>
-__device__ __forceinline__ void store_ll_at(const Quads<T, Q>& a, int r, const StoreGeo& g, S* at,
-                                            bool lane_ok, bool vec, bool keep) {
-    if (!lane_ok || r < g.r_lo || r >= g.r_hi || r >= g.ne_r) return;
-    store_cols<S, T, Q>(at, a.c[0], g.ne_c - g.g0, vec, keep);
-}
-
-template <class S, class T, int Q>
-__device__ __forceinline__ void store_ll(const Quads<T, Q>& a, int r, const StoreGeo& g, S* ll,
-                                         long long pitch, bool lane_ok, bool vec, bool keep) {
-    if (!lane_ok || r < g.r_lo || r >= g.r_hi || r >= g.ne_r) return;
-    store_cols<S, T, Q>(ll + (long long)r * pitch + g.g0, a.c[0], g.ne_c - g.g0, vec, keep);
 }
 
 __device__ __forceinline__ StoreGeo make_geo(int h, int w, int g0, int Q, int r_lo, int r_hi,
-                                             long long pitch) {
+                                             bool lane_ok) {
     StoreGeo g;
     g.ne_r = (h + 1) >> 1;
     g.no_r = h >> 1;
     g.ne_c = (w + 1) >> 1;
-    g.no_c = w >> 1;
     g.g0 = g0;
     g.r_lo = r_lo;
     g.r_hi = r_hi;
-    g.vec_hl = (g.ne_c % Q == 0) && (pitch % Q == 0);
-    g.vec_lh = (pitch % Q == 0);
+    g.n_e = lane_ok ? min(max(g.ne_c - g0, 0), Q) : 0;
+    g.n_o = lane_ok ? min(max((w >> 1) - g0, 0), Q) : 0;
+    g.al = g.ne_c & (Q - 1);
     return g;
+}
+// Every lane of the warp stores whole aligned vectors of this level or nothing.
+__device__ __forceinline__ bool geo_whole(const StoreGeo& g, int Q) {
+    return g.al == 0 && __all_sync(kFull, (g.n_e == 0 || g.n_e == Q) && g.n_o == g.n_e);
 }
 
 // Pair two consecutive LL rows (even row e, odd row o) of Q values into a
@@ -157,9 +167,60 @@ struct FwdWarp {
     S* mallat;
     S* ll;
     long long mpitch, llpitch;
-    bool lane_ok, vec_ll;
+    bool whole;    // every lane stores whole aligned vectors (all fused levels)
     bool ll_keep;  // the next launch reads the LL back: store it L2 evict-last
     int lane;
+    // border strips: columns outside the image that this lane fills with the
+    // mirrored ones (element offsets within a row of the box, destination in
+    // the low half; -1: none)
+    int fix_l, fix_r;
+    bool fix;        // warp-uniform: this strip has such columns
+    int ref1, ref2;  // columns of the next level's input past which a row is mirrored again (0: no)
+
+    // Columns outside the image take the mirrored ones (whole-sample symmetric
+    // extension), in shared memory, before any lane reads them.
+    __device__ __forceinline__ void extend_columns(S* sm) {
+        // (every load before the first store, or the loads would wait for the
+        // stores they might alias)
+        S l[2 * SR], r[2 * SR];
+        const int ls = (fix_l >> 16) & (BW - 1), rs = (fix_r >> 16) & (BW - 1);
+#pragma unroll
+        for (int k = 0; k < 2 * SR; ++k) {
+            l[k] = sm[k * BW + ls];
+            r[k] = sm[k * BW + rs];
+        }
+#pragma unroll
+        for (int k = 0; k < 2 * SR; ++k) {
+            if (fix_l >= 0) sm[k * BW + (fix_l & 0xffff)] = l[k];
+            if (fix_r >= 0) sm[k * BW + (fix_r & 0xffff)] = r[k];
+        }
+        __syncwarp();
+    }
+
+    // The R LL rows of a level become the next level's input, which is mirrored
+    // about its own last column n - 1.  The computed columns past it already
+    // equal that for an odd width; an even one repeats its last column instead
+    // (the border lies between two samples), so those columns are rewritten.
+    // At the left border both agree unless the signal is shorter than the halo.
+    template <int Q, int R>
+    __device__ __forceinline__ void extend_ll(S* sm, Block<T, Q, R>& b, int g0, int n) {
+        T* scratch = reinterpret_cast<T*>(sm);  // the slot's rows have been read
+        const int gw = g0 - Q * lane;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < R; ++k) st_vec<T, Q>(scratch + k * 32 * Q + Q * lane, b.r[k].c[0]);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            const int g = g0 + j;
+            if (g < 0 || g >= n) {
+                const int src = min(max(reflect(min(g, n + 15), n) - gw, 0), 32 * Q - 1);
+#pragma unroll
+                for (int k = 0; k < R; ++k) b.r[k].c[0][j] = scratch[k * 32 * Q + src];
+            }
+        }
+        __syncwarp();
+    }
 
     // One slot: level-1 input quadruple rows q0 .. q0+SR-1 (q0 a multiple of
     // SR) in shared memory (2 SR image rows of BW pixels), pushed as one
@@ -181,45 +242,18 @@ struct FwdWarp {
         }
     }
 
-    // Store the R2 level-2 rows a level-2 push of input rows from in2 emitted.
-    template <bool EDGE, int R2>
-    __device__ __forceinline__ void store_level2(const Block<T, Q2, R2>& b2, int in2) {
-        const int r2 = in2 - LAG;
-        if constexpr (!EDGE) {
-            S* hl = mallat + (long long)r2 * mpitch + (s2.g0 + s2.ne_c);
-            S* lh = hl + ((long long)s2.ne_r * mpitch - s2.ne_c);
-            S* lrow = ll + (long long)r2 * llpitch + s2.g0;
-#pragma unroll
-            for (int k = 0; k < R2; ++k) {
-                const bool ok = lane_ok && r2 + k >= s2.r_lo && r2 + k < s2.r_hi;
-                st_fast<S, T, Q2>(hl, b2.r[k].c[1], ok);
-                st_fast<S, T, Q2>(lh, b2.r[k].c[2], ok);
-                st_fast<S, T, Q2>(lh + s2.ne_c, b2.r[k].c[3], ok);
-                hl += mpitch;
-                lh += mpitch;
-                if constexpr (NL == 2) {
-                    st_fast<S, T, Q2>(lrow, b2.r[k].c[0], ok, ll_keep);
-                    lrow += llpitch;
-                }
-            }
-        } else {
-            S* base = mallat + (long long)r2 * mpitch + s2.g0;
-            const long long dlh = (long long)s2.ne_r * mpitch;
-            S* lrow = ll + (long long)r2 * llpitch + s2.g0;
-#pragma unroll
-            for (int k = 0; k < R2; ++k) {
-                store_details_at<S, T, Q2>(b2.r[k], r2 + k, s2, base, dlh, lane_ok);
-                base += mpitch;
-                if constexpr (NL == 2) {
-                    store_ll_at<S, T, Q2>(b2.r[k], r2 + k, s2, lrow, lane_ok, vec_ll, ll_keep);
-                    lrow += llpitch;
-                }
-            }
-        }
+    // The rows of level L that a push emitted, from row r on.
+    template <int E, int L, int Q, int R>
+    __device__ __forceinline__ void store_level(const Block<T, Q, R>& b, int r, const StoreGeo& g) {
+        if (E == kInner && __builtin_expect(whole, 1))
+            store_rows<S, T, Q, R, true, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
+        else
+            store_rows<S, T, Q, R, false, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
     }
 
-    template <bool EDGE>
-    __device__ __forceinline__ void slot(const S* sm, int q0) {
+    template <int E>
+    __device__ __forceinline__ void slot(S* sm, int q0) {
+        if (__builtin_expect(fix, 0)) extend_columns(sm);
         Block<T, Q1, SR> b1;
 #pragma unroll
         for (int k = 0; k < SR; ++k) {
@@ -235,53 +269,20 @@ struct FwdWarp {
                 row.c[3][j] = Storage<S>::ld(od[2 * j + 1]);
             }
         }
-        e1.template push<EDGE, SR>(b1, q0, x1);
-        const int r1 = q0 - LAG;  // first emitted level-1 row
-        if constexpr (!EDGE) {
-            // border-free slot: band addresses advanced by the pitch, one
-            // predicate per row
-            S* hl = mallat + (long long)r1 * mpitch + (s1.g0 + s1.ne_c);
-            S* lh = hl + ((long long)s1.ne_r * mpitch - s1.ne_c);
-            S* lrow = ll + (long long)r1 * llpitch + s1.g0;
-#pragma unroll
-            for (int k = 0; k < SR; ++k) {
-                const bool ok = lane_ok && r1 + k >= s1.r_lo && r1 + k < s1.r_hi;
-                st_fast<S, T, Q1>(hl, b1.r[k].c[1], ok);
-                st_fast<S, T, Q1>(lh, b1.r[k].c[2], ok);
-                st_fast<S, T, Q1>(lh + s1.ne_c, b1.r[k].c[3], ok);
-                hl += mpitch;
-                lh += mpitch;
-                if constexpr (NL == 1) {
-                    st_fast<S, T, Q1>(lrow, b1.r[k].c[0], ok, ll_keep);
-                    lrow += llpitch;
-                }
-            }
-        } else {
-            // one row address per slot, advanced by the pitch (bands of row r
-            // at base, base + ne_c, base + ne_r pitch (+ ne_c))
-            S* base = mallat + (long long)r1 * mpitch + s1.g0;
-            const long long dlh = (long long)s1.ne_r * mpitch;
-            S* lrow = ll + (long long)r1 * llpitch + s1.g0;
-#pragma unroll
-            for (int k = 0; k < SR; ++k) {
-                store_details_at<S, T, Q1>(b1.r[k], r1 + k, s1, base, dlh, lane_ok);
-                base += mpitch;
-                if constexpr (NL == 1) {
-                    store_ll_at<S, T, Q1>(b1.r[k], r1 + k, s1, lrow, lane_ok, vec_ll, ll_keep);
-                    lrow += llpitch;
-                }
-            }
-        }
+        e1.template push<E, SR>(b1, q0, x1);
+        store_level<E, 1>(b1, q0 - LAG, s1);
         if constexpr (NL >= 2) {
+            if (__builtin_expect(ref1 != 0, 0)) extend_ll(sm, b1, s1.g0, ref1);
             // level-2 input rows q0/2 - 1 .. q0/2 + R2 - 2 = LL rows q0 - 2 .. q0 + SR - 3
             constexpr int R2 = SR / 2;
             Block<T, Q2, R2> b2;
             pair_level1<R2>(b1, b2);
             const int in2 = q0 / 2 - 1;
-            e2.template push<EDGE, R2>(b2, in2, x2);
-            store_level2<EDGE, R2>(b2, in2);
+            e2.template push<E, R2>(b2, in2, x2);
+            store_level<E, 2>(b2, in2 - LAG, s2);
             if constexpr (NL >= 3) {
                 static_assert(Q1 >= 4, "three fused levels need 4 columns per lane");
+                if (__builtin_expect(ref2 != 0, 0)) extend_ll(sm, b2, s2.g0, ref2);
                 Block<T, Q3, 1> b3;
                 int in3;
                 if constexpr (LAG == 2) {  // level-2 rows q0/2-3, q0/2-2; q0/2-4 kept
@@ -292,9 +293,8 @@ struct FwdWarp {
                     pair_rows<T, Q2>(b2.r[0].c[0], b2.r[1].c[0], b3.r[0]);
                     in3 = q0 / 4 - 1;
                 }
-                e3.template push<EDGE, 1>(b3, in3, x3);
-                store_details<S, T, Q3>(b3.r[0], in3 - LAG, s3, mallat, mpitch, lane_ok);
-                store_ll<S, T, Q3>(b3.r[0], in3 - LAG, s3, ll, llpitch, lane_ok, vec_ll, ll_keep);
+                e3.template push<E, 1>(b3, in3, x3);
+                store_level<E, 3>(b3, in3 - LAG, s3);
             }
         }
     }
@@ -313,14 +313,12 @@ __device__ __forceinline__ bool rows_interior(int q0, int sr, int nl, int lag, c
     return true;
 }
 
-// CTAs per SM the register budget is sized for: 16 warps (128 registers) with
-// 2 quadruple columns per lane; with 4, 12 warps (168 registers) for slots of
-// 2 quadruple rows, 8 for three fused levels.
-// (measured: 13-16 warps with 4 columns, at 128 registers and 32-60 bytes
-// of spills, were 2-20 % slower than 12 at 168 registers)
-template <int NL, int Q1>
+// CTAs per SM the register budget is sized for: 16 warps (128 registers), or
+// 12 (168) for the plain non-separable steps at 4 quadruple columns per lane,
+// 8 for three fused levels.
+template <int SCH, int NL, int Q1>
 __host__ __device__ constexpr int fwd_min_blocks() {
-    return (Q1 <= 2 ? 16 : (fwd_slot_quads<NL, Q1>() == 2 ? 12 : 8)) / kFwdWarps;
+    return (NL >= 3 ? 8 : (Q1 >= 4 && SCH == SCH_NONSEP ? 12 : 16)) / kFwdWarps;
 }
 
 // One warp's work item `wid` of a launch described by `a` (input through the
@@ -369,41 +367,54 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
 
     FW W;
     W.lane = lane;
-    W.lane_ok = lane >= a.lane_lo && lane < a.lane_hi;
+    const bool lane_ok = lane >= a.lane_lo && lane < a.lane_hi;
     W.mallat = reinterpret_cast<S*>(a.mallat);
     W.mpitch = a.mallat_pitch;
     W.ll = reinterpret_cast<S*>(a.ll);
     W.llpitch = a.ll_pitch;
-    constexpr int QN = NL == 1 ? Q1 : (NL == 2 ? FW::Q2 : FW::Q3);
-    W.vec_ll = (a.ll_pitch % QN) == 0;
     W.ll_keep = a.ll_keep != 0;
     int no_r[3] = {0, 0, 0};
-    bool hfast = true;
+    bool active;  // both axes of every fused level
     {
         const int g1 = (xb >> 1) + Q1 * lane;
-        W.x1 = make_ctx(g1, Q1, a.lv[0].h, a.lv[0].w, a.lane_lo, a.lane_hi, a.lv[0].s);
-        W.s1 = make_geo(a.lv[0].h, a.lv[0].w, g1, Q1, R0 << (NL - 1), R1 << (NL - 1), a.mallat_pitch);
+        W.x1 = make_ctx(g1, Q1, a.lv[0].h, a.lv[0].w, a.lv[0].s);
+        W.s1 = make_geo(a.lv[0].h, a.lv[0].w, g1, Q1, R0 << (NL - 1), R1 << (NL - 1), lane_ok);
         no_r[0] = a.lv[0].h >> 1;
-        hfast = hfast && (xb >> 1) >= 2 && (xb >> 1) + 32 * Q1 + 2 <= (a.lv[0].w >> 1);
+        active = a.lv[0].w > 1 && a.lv[0].h > 1;
+        W.whole = geo_whole(W.s1, Q1);
     }
     if constexpr (NL >= 2) {
         const int g2 = (xb >> 2) + FW::Q2 * lane;
-        W.x2 = make_ctx(g2, FW::Q2, a.lv[1].h, a.lv[1].w, a.lane_lo, a.lane_hi, a.lv[1].s);
-        W.s2 = make_geo(a.lv[1].h, a.lv[1].w, g2, FW::Q2, R0 << (NL - 2), R1 << (NL - 2), a.mallat_pitch);
+        W.x2 = make_ctx(g2, FW::Q2, a.lv[1].h, a.lv[1].w, a.lv[1].s);
+        W.s2 = make_geo(a.lv[1].h, a.lv[1].w, g2, FW::Q2, R0 << (NL - 2), R1 << (NL - 2), lane_ok);
         no_r[1] = a.lv[1].h >> 1;
-        hfast = hfast && (xb >> 2) >= 2 && (xb >> 2) + 32 * FW::Q2 + 2 <= (a.lv[1].w >> 1);
+        active = active && a.lv[1].w > 1 && a.lv[1].h > 1;
+        W.whole = geo_whole(W.s2, FW::Q2) && W.whole;
     }
     if constexpr (NL >= 3) {
         const int g3 = (xb >> 3) + FW::Q3 * lane;
-        W.x3 = make_ctx(g3, FW::Q3, a.lv[2].h, a.lv[2].w, a.lane_lo, a.lane_hi, a.lv[2].s);
-        W.s3 = make_geo(a.lv[2].h, a.lv[2].w, g3, FW::Q3, R0, R1, a.mallat_pitch);
+        W.x3 = make_ctx(g3, FW::Q3, a.lv[2].h, a.lv[2].w, a.lv[2].s);
+        W.s3 = make_geo(a.lv[2].h, a.lv[2].w, g3, FW::Q3, R0, R1, lane_ok);
         no_r[2] = a.lv[2].h >> 1;
-        hfast = hfast && (xb >> 3) >= 2 && (xb >> 3) + 32 * FW::Q3 + 2 <= (a.lv[2].w >> 1);
+        active = active && a.lv[2].w > 1 && a.lv[2].h > 1;
+        W.whole = geo_whole(W.s3, FW::Q3) && W.whole;
     }
-    // the border-free code stores whole vectors only
-    hfast = hfast && W.s1.vec_hl && W.s1.vec_lh && W.vec_ll;
-    if constexpr (NL >= 2) hfast = hfast && W.s2.vec_hl && W.s2.vec_lh;
-    if constexpr (NL >= 3) hfast = hfast && W.s3.vec_hl && W.s3.vec_lh;
+    // columns outside the image: up to 32 on each side, one per lane (the
+    // halo of three fused levels takes 28)
+    const int w0 = a.lv[0].w;
+    W.fix_l = W.fix_r = -1;
+    if (xb + lane < 0) W.fix_l = lane | (min(max(reflect(xb + lane, w0) - xb, 0), BW - 1) << 16);
+    if (w0 + lane < xb + BW)
+        W.fix_r = (w0 + lane - xb) | (min(max(reflect(w0 + lane, w0) - xb, 0), BW - 1) << 16);
+    W.fix = xb < 0 || xb + BW > w0;
+    // a level of even width whose right border this box holds (a signal
+    // shorter than its halo lies in one box, left border included)
+    W.ref1 = NL >= 2 && !(w0 & 1) && xb + BW > w0 ? (w0 + 1) >> 1 : 0;
+    W.ref2 = 0;
+    if constexpr (NL >= 3) {
+        const int w1 = a.lv[1].w;
+        if (!(w1 & 1) && xb + BW > w0) W.ref2 = (w1 + 1) >> 1;
+    }
     W.e1.init();
     if constexpr (NL >= 2) W.e2.init();
     if constexpr (NL >= 3) W.e3.init();
@@ -433,7 +444,7 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
     // slot on (rows far enough from the top) and up to some slot (clear of the
     // bottom), so two scans find it instead of one test per slot
     int si0 = nslots, si1 = nslots;
-    if (hfast) {
+    if (active) {
         si0 = 0;
         while (si0 < nslots && !rows_interior(qstart + SR * si0, SR, NL, RHO, no_r)) ++si0;
         si1 = nslots;
@@ -451,12 +462,12 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
         }
         const int q0 = qstart + SR * s;
         if (s >= si0 && s < si1)
-            W.template slot<false>(ring + b * kSlotElems, q0);
+            W.template slot<kInner>(ring + b * kSlotElems, q0);
         else
-            W.template slot<true>(ring + b * kSlotElems, q0);
+            W.template slot<kEdgeRows>(ring + b * kSlotElems, q0);
+        fence_proxy_async_smem();  // every lane: its reads and writes before the refill
         __syncwarp();
         if (lane == 0 && s + kFwdSlots < nslots) {
-            fence_proxy_async_smem();
             mbar_arrive_expect_tx(bar_s + 8 * b, kSlotBytes);
             tma_load_2d(ring_s + b * kSlotBytes, mapp, xb, y0 + (s + kFwdSlots) * SLOT_ROWS,
                         bar_s + 8 * b);

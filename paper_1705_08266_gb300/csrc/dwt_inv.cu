@@ -112,7 +112,7 @@ struct InvWarp {
         constexpr int Q = 4 >> (L - 1);
         load_details<T, Q>(a, i, g[L - 1], mallat, pitch);
         int r = i;
-        if (!eng<L>().template push_counted<true>(a, r, x[L - 1])) return;
+        if (!eng<L>().template push_counted<kEdgeAll>(a, r, x[L - 1])) return;
         // emitted quadruple row r -> rows 2r (c0 c1 interleaved) and 2r+1 (c2 c3)
         if constexpr (L == 1) {
             if (!lane_ok || r < A0 || r >= A1) return;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(128) inv_fused_kernel(const FusedArgs a) {
     for (int l = 0; l < NL; ++l) {
         const int Q = 4 >> l;
         const int g0 = (W.xb >> (l + 1)) + Q * lane;
-        W.x[l] = make_ctx(g0, Q, a.lv[l].h, a.lv[l].w, a.lane_lo, a.lane_hi, a.lv[l].s);
+        W.x[l] = make_ctx(g0, Q, a.lv[l].h, a.lv[l].w, a.lv[l].s);
         W.g[l] = make_igeo(a.lv[l].h, a.lv[l].w, g0, Q, a.mallat_pitch, a.ll_pitch);
     }
     W.e1.init();

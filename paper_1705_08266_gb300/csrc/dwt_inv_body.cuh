@@ -48,10 +48,22 @@ struct InvLayout {
 };
 
 // Lane's Q values of one band row held in shared memory at p (+ lane * Q).
-template <class S, class T, int Q>
+// A box starts at a multiple of 16 bytes, so its offset in the box is any;
+// EVEN: it is even, and the values are read in pairs.
+template <class S, class T, int Q, bool EVEN = false>
 __device__ __forceinline__ void lds_cols(T (&v)[Q], const S* p) {
+    if constexpr (EVEN && Q % 2 == 0) {
 #pragma unroll
-    for (int j = 0; j < Q; ++j) v[j] = Storage<S>::ld(p[j]);
+        for (int j = 0; j < Q; j += 2) {
+            S w[2];
+            ld_vec<S, 2>(w, p + j);
+            v[j] = Storage<S>::ld(w[0]);
+            v[j + 1] = Storage<S>::ld(w[1]);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < Q; ++j) v[j] = Storage<S>::ld(p[j]);
+    }
 }
 
 template <class S, int SCH, int NL, int Q1>
@@ -67,21 +79,98 @@ struct InvWarpT {
     int o1h, o1l, o2h, o2l;
     S* out;
     long long opitch;
-    int out_h, out_w, xb, lane, A0, A1;
+    int out_h, lane, A0, A1;
     int x0l;        // first output column of this lane
-    bool lane_ok, vec_out;
-    bool vec_row;   // this lane's 2 Q1 output columns are one aligned vector inside the row
+    int n_out;      // output columns this lane stores
+    bool whole;     // warp-uniform: every lane stores whole vectors or nothing
+    bool even;      // warp-uniform: the level-1 box offsets are even
+    // border strips: per level and band parity (even columns: LL, LH; odd: HL,
+    // HH) the column outside the band that this lane fills with the mirrored
+    // one (offsets from the lane-0 column, destination in the low half; -1: none)
+    int fix1e, fix1o, fix2e, fix2o;
+    bool fix;        // warp-uniform: this strip has such columns
+    int ref1;        // width of level 1 if its LL rows are mirrored again past it (0: no)
 
     static constexpr int SR = Lay::SR;
     static constexpr int SR2 = Lay::SR2;
 
-    template <bool EDGE>
-    __device__ __forceinline__ void slot(const S* sm, int q0, bool level1) {
+    // ROWS rows of NB bands, band i at p + i REGION with its lane-0 column at
+    // off[i] and this lane's column f[i].  Every load comes before the first store, or the loads
+    // would wait for the stores they might alias.
+    template <int NB, int ROWS, int PITCH, int REGION>
+    __device__ __forceinline__ static void fix_bands(S* p, const int (&off)[NB], const int (&f)[NB]) {
+        S v[NB][ROWS];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+                v[i][r] = p[i * REGION + off[i] + r * PITCH + max(f[i] >> 16, 0)];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+                if (f[i] >= 0) p[i * REGION + off[i] + r * PITCH + (f[i] & 0xffff)] = v[i][r];
+    }
+
+    // Columns outside the bands take the mirrored ones, in shared memory,
+    // before any lane reads them (a band's box holds its neighbour bands there).
+    __device__ __forceinline__ void extend_columns(S* sm, bool level1) {
+        if constexpr (NL == 1) {
+            fix_bands<4, SR, Lay::W1, Lay::R1>(sm, {o1l, o1h, o1l, o1h}, {fix1e, fix1o, fix1e, fix1o});
+        } else {
+            if (level1) fix_bands<3, SR, Lay::W1, Lay::R1>(sm, {o1h, o1l, o1h}, {fix1o, fix1e, fix1o});
+            fix_bands<4, SR2, Lay::W2, Lay::R2>(sm + 3 * Lay::R1, {o2l, o2h, o2l, o2h},
+                                                {fix2e, fix2o, fix2e, fix2o});
+        }
+        __syncwarp();
+    }
+
+    // The level-2 output becomes level 1's LL.  Past the last column it is
+    // mirrored about that column; an even width wants it repeated instead (the
+    // border of level 1 lies between two samples), so those columns are
+    // rewritten.  Scratch: the level-2 boxes, which have been read.
+    __device__ __forceinline__ void extend_ll(S* sm2, Block<T, Q1, SR>& b) {
+        static_assert(NL == 1 || 4 * Lay::R2 * sizeof(S) >= SR * 32 * Q1 * sizeof(T), "scratch");
+        T* scratch = reinterpret_cast<T*>(sm2);
+        const int g0 = x0l >> 1, gw = g0 - Q1 * lane, n = (ref1 + 1) >> 1;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < SR; ++k) st_vec<T, Q1>(scratch + k * 32 * Q1 + Q1 * lane, b.r[k].c[0]);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < Q1; ++j) {
+            const int g = g0 + j;
+            if (g < 0 || g >= n) {
+                const int src = min(max((reflect(2 * min(g, n + 15), ref1) >> 1) - gw, 0), 32 * Q1 - 1);
+#pragma unroll
+                for (int k = 0; k < SR; ++k) b.r[k].c[0][j] = scratch[k * 32 * Q1 + src];
+            }
+        }
+        __syncwarp();
+    }
+
+    // The level-1 bands of the slot (the detail bands, and the LL of one level).
+    template <bool EVEN>
+    __device__ __forceinline__ void load_level1(Block<T, Q1, SR>& b, const S* sm) {
+        constexpr int D = NL == 1 ? 1 : 0;  // first detail band
+#pragma unroll
+        for (int k = 0; k < SR; ++k) {
+            const S* row = sm + k * Lay::W1 + Q1 * lane;
+            if constexpr (NL == 1) lds_cols<S, T, Q1, EVEN>(b.r[k].c[0], row + o1l);
+            lds_cols<S, T, Q1, EVEN>(b.r[k].c[1], row + (D + 0) * Lay::R1 + o1h);
+            lds_cols<S, T, Q1, EVEN>(b.r[k].c[2], row + (D + 1) * Lay::R1 + o1l);
+            lds_cols<S, T, Q1, EVEN>(b.r[k].c[3], row + (D + 2) * Lay::R1 + o1h);
+        }
+    }
+
+    template <int E>
+    __device__ __forceinline__ void slot(S* sm, int q0, bool level1) {
+        if (__builtin_expect(fix, 0)) extend_columns(sm, level1);
         Block<T, Q1, SR> b1;
         if constexpr (NL == 2) {
             constexpr int QQ = Q2;
             Block<T, QQ, SR2> b2;
-            const S* base2 = sm + 3 * Lay::R1;
+            S* base2 = sm + 3 * Lay::R1;
 #pragma unroll
             for (int k = 0; k < SR2; ++k) {
                 lds_cols<S, T, QQ>(b2.r[k].c[0], base2 + 0 * Lay::R2 + k * Lay::W2 + o2l + QQ * lane);
@@ -89,7 +178,7 @@ struct InvWarpT {
                 lds_cols<S, T, QQ>(b2.r[k].c[2], base2 + 2 * Lay::R2 + k * Lay::W2 + o2l + QQ * lane);
                 lds_cols<S, T, QQ>(b2.r[k].c[3], base2 + 3 * Lay::R2 + k * Lay::W2 + o2h + QQ * lane);
             }
-            e2.template push<EDGE, SR2>(b2, q0 / 2 + LAG, x2);
+            e2.template push<E, SR2>(b2, q0 / 2 + LAG, x2);
             if (!level1) return;
             // level-2 rows q0/2 .. q0/2 + SR2 - 1 -> LL rows q0 .. q0 + SR - 1 of level 1
 #pragma unroll
@@ -102,22 +191,11 @@ struct InvWarpT {
                     b1.r[2 * k + 1].c[0][2 * j + 1] = b2.r[k].c[3][j];
                 }
             }
-#pragma unroll
-            for (int k = 0; k < SR; ++k) {
-                lds_cols<S, T, Q1>(b1.r[k].c[1], sm + 0 * Lay::R1 + k * Lay::W1 + o1h + Q1 * lane);
-                lds_cols<S, T, Q1>(b1.r[k].c[2], sm + 1 * Lay::R1 + k * Lay::W1 + o1l + Q1 * lane);
-                lds_cols<S, T, Q1>(b1.r[k].c[3], sm + 2 * Lay::R1 + k * Lay::W1 + o1h + Q1 * lane);
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < SR; ++k) {
-                lds_cols<S, T, Q1>(b1.r[k].c[0], sm + 0 * Lay::R1 + k * Lay::W1 + o1l + Q1 * lane);
-                lds_cols<S, T, Q1>(b1.r[k].c[1], sm + 1 * Lay::R1 + k * Lay::W1 + o1h + Q1 * lane);
-                lds_cols<S, T, Q1>(b1.r[k].c[2], sm + 2 * Lay::R1 + k * Lay::W1 + o1l + Q1 * lane);
-                lds_cols<S, T, Q1>(b1.r[k].c[3], sm + 3 * Lay::R1 + k * Lay::W1 + o1h + Q1 * lane);
-            }
+            if (__builtin_expect(ref1 != 0, 0)) extend_ll(base2, b1);
         }
-        e1.template push<EDGE, SR>(b1, q0, x1);
+        if (__builtin_expect(even, 1)) load_level1<true>(b1, sm);
+        else load_level1<false>(b1, sm);
+        e1.template push<E, SR>(b1, q0, x1);
         const int r1 = q0 - LAG;
         // quadruple row r -> output rows 2r (c0 c1 interleaved) and 2r + 1
         // (c2 c3); one row address per slot, advanced by the pitch
@@ -125,7 +203,7 @@ struct InvWarpT {
 #pragma unroll
         for (int k = 0; k < SR; ++k) {
             const int r = r1 + k;
-            const bool ok = lane_ok && r >= A0 && r < A1;
+            const bool ok = r >= A0 && r < A1;
             T ev[2 * Q1], od[2 * Q1];
 #pragma unroll
             for (int j = 0; j < Q1; ++j) {
@@ -134,39 +212,31 @@ struct InvWarpT {
                 od[2 * j] = b1.r[k].c[2][j];
                 od[2 * j + 1] = b1.r[k].c[3][j];
             }
-            if constexpr (!EDGE) {
-                // border-free slot: whole vectors inside the image, one predicate
-                store_fast_px(ev, p, ok);
-                store_fast_px(od, p + opitch, ok);
-            } else if (ok) {
-                store_px(ev, 2 * r, p);
-                store_px(od, 2 * r + 1, p + opitch);
+            if (__builtin_expect(whole, 1)) {
+                st_px<true>(ev, p, ok);
+                st_px<true>(od, p + opitch, ok && (E == kInner || 2 * r + 1 < out_h));
+            } else {
+                st_px<false>(ev, p, ok);
+                st_px<false>(od, p + opitch, ok && (E == kInner || 2 * r + 1 < out_h));
             }
             p += 2 * opitch;
         }
     }
 
-    __device__ __forceinline__ void store_fast_px(const T (&v)[2 * Q1], S* p, bool ok) {
+    // One output row of this lane at p: a whole aligned vector (output rows
+    // start on 16 bytes, lanes on whole vectors of them), or the columns left
+    // at the right border.
+    template <bool WHOLE>
+    __device__ __forceinline__ void st_px(const T (&v)[2 * Q1], S* p, bool ok) {
         S w[2 * Q1];
 #pragma unroll
         for (int j = 0; j < 2 * Q1; ++j) w[j] = Storage<S>::st(v[j]);
-        if (ok && store_ok(p, 2 * Q1 * (int)sizeof(S))) st_vec<S, 2 * Q1>(p, w);
-    }
-
-    // Output row y at p (= out + y * opitch + x0l).
-    __device__ __forceinline__ void store_px(const T (&v)[2 * Q1], int y, S* p) {
-        if (y >= out_h) return;
-        S w[2 * Q1];
-#pragma unroll
-        for (int j = 0; j < 2 * Q1; ++j) w[j] = Storage<S>::st(v[j]);
-        if (!store_ok(p + max(-x0l, 0), (min(x0l + 2 * Q1, out_w) - max(x0l, 0)) * (int)sizeof(S)))
-            return;
-        if (vec_row) {
-            st_vec<S, 2 * Q1>(p, w);
-        } else {
+        if (WHOLE || n_out == 2 * Q1) {
+            if (ok && n_out > 0 && store_ok(p, 2 * Q1 * (int)sizeof(S))) st_vec<S, 2 * Q1>(p, w);
+        } else if (ok && store_ok(p, n_out * (int)sizeof(S))) {
 #pragma unroll
             for (int j = 0; j < 2 * Q1; ++j)
-                if (x0l + j >= 0 && x0l + j < out_w) p[j] = w[j];
+                if (j < n_out) p[j] = w[j];
         }
     }
 };
@@ -205,43 +275,64 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
     const int strip = wid % a.nstrips;
     W w;
     w.lane = lane;
-    w.xb = strip * a.valid_px - a.xoff;
-    w.lane_ok = lane >= a.lane_lo && lane < a.lane_hi;
+    const int xb = strip * a.valid_px - a.xoff;
+    const bool lane_ok = lane >= a.lane_lo && lane < a.lane_hi;
     w.out = reinterpret_cast<S*>(a.out);
     w.opitch = a.out_pitch;
     w.out_h = a.lv[0].h;
-    w.out_w = a.lv[0].w;
-    w.vec_out = (a.out_pitch % (2 * Q1)) == 0;
-    w.x0l = w.xb + 2 * Q1 * lane;
+    w.x0l = xb + 2 * Q1 * lane;
+    w.n_out = lane_ok ? min(max(a.lv[0].w - w.x0l, 0), 2 * Q1) : 0;
+    w.whole = __all_sync(kFull, w.n_out == 0 || w.n_out == 2 * Q1);
     set_store_windows(a.out, a.out_elems * (long long)sizeof(S), nullptr, 0, a.err);
-    w.vec_row = w.vec_out && w.x0l >= 0 && w.x0l + 2 * Q1 <= a.lv[0].w;
     const int ne1 = (a.lv[0].h + 1) >> 1;
     seg_rows(a, wid / a.nstrips, ne1, w.A0, w.A1);
 
     int no_r[2] = {a.lv[0].h >> 1, NL >= 2 ? (a.lv[1].h >> 1) : 0};
-    const int g1w = w.xb >> 1;
+    const int g1w = xb >> 1;
     const int ne_c1 = (a.lv[0].w + 1) >> 1, ne_r1 = ne1;
-    w.x1 = make_ctx(g1w + Q1 * lane, Q1, a.lv[0].h, a.lv[0].w, a.lane_lo, a.lane_hi, a.lv[0].s);
+    w.x1 = make_ctx(g1w + Q1 * lane, Q1, a.lv[0].h, a.lv[0].w, a.lv[0].s);
     const int xh1 = ne_c1 + g1w, xl1 = g1w;
     constexpr int AM = Lay::A - 1;
     const int bx1h = xh1 & ~AM, bx1l = xl1 & ~AM;
     w.o1h = xh1 - bx1h;
     w.o1l = xl1 - bx1l;
-    bool hfast = g1w >= 2 && g1w + 32 * Q1 + 2 <= (a.lv[0].w >> 1);
+    w.even = !((w.o1h | w.o1l) & 1);
+    bool active = a.lv[0].w > 1 && a.lv[0].h > 1;  // both axes of every fused level
+    // the column of a band (parity par of a level of width n) outside it that
+    // this lane fills: lanes 0-15 left of it, 16-31 right of it (the halo of
+    // two fused levels takes 8)
+    auto fix_of = [&](int gw, int n, int par, int Q) {
+        const int nb = (n + 1 - par) >> 1;
+        const int g = lane < 16 ? gw + lane : nb + lane - 16;
+        if (nb <= 0 || (lane < 16 ? g >= 0 : g < gw || g >= gw + 32 * Q)) return -1;
+        const int src = (reflect(2 * g + par, n) - par) >> 1;
+        return (g - gw) | (min(max(src - gw, 0), 32 * Q - 1) << 16);
+    };
+    w.fix = xb < 0 || xb + 64 * Q1 > a.lv[0].w;
+    w.fix1e = w.fix1o = w.fix2e = w.fix2o = -1;
+    if (w.fix) {
+        w.fix1e = fix_of(g1w, a.lv[0].w, 0, Q1);
+        w.fix1o = fix_of(g1w, a.lv[0].w, 1, Q1);
+    }
+    w.ref1 = 0;
     int bx2h = 0, bx2l = 0, ne_r2 = 0;
     if constexpr (NL >= 2) {
-        const int g2w = w.xb >> 2;
+        const int g2w = xb >> 2;
         const int ne_c2 = (a.lv[1].w + 1) >> 1;
         ne_r2 = (a.lv[1].h + 1) >> 1;
-        w.x2 = make_ctx(g2w + W::Q2 * lane, W::Q2, a.lv[1].h, a.lv[1].w, a.lane_lo, a.lane_hi, a.lv[1].s);
+        w.x2 = make_ctx(g2w + W::Q2 * lane, W::Q2, a.lv[1].h, a.lv[1].w, a.lv[1].s);
         const int xh2 = ne_c2 + g2w, xl2 = g2w;
         bx2h = xh2 & ~AM;
         bx2l = xl2 & ~AM;
         w.o2h = xh2 - bx2h;
         w.o2l = xl2 - bx2l;
-        hfast = hfast && g2w >= 2 && g2w + 32 * W::Q2 + 2 <= (a.lv[1].w >> 1);
+        active = active && a.lv[1].w > 1 && a.lv[1].h > 1;
+        if (w.fix) {
+            w.fix2e = fix_of(g2w, a.lv[1].w, 0, W::Q2);
+            w.fix2o = fix_of(g2w, a.lv[1].w, 1, W::Q2);
+        }
+        if (!(a.lv[0].w & 1) && xb + 64 * Q1 > a.lv[0].w) w.ref1 = a.lv[0].w;
     }
-    hfast = hfast && w.vec_out;  // the border-free code stores whole vectors
     w.e1.init();
     if constexpr (NL >= 2) w.e2.init();
 
@@ -257,45 +348,38 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
 
     const uint32_t ring_s = smem_u32(ring);
     const uint32_t bar_s = smem_u32(bars);
+    // Lane k issues box k of a slot, all with one instruction: 2 fused levels
+    // HL1 LH1 HH1, LL2 HL2 LH2 HH2; one level LL1 HL1 LH1 HH1.
+    constexpr int NB = NL == 1 ? 4 : 7;  // boxes per slot
+    constexpr int N1 = NL == 1 ? 4 : 3;  // of level 1
+    const bool fine = lane < N1;
+    const int band = fine ? lane + (4 - N1) : lane - N1;  // 0 LL, 1 HL, 2 LH, 3 HH
+    const CUtensorMap* map = band == 0 ? mlp : (fine ? m1p : m2p);
+    const int box_x = fine ? ((band & 1) ? bx1h : bx1l) : ((band & 1) ? bx2h : bx2l);
+    int box_y = fine ? (band >= 2 ? ne_r1 : 0) + qbase : (band >= 2 ? ne_r2 : 0) + qbase / 2 + LAG;
+    const uint32_t box_dst = (uint32_t)((fine ? lane * Lay::R1 : N1 * Lay::R1 + band * Lay::R2) * sizeof(S));
+    // slots are issued in order, one after the other
     auto issue = [&](int s) {
         const int b = s % kInvSlots;
-        const uint32_t dst = ring_s + (uint32_t)(b * Lay::SLOT * sizeof(S));
         const uint32_t bar = bar_s + 8 * b;
-        const int q0 = qbase + SR * s;
         const bool l1 = s >= PRO_SLOTS;
-        uint32_t bytes = 0;
-        if (l1) bytes += (NL == 1 ? 4 : 3) * Lay::BYTES1;
-        if (NL == 2) bytes += 4 * Lay::BYTES2;
-        mbar_arrive_expect_tx(bar, bytes);
-        if constexpr (NL == 1) {
-            tma_load_2d(dst + 0 * Lay::R1 * sizeof(S), mlp, bx1l, q0, bar);
-            tma_load_2d(dst + 1 * Lay::R1 * sizeof(S), m1p, bx1h, q0, bar);
-            tma_load_2d(dst + 2 * Lay::R1 * sizeof(S), m1p, bx1l, ne_r1 + q0, bar);
-            tma_load_2d(dst + 3 * Lay::R1 * sizeof(S), m1p, bx1h, ne_r1 + q0, bar);
-        } else {
-            if (l1) {
-                tma_load_2d(dst + 0 * Lay::R1 * sizeof(S), m1p, bx1h, q0, bar);
-                tma_load_2d(dst + 1 * Lay::R1 * sizeof(S), m1p, bx1l, ne_r1 + q0, bar);
-                tma_load_2d(dst + 2 * Lay::R1 * sizeof(S), m1p, bx1h, ne_r1 + q0, bar);
-            }
-            const uint32_t d2 = dst + 3 * Lay::R1 * sizeof(S);
-            const int y2 = q0 / 2 + LAG;
-            tma_load_2d(d2 + 0 * Lay::R2 * sizeof(S), mlp, bx2l, y2, bar);
-            tma_load_2d(d2 + 1 * Lay::R2 * sizeof(S), m2p, bx2h, y2, bar);
-            tma_load_2d(d2 + 2 * Lay::R2 * sizeof(S), m2p, bx2l, ne_r2 + y2, bar);
-            tma_load_2d(d2 + 3 * Lay::R2 * sizeof(S), m2p, bx2h, ne_r2 + y2, bar);
-        }
+        if (lane == 0)
+            mbar_arrive_expect_tx(bar, (l1 ? N1 * Lay::BYTES1 : 0) + (NL == 2 ? 4 * Lay::BYTES2 : 0));
+        __syncwarp();
+        if (lane < NB && (l1 || !fine))
+            tma_load_2d(ring_s + (uint32_t)(b * Lay::SLOT * sizeof(S)) + box_dst, map, box_x, box_y, bar);
+        box_y += fine ? SR : SR / 2;
     };
     if (lane == 0) {
         for (int b = 0; b < kInvSlots; ++b) mbar_init(bar_s + 8 * b, 1);
         fence_mbar_init();
-        for (int s = 0; s < kInvSlots && s < nslots; ++s) issue(s);
     }
     __syncwarp();
+    for (int s = 0; s < kInvSlots && s < nslots; ++s) issue(s);
 
     // the border-free slots form one run [si0, si1) (see the forward body)
     int si0 = nslots, si1 = nslots;
-    if (hfast) {
+    if (active) {
         si0 = 0;
         while (si0 < nslots && !inv_rows_interior(qbase + SR * si0, SR, NL, LAG, no_r)) ++si0;
         si1 = nslots;
@@ -314,12 +398,12 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
         const int q0 = qbase + SR * s;
         const bool l1 = s >= PRO_SLOTS;
         if (s >= si0 && s < si1)
-            w.template slot<false>(ring + b * Lay::SLOT, q0, l1);
+            w.template slot<kInner>(ring + b * Lay::SLOT, q0, l1);
         else
-            w.template slot<true>(ring + b * Lay::SLOT, q0, l1);
+            w.template slot<kEdgeRows>(ring + b * Lay::SLOT, q0, l1);
         __syncwarp();
-        if (lane == 0 && s + kInvSlots < nslots) {
-            fence_proxy_async_smem();
+        if (s + kInvSlots < nslots) {
+            fence_proxy_async_smem();  // every lane: its reads and writes before the refill
             issue(s + kInvSlots);
         }
     }

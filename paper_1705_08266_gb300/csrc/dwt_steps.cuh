@@ -133,6 +133,25 @@ __device__ __forceinline__ void f_S_red(V& c0, V& c1, V& c2, V c3, V c1l, V c3l,
     c1 = vfma(UV, c3, c1);
 }
 
+// A quadruple's (c0, c1) and (c2, c3) are neighbouring pixels of an image row,
+// so they sit in register pairs as they are loaded: the vertical part of a
+// step runs on these pairs, (x, y) += p ((a0, a1) + (b0, b1)), as two packed
+// instructions.  PACK = false: scalar, for a step whose results leave the pair
+// anyway (the same bits).
+template <bool PACK>
+__device__ __forceinline__ void v_part(float& x, float& y, float a0, float a1, float b0, float b1,
+                                       float p) {
+    if constexpr (PACK) {
+        const float2 s = vadd(make_float2(a0, a1), make_float2(b0, b1));
+        const float2 r = vfma(splat<float2>(p), s, make_float2(x, y));
+        x = r.x;
+        y = r.y;
+    } else {
+        x = vfma(p, vadd(a0, b0), x);
+        y = vfma(p, vadd(a1, b1), y);
+    }
+}
+
 // -------------------------------------------------------------- integer ----
 // Reversible LeGall 5/3.  Floors are arithmetic right shifts (round toward
 // -inf).  The order T^H, T^V, S^H, S^V is the definition; the non-separable
