@@ -24,6 +24,10 @@ struct Group {
 
 }  // namespace
 
+// Row decomposition of a batched launch (see dwt2d_batch_create): warps per
+// SM of a large and of a small launch, and the segment rows in between.
+constexpr int kBatchWarpsLarge = 144, kBatchWarpsSmall = 12, kBatchSegRows = 16;
+
 constexpr int kMaxHostBands = 64;  // row bands of the pipelined host-buffer entry points
 
 struct dwt2d_plan_s {
@@ -71,13 +75,13 @@ struct dwt2d_plan_s {
 // A batch: per-image plans, workspace regions and the launch list.
 struct dwt2d_batch_s {
     struct Launch {
-        int fwd, elem_kind, nl;
+        int fwd, elem_kind, nl, q1;
         int first, count;  // entries [first, first + count) of the table
         int grid;
     };
     dwt2d_scheme scheme;
     bool pdl;  // launches with programmatic stream serialization
-    int q1;    // quadruple columns per lane of every launch (2 or 4)
+    int q1;    // queue mode: quadruple columns per lane (2 or 4)
     std::vector<dwt2d_batch_item> items;
     std::vector<dwt2d_plan_s*> plans;
     std::vector<size_t> region;             // workspace offset of each image's LL buffers
@@ -1319,14 +1323,18 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
             delete b;
             return s;
         }
-        p->fwd_q1 = p->inv_q1 = q1;
         b->plans.push_back(p);
     }
     // Launch list: phase k, then direction, storage type, fusion depth.  One
     // launch spreads its rows evenly: every warp streams the same number of
     // rows (segq), chosen so that the launch has about warps_per_sm warps per
-    // SM (default 48: four waves of the 12 resident, which evens out images
-    // whose border strips run the slower edge path).
+    // SM.  Default: 144 (12 waves of the 12 resident, so that the last one is
+    // short) while that leaves segments of 16 rows, whose halo rows cost a
+    // third; smaller launches run fewer waves of 16-row segments down to a
+    // single one, whose segments shrink.  256 images of 65-4096 pixels a side:
+    // 2134 us at a fixed 48, 1820 us; 64 images of 65-600: 150 and 132 us.
+    // 4 columns per lane where the launch is that large and 256-pixel strips
+    // cover its images with fewer pixels than 128-pixel ones.
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1338,11 +1346,18 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
         for (int fwd = 1; fwd >= 0; --fwd) {
             for (int ek = 0; ek < 4; ++ek) {
                 for (int nl = 1; nl <= 2; ++nl) {
-                    dwt2d_batch_s::Launch L = {fwd, ek, nl, (int)b->refs.size(), 0, 0};
-                    struct Cand { int i, w0, rows, rho, nstrips; };
+                    dwt2d_batch_s::Launch L = {fwd, ek, nl, 2, (int)b->refs.size(), 0, 0};
+                    struct Cand { int i, w0, rows, rho; };
                     std::vector<Cand> cand;
-                    long long work = 0;  // strips x rows over the launch
+                    // strips x rows over the launch with 2 and with 4 columns per lane
+                    long long work2 = 0, work4 = 0;
                     int min_segq = 1;
+                    auto strips = [&](const dwt2d_plan_s* p, const Cand& c, int q, int segq, FusedArgs* a) {
+                        memset(a, 0, sizeof(*a));
+                        int grid = 0;
+                        decompose(p, c.w0, c.rows, nl, c.rho, q, 1, a, &grid, 4, segq);
+                        return (long long)a->nstrips;
+                    };
                     for (int i = 0; i < n; ++i) {
                         const dwt2d_plan_s* p = b->plans[i];
                         if ((items[i].inverse == 0) != (fwd == 1) || elem_kind_of(p->dtype) != ek ||
@@ -1357,27 +1372,31 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                         c.w0 = p->ws[g.first];
                         c.rows = fwd ? (p->hs[g.first + g.n - 1] + 1) / 2 : (p->hs[g.first] + 1) / 2;
                         FusedArgs a;
-                        memset(&a, 0, sizeof(a));
-                        int grid = 0;
-                        decompose(p, c.w0, c.rows, nl, c.rho, q1, 1, &a, &grid, 4);
-                        c.nstrips = a.nstrips;
-                        work += (long long)c.nstrips * c.rows;
+                        work2 += strips(p, c, 2, 0, &a) * c.rows;
+                        work4 += strips(p, c, 4, 0, &a) * c.rows;
                         min_segq = std::max(min_segq, p->min_segq);
                         cand.push_back(c);
                     }
                     if (cand.empty()) continue;
-                    const long long target = (long long)sms * (wps > 0 ? wps : 48);
-                    const int segq = (int)std::max<long long>(min_segq, (work + target - 1) / target);
+                    if (tun.cols_per_lane != 0 || b->queue) {
+                        L.q1 = b->q1;
+                    } else if (fwd && ek != 1 && 2 * work4 < work2 &&
+                               work4 >= (long long)sms * kBatchWarpsLarge * kBatchSegRows) {
+                        L.q1 = 4;
+                    }
+                    const long long work = L.q1 == 4 ? work4 : work2;
+                    auto rows_at = [&](long long w) { return (work + sms * w - 1) / (sms * w); };
+                    const int segq = (int)std::max<long long>(
+                        min_segq, wps > 0 ? rows_at(wps)
+                                          : std::max(rows_at(kBatchWarpsLarge),
+                                                     std::min<long long>(kBatchSegRows,
+                                                                         rows_at(kBatchWarpsSmall))));
                     long long warps = 0;
                     for (const Cand& c : cand) {
-                        const dwt2d_plan_s* p = b->plans[c.i];
                         FusedArgs a;
-                        memset(&a, 0, sizeof(a));
-                        int grid = 0;
-                        decompose(p, c.w0, c.rows, nl, c.rho, q1, 1, &a, &grid, 4, segq);
+                        warps += strips(b->plans[c.i], c, L.q1, segq, &a) * a.nsegs;
                         b->refs.push_back({c.i, k});
                         b->segq.push_back(segq);
-                        warps += (long long)a.nstrips * a.nsegs;
                         ++L.count;
                     }
                     if (warps > (1LL << 30)) {
@@ -1459,13 +1478,14 @@ static dwt2d_status batch_upload(dwt2d_batch_t b, void* d_ws, void* h_staging, s
         for (int j = L.first; j < L.first + L.count; ++j) {
             const int i = b->refs[j].first, k = b->refs[j].second;
             const dwt2d_batch_item& it = b->items[i];
-            const dwt2d_plan_s* p = b->plans[i];
+            dwt2d_plan_s* p = b->plans[i];
+            p->fwd_q1 = p->inv_q1 = L.q1;
             GroupLaunch gl;
             dwt2d_status s = build_group(p, it.inverse == 0, k, it.d_src, it.src_pitch_bytes / p->elem,
                                          it.d_dst, it.dst_pitch_bytes / p->elem, wsb + b->region[i],
                                          err, 1, 1, &gl, b->segq[j]);
             if (s != DWT2D_OK) return s;
-            if (gl.path == 2 || gl.nl != L.nl || gl.q1 != b->q1) return DWT2D_ERR_INVALID;  // planned otherwise
+            if (gl.path == 2 || gl.nl != L.nl || gl.q1 != L.q1) return DWT2D_ERR_INVALID;  // planned otherwise
             BatchEntry& e = b->table[j];
             memcpy(e.m, gl.m, sizeof(e.m));
             e.args = gl.a;
@@ -1477,8 +1497,8 @@ static dwt2d_status batch_upload(dwt2d_batch_t b, void* d_ws, void* h_staging, s
         // kernel attributes once, outside any capture
         const int sch = base_scheme(b->scheme);
         const cudaError_t e =
-            L.fwd ? launch_fwd_batched(L.elem_kind, sch, L.nl, b->q1, nullptr, 0, 0, st, false)
-                  : launch_inv_batched(L.elem_kind, sch, L.nl, b->q1, nullptr, 0, 0, st, false);
+            L.fwd ? launch_fwd_batched(L.elem_kind, sch, L.nl, L.q1, nullptr, 0, 0, st, false)
+                  : launch_inv_batched(L.elem_kind, sch, L.nl, L.q1, nullptr, 0, 0, st, false);
         if (e != cudaSuccess) return DWT2D_ERR_CUDA;
     }
     // the tables go up from the caller's pinned staging buffer when given one
@@ -1566,9 +1586,9 @@ dwt2d_status dwt2d_batch_launch(dwt2d_batch_t b, void* d_ws, void* stream) {
     }
     for (const auto& L : b->launches) {
         const cudaError_t e =
-            L.fwd ? launch_fwd_batched(L.elem_kind, sch, L.nl, b->q1, table + L.first, L.count, L.grid,
+            L.fwd ? launch_fwd_batched(L.elem_kind, sch, L.nl, L.q1, table + L.first, L.count, L.grid,
                                        st, b->pdl)
-                  : launch_inv_batched(L.elem_kind, sch, L.nl, b->q1, table + L.first, L.count, L.grid,
+                  : launch_inv_batched(L.elem_kind, sch, L.nl, L.q1, table + L.first, L.count, L.grid,
                                        st, b->pdl);
         if (e != cudaSuccess) return DWT2D_ERR_CUDA;
     }
