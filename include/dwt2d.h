@@ -132,10 +132,11 @@ typedef struct {
     int32_t inv_warps_per_sm;      /* the same for the inverse (default 12) */
     int32_t fwd_warps_per_sm_large;/* forward launches whose row segments stay at least
                                       large_segment rows long at this many warps per SM take it
-                                      (default 48 for CDF 9/7, 44 for LeGall 5/3 at 2 columns per
-                                      lane, 24 at 4; -1: never) */
-    int32_t inv_warps_per_sm_large;/* the same for the inverse (default 64 at 2 columns per lane,
-                                      24 at 4; -1: never) */
+                                      (default 48 for CDF 9/7, 64 for LeGall 5/3 at 2 columns per
+                                      lane, 32 at 4; -1: never) */
+    int32_t inv_warps_per_sm_large;/* the same for the inverse (default 64 for CDF 9/7 in 32 bits,
+                                      32 in 16, 80 for LeGall 5/3 at 2 columns per lane, 24 at 4;
+                                      -1: never) */
     int32_t large_segment;         /* that threshold, quadruple rows of the launch's last level
                                       (default 16) */
     int32_t min_segment;           /* shortest row segment of a warp (default 2) */
@@ -155,7 +156,7 @@ typedef struct {
                                       cut into segments this many times shorter, 2-64, so that
                                       the launch drains quickly (default 3 at 2 columns per lane,
                                       4 at 4; -1: off) */
-    int32_t inv_short_tail;        /* the same for the inverse (default 4) */
+    int32_t inv_short_tail;        /* the same for the inverse (default 4; 3 for LeGall 5/3) */
 } dwt2d_plan_options;
 
 /*
@@ -341,16 +342,18 @@ typedef struct {
 
 /* Tuning knobs (0 = library default): levels fused in the first launch of an
  * image (1 or 2; default 2), at most per later launch (1 or 2; default 2),
- * warps per SM that the rows of one launch are cut into (default 48; the
- * batched kernels keep 12 warps per SM resident, 8 for the persistent form
- * at 4 columns per lane, so 48 is four or six waves), the
- * smallest row segment of a warp (quadruple rows of the last fused level;
- * default 2), and whether the batch's launches use programmatic stream
+ * warps per SM that the rows of one launch are cut into (the batched kernels
+ * keep 12 warps per SM resident, 8 for the persistent form at 4 columns per
+ * lane; default 144 while segments keep 16 rows, down to 12 for small
+ * launches), the smallest row segment of a warp (quadruple rows of the last
+ * fused level; default 2), and whether the batch's launches use programmatic stream
  * serialization (1 on, -1 or 0 off: measured neutral to 1 % slower for
  * batches).  Every warp of a launch streams the same number of rows.
  * cols_per_lane: quadruple columns per lane at the first level of a launch
- * (0 or 2: 2, a 128-pixel strip per warp; 4: a 256-pixel strip with half the
- * strips' halo overlap; any other value is DWT2D_ERR_INVALID). */
+ * (2: a 128-pixel strip per warp; 4: a 256-pixel strip with half the strips'
+ * halo overlap; 0: 2, but 4 for large forward CDF 9/7 launches of the table
+ * form that 256-pixel strips cover with fewer pixels; any other value is
+ * DWT2D_ERR_INVALID). */
 typedef struct {
     int32_t fuse_first, fuse_max, warps_per_sm, min_segment;
     int32_t programmatic_launch;

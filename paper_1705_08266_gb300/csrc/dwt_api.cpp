@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "dwt2d.h"
@@ -20,6 +21,15 @@ constexpr size_t kHeader = 256;  // status word + padding at the start of the wo
 struct Group {
     int first;  // first level of the group (0-based)
     int n;      // levels fused
+};
+
+// One streaming launch of a plan: a level group, its argument block, its
+// tensor maps and its grid.
+struct GroupLaunch {
+    int path;  // 0: forward (TMA); 1: inverse (TMA ring); 2: inverse (row-wise loads)
+    int nl, q1, grid;
+    FusedArgs a;
+    CUtensorMap m[3];
 };
 
 }  // namespace
@@ -62,6 +72,11 @@ struct dwt2d_plan_s {
     size_t size_a, size_b;  // bytes of the two LL buffers
     long long pitch_a, pitch_b, pitch_x;  // elements
     size_t ws_bytes;
+    // the launches of a forward call (k < ngroups), then those of an inverse
+    // call, without buffers: their shapes depend on the plan alone, and
+    // deriving them on every call took about as long as a kernel launch (null
+    // for the plans of a batch, which shapes its own launches)
+    GroupLaunch* shapes;
     // profiling hook: events[2i] / events[2i+1] around launch i
     cudaEvent_t* events;
     int nevents;
@@ -314,55 +329,30 @@ int elem_kind_of(dwt2d_dtype d) {
     }
 }
 
-// One streaming launch of a plan: level group `gi`, its argument block, its
-// tensor maps and its grid.
-struct GroupLaunch {
-    int path;  // 0: forward (TMA); 1: inverse (TMA ring); 2: inverse (row-wise loads)
-    int nl, q1, grid;
-    FusedArgs a;
-    CUtensorMap m[3];
-};
-
 // Launch k of a plan in its direction (forward: group k; inverse: group
-// ngroups - 1 - k).  Inter-launch LL buffers live in the plan's workspace
-// layout at `ws`; the status word is `err`.
-dwt2d_status build_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src, long long src_pe,
-                         void* dst, long long dst_pe, char* ws, int* err, int fwd_target,
-                         int inv_target, GroupLaunch* out, int segq_fixed = 0,
-                         bool uniform_segments = false, bool plan_only = false) {
+// ngroups - 1 - k) but for its buffers: levels, scales, columns per lane and
+// row decomposition.
+void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv_target, GroupLaunch* out,
+                 int segq_fixed = 0, bool uniform_segments = false) {
     const int sch = base_scheme(p->scheme);
     const int elem_kind = elem_kind_of(p->dtype);
     const int rho = p->wavelet == DWT2D_CDF97 ? 2 : 1;
-    void* bufs[2] = {ws + p->off_a, ws + p->off_b};
-    const long long bpitch[2] = {p->pitch_a, p->pitch_b};
-    const long long belems[2] = {(long long)(p->size_a / p->elem), (long long)(p->size_b / p->elem)};
     FusedArgs& a = out->a;
     memset(&a, 0, sizeof(a));
-    a.err = err;
+    const Group g = p->groups[fwd ? k : p->ngroups - 1 - k];
+    for (int i = 0; i < g.n; ++i) {
+        a.lv[i].h = p->hs[g.first + i];
+        a.lv[i].w = p->ws[g.first + i];
+        level_scale(a.lv[i].h, a.lv[i].w, !fwd, a.lv[i].s);
+    }
+    out->nl = g.n;
     if (fwd) {
-        const int gi = k;
-        const Group g = p->groups[gi];
-        for (int i = 0; i < g.n; ++i) {
-            a.lv[i].h = p->hs[g.first + i];
-            a.lv[i].w = p->ws[g.first + i];
-            level_scale(a.lv[i].h, a.lv[i].w, false, a.lv[i].s);
-        }
-        // input: the image, else the LL the previous launch wrote
-        const void* in = gi == 0 ? src : bufs[(gi - 1) & 1];
-        const long long in_pitch = gi == 0 ? src_pe : bpitch[(gi - 1) & 1];
-        a.mallat = dst;
-        a.mallat_pitch = dst_pe;
-        a.mallat_elems = (long long)p->H * dst_pe;
-        const bool last = gi == p->ngroups - 1;
-        a.ll = last ? dst : bufs[gi & 1];
-        a.ll_pitch = last ? dst_pe : bpitch[gi & 1];
-        a.ll_elems = last ? a.mallat_elems : belems[gi & 1];
         const int hN = a.lv[g.n - 1].h;
         // an LL the next launch reads stays in L2 (evict-last stores) when it
         // takes at most a third of it: 2-4 % faster at 8192^2 float32 and
         // 16384^2 16-bit, slower once it crowds out the launch's own stream
         const long long ll_bytes = (long long)((hN + 1) / 2) * ((a.lv[g.n - 1].w + 1) / 2) * p->elem;
-        a.ll_keep = !last && 3 * ll_bytes <= p->l2_bytes;
+        a.ll_keep = k != p->ngroups - 1 && 3 * ll_bytes <= p->l2_bytes;
         const int rows = (hN + 1) / 2;
         // quadruple columns per lane: 4 for three fused levels; with
         // fwd_q1 == 0 (automatic), 4 for a float launch whose rows still give
@@ -380,10 +370,6 @@ dwt2d_status build_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src
             use4 = big4.segq >= p->large_segq;
             if (use4) q1 = 4;
         }
-        dwt2d_status s = plan_only ? DWT2D_OK
-                                   : make_map(&out->m[0], in, a.lv[0].h, a.lv[0].w, in_pitch, p->elem,
-                                              elem_kind, 64 * q1, fwd_slot_rows(g.n, q1));
-        if (s != DWT2D_OK) return s;
         if (use4) {
             a = big4;
             out->grid = grid4;
@@ -405,49 +391,13 @@ dwt2d_status build_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src
             }
         }
         out->path = 0;
-        out->nl = g.n;
         out->q1 = q1;
-        return DWT2D_OK;
+        return;
     }
-    // inverse: coarse group first; the coarsest LL sits at the top-left of the
-    // Mallat array, later ones in the buffer the previous launch wrote
-    const int gi = p->ngroups - 1 - k;
-    const Group g = p->groups[gi];
-    for (int i = 0; i < g.n; ++i) {
-        a.lv[i].h = p->hs[g.first + i];
-        a.lv[i].w = p->ws[g.first + i];
-        level_scale(a.lv[i].h, a.lv[i].w, true, a.lv[i].s);
-    }
-    const void* ll_in = k == 0 ? src : bufs[(k - 1) & 1];
-    const long long ll_pitch = k == 0 ? src_pe : bpitch[(k - 1) & 1];
-    a.mallat = const_cast<void*>(src);
-    a.mallat_pitch = src_pe;
-    a.ll = const_cast<void*>(ll_in);
-    a.ll_pitch = ll_pitch;
-    const bool last = gi == 0;
-    a.out = last ? dst : bufs[k & 1];
-    a.out_pitch = last ? dst_pe : bpitch[k & 1];
-    a.out_elems = last ? (long long)p->H * dst_pe : belems[k & 1];
-    out->nl = g.n;
     if (g.n <= 2) {
-        // TMA ring: boxes of the Mallat array and of the LL source.  2 columns
-        // per lane unless 4 are asked for (measured: 4 is 7 % slower for the
-        // 8192^2 finest launch, 5 % faster at 16384^2 float32)
+        // 2 columns per lane unless 4 are asked for
         const int rows = (a.lv[0].h + 1) / 2;
         const int q1 = p->inv_q1 == 4 ? 4 : 2;
-        const int al = 16 / p->elem;  // boxes start at a 16-byte boundary
-        const int w1 = 32 * q1 + al, w2 = 16 * q1 + al;
-        const int sr = inv_slot_rows(q1);  // level-1 box rows; level-2 boxes sr / 2
-        dwt2d_status s = plan_only ? DWT2D_OK
-                                   : make_map(&out->m[0], src, p->H, p->W, src_pe, p->elem, elem_kind, w1, sr);
-        if (s == DWT2D_OK && !plan_only)
-            s = make_map(&out->m[1], src, p->H, p->W, src_pe, p->elem, elem_kind, w2, sr / 2);
-        const int llh = (a.lv[g.n - 1].h + 1) / 2, llw = (a.lv[g.n - 1].w + 1) / 2;
-        const bool ll_is_src = k == 0;
-        if (s == DWT2D_OK && !plan_only)
-            s = make_map(&out->m[2], ll_in, ll_is_src ? p->H : llh, ll_is_src ? p->W : llw, ll_pitch,
-                         p->elem, elem_kind, g.n == 1 ? w1 : w2, g.n == 1 ? sr : sr / 2);
-        if (s != DWT2D_OK) return s;
         const int res = resident_per_sm(false, g.n, q1, sch);
         const int large = q1 == 4 ? p->inv_warps_large4 : p->inv_warps_large;
         const int sd = uniform_segments ? 0 : p->inv_short;
@@ -472,7 +422,63 @@ dwt2d_status build_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src
         out->path = 2;
         out->q1 = 4;
     }
-    return DWT2D_OK;
+}
+
+// The buffers of launch k: pointers, pitches and tensor maps.  Inter-launch
+// LL buffers live in the plan's workspace layout at `ws`; the status word is
+// `err`.
+dwt2d_status bind_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src, long long src_pe,
+                        void* dst, long long dst_pe, char* ws, int* err, GroupLaunch* out) {
+    const int elem_kind = elem_kind_of(p->dtype);
+    void* bufs[2] = {ws + p->off_a, ws + p->off_b};
+    const long long bpitch[2] = {p->pitch_a, p->pitch_b};
+    const long long belems[2] = {(long long)(p->size_a / p->elem), (long long)(p->size_b / p->elem)};
+    FusedArgs& a = out->a;
+    a.err = err;
+    const bool last = k == p->ngroups - 1;
+    // input: the image (coefficients), else the LL the previous launch wrote
+    const void* in = k == 0 ? src : bufs[(k - 1) & 1];
+    const long long in_pitch = k == 0 ? src_pe : bpitch[(k - 1) & 1];
+    if (fwd) {
+        a.mallat = dst;
+        a.mallat_pitch = dst_pe;
+        a.mallat_elems = (long long)p->H * dst_pe;
+        a.ll = last ? dst : bufs[k & 1];
+        a.ll_pitch = last ? dst_pe : bpitch[k & 1];
+        a.ll_elems = last ? a.mallat_elems : belems[k & 1];
+        return make_map(&out->m[0], in, a.lv[0].h, a.lv[0].w, in_pitch, p->elem, elem_kind, 64 * out->q1,
+                        fwd_slot_rows(out->nl, out->q1));
+    }
+    // inverse: coarse group first; the coarsest LL sits at the top-left of the
+    // Mallat array, later ones in the buffer the previous launch wrote
+    a.mallat = const_cast<void*>(src);
+    a.mallat_pitch = src_pe;
+    a.ll = const_cast<void*>(in);
+    a.ll_pitch = in_pitch;
+    a.out = last ? dst : bufs[k & 1];
+    a.out_pitch = last ? dst_pe : bpitch[k & 1];
+    a.out_elems = last ? (long long)p->H * dst_pe : belems[k & 1];
+    if (out->path != 1) return DWT2D_OK;
+    // TMA ring: boxes of the Mallat array and of the LL source
+    const int q1 = out->q1, nl = out->nl;
+    const int al = 16 / p->elem;  // boxes start at a 16-byte boundary
+    const int w1 = 32 * q1 + al, w2 = 16 * q1 + al;
+    const int sr = inv_slot_rows(q1);  // level-1 box rows; level-2 boxes sr / 2
+    dwt2d_status s = make_map(&out->m[0], src, p->H, p->W, src_pe, p->elem, elem_kind, w1, sr);
+    if (s == DWT2D_OK) s = make_map(&out->m[1], src, p->H, p->W, src_pe, p->elem, elem_kind, w2, sr / 2);
+    const int llh = (a.lv[nl - 1].h + 1) / 2, llw = (a.lv[nl - 1].w + 1) / 2;
+    if (s == DWT2D_OK)
+        s = make_map(&out->m[2], in, k == 0 ? p->H : llh, k == 0 ? p->W : llw, in_pitch, p->elem, elem_kind,
+                     nl == 1 ? w1 : w2, nl == 1 ? sr : sr / 2);
+    return s;
+}
+
+dwt2d_status build_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src, long long src_pe,
+                         void* dst, long long dst_pe, char* ws, int* err, int fwd_target,
+                         int inv_target, GroupLaunch* out, int segq_fixed = 0,
+                         bool uniform_segments = false) {
+    shape_group(p, fwd, k, fwd_target, inv_target, out, segq_fixed, uniform_segments);
+    return bind_group(p, fwd, k, src, src_pe, dst, dst_pe, ws, err, out);
 }
 
 dwt2d_status run_fused(const dwt2d_plan_s* p, bool fwd, const void* src, int64_t sp, void* dst,
@@ -483,8 +489,10 @@ dwt2d_status run_fused(const dwt2d_plan_s* p, bool fwd, const void* src, int64_t
     int* err = reinterpret_cast<int*>(wsb);
     for (int k = 0; k < p->ngroups; ++k) {
         GroupLaunch gl;
-        dwt2d_status s = build_group(p, fwd, k, src, sp / p->elem, dst, dp / p->elem, wsb, err,
-                                     p->fwd_warps_target, p->inv_warps_target, &gl);
+        if (p->shapes) gl = p->shapes[fwd ? k : p->ngroups + k];
+        else shape_group(p, fwd, k, p->fwd_warps_target, p->inv_warps_target, &gl);
+        const dwt2d_status s =
+            bind_group(p, fwd, k, src, sp / p->elem, dst, dp / p->elem, wsb, err, &gl);
         if (s != DWT2D_OK) return s;
         gl.a.pdl = p->pdl;
         cudaError_t e;
@@ -660,16 +668,31 @@ size_t dwt::plan_workspace_bytes(dwt2d_plan_t p) { return p ? p->ws_bytes : 0; }
 
 extern "C" {
 
+// What a plan needs to know of the current device.
+struct DeviceInfo {
+    int sms;
+    long long l2_bytes;
+};
+static DeviceInfo device_info() {
+    int dev = 0, sms = 148, l2 = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaGetLastError();
+    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) l2 = 0;
+    cudaGetLastError();
+    return {sms, l2};
+}
+
 static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width, int32_t levels,
                                 dwt2d_wavelet wavelet, dwt2d_scheme scheme, dwt2d_boundary boundary,
                                 dwt2d_dtype dtype, size_t* workspace_bytes, const dwt2d_tuning* tuning,
-                                const dwt2d_plan_options* opts);
+                                const dwt2d_plan_options* opts, const DeviceInfo& dev);
 
 dwt2d_status dwt2d_plan(dwt2d_plan_t* out, int32_t height, int32_t width, int32_t levels,
                         dwt2d_wavelet wavelet, dwt2d_scheme scheme, dwt2d_boundary boundary,
                         dwt2d_dtype dtype, size_t* workspace_bytes) {
     return plan_create(out, height, width, levels, wavelet, scheme, boundary, dtype, workspace_bytes,
-                       nullptr, nullptr);
+                       nullptr, nullptr, device_info());
 }
 
 dwt2d_status dwt2d_plan_ex(dwt2d_plan_t* out, int32_t height, int32_t width, int32_t levels,
@@ -677,7 +700,7 @@ dwt2d_status dwt2d_plan_ex(dwt2d_plan_t* out, int32_t height, int32_t width, int
                            dwt2d_dtype dtype, const dwt2d_plan_options* options,
                            size_t* workspace_bytes) {
     return plan_create(out, height, width, levels, wavelet, scheme, boundary, dtype, workspace_bytes,
-                       nullptr, options);
+                       nullptr, options, device_info());
 }
 
 }  // extern "C"
@@ -706,7 +729,7 @@ static bool options_ok(const dwt2d_plan_options& o) {
 static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width, int32_t levels,
                                 dwt2d_wavelet wavelet, dwt2d_scheme scheme, dwt2d_boundary boundary,
                                 dwt2d_dtype dtype, size_t* workspace_bytes, const dwt2d_tuning* tuning,
-                                const dwt2d_plan_options* opts) {
+                                const dwt2d_plan_options* opts, const DeviceInfo& dev) {
     if (!out || !workspace_bytes) return DWT2D_ERR_INVALID;
     *out = nullptr;
     dwt2d_plan_options o;
@@ -760,15 +783,9 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
         ++p->ngroups;
         l += n;
     }
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaGetLastError();
+    const int sms = dev.sms;
     p->sm_count = sms;
-    int l2 = 0;
-    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) l2 = 0;
-    cudaGetLastError();
-    p->l2_bytes = l2;
+    p->l2_bytes = dev.l2_bytes;
     p->fwd_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.fwd_warps_per_sm, 16));
     p->inv_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
@@ -855,6 +872,12 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
         p->pitch_x = px;
     }
     p->ws_bytes = off;
+    if (!tuning && !multipass(scheme)) {
+        p->shapes = new (std::nothrow) GroupLaunch[2 * p->ngroups]();
+        for (int k = 0; p->shapes && k < 2 * p->ngroups; ++k)
+            shape_group(p, k < p->ngroups, k % p->ngroups, p->fwd_warps_target, p->inv_warps_target,
+                        &p->shapes[k]);
+    }
     *workspace_bytes = off;
     *out = p;
     return DWT2D_OK;
@@ -1257,9 +1280,7 @@ dwt2d_status dwt2d_plan_launch_info(dwt2d_plan_t p, int32_t inverse, int32_t i, 
     if (multipass(p->scheme) || (convolution(p->scheme) && !inverse)) return DWT2D_ERR_UNSUPPORTED;
     if (i >= p->ngroups) return DWT2D_ERR_INVALID;
     GroupLaunch gl;
-    const dwt2d_status s = build_group(p, !inverse, i, nullptr, 1, nullptr, 1, nullptr, nullptr,
-                                       p->fwd_warps_target, p->inv_warps_target, &gl, 0, false, true);
-    if (s != DWT2D_OK) return s;
+    shape_group(p, !inverse, i, p->fwd_warps_target, p->inv_warps_target, &gl);
     if (fused) *fused = gl.nl;
     if (cols_per_lane) *cols_per_lane = gl.q1;
     if (warps) *warps = gl.a.nstrips * gl.a.nsegs;
@@ -1279,6 +1300,7 @@ void dwt2d_plan_destroy(dwt2d_plan_t p) {
         cudaStreamDestroy(p->host_out);
         for (auto& e : p->host_ev) cudaEventDestroy(e);
     }
+    if (p) delete[] p->shapes;
     free(p);
 }
 
@@ -1308,12 +1330,13 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
     b->items.assign(items, items + n);
     size_t off = kHeader;
     b->table_off = off;
+    const DeviceInfo dev = device_info();
     for (int i = 0; i < n; ++i) {
         const dwt2d_batch_item& it = items[i];
         dwt2d_plan_t p = nullptr;
         size_t wsb = 0;
         dwt2d_status s = plan_create(&p, it.height, it.width, it.levels, it.wavelet, scheme,
-                                     DWT2D_SYMMETRIC_WHOLE, it.dtype, &wsb, &tun, nullptr);
+                                     DWT2D_SYMMETRIC_WHOLE, it.dtype, &wsb, &tun, nullptr, dev);
         if (s == DWT2D_OK && (it.inverse != 0 && it.inverse != 1)) s = DWT2D_ERR_INVALID;
         if (s == DWT2D_OK) s = check_buffers(p, it.d_src, it.src_pitch_bytes, it.d_dst,
                                              it.dst_pitch_bytes, it.d_src);
@@ -1335,10 +1358,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
     // 2134 us at a fixed 48, 1820 us; 64 images of 65-600: 150 and 132 us.
     // 4 columns per lane where the launch is that large and 256-pixel strips
     // cover its images with fewer pixels than 128-pixel ones.
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaGetLastError();
+    const int sms = dev.sms;
     int max_groups = 0;
     for (auto* p : b->plans) max_groups = std::max(max_groups, p->ngroups);
     b->warps = 0;
@@ -1416,7 +1436,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
     b->sms = sms;
     // queues: the launches of one (direction, storage type), in launch order
     // (level group by level group)
-    for (int fwd = 1; fwd >= 0; --fwd) {
+    for (int fwd = 1; fwd >= 0 && b->queue; --fwd) {
         for (int ek = 0; ek < 4; ++ek) {
             dwt2d_batch_s::Queue q = {fwd, ek, (int)b->qorder.size(), 0, 0};
             for (const auto& L : b->launches) {
@@ -1451,7 +1471,8 @@ dwt2d_status dwt2d_batch_upload(dwt2d_batch_t b, void* d_ws, void* stream) {
 
 dwt2d_status dwt2d_batch_staging_bytes(dwt2d_batch_t b, size_t* bytes) {
     if (!b || !bytes) return DWT2D_ERR_INVALID;
-    *bytes = (b->refs.size() + b->qorder.size()) * sizeof(BatchEntry);
+    // the table of the batch's form: the launches', or the queues' (the same entries)
+    *bytes = b->refs.size() * sizeof(BatchEntry);
     return DWT2D_OK;
 }
 
@@ -1494,26 +1515,17 @@ static dwt2d_status batch_upload(dwt2d_batch_t b, void* d_ws, void* h_staging, s
             e.first_warp = first_warp;
             first_warp += gl.a.nstrips * gl.a.nsegs;
         }
-        // kernel attributes once, outside any capture
-        const int sch = base_scheme(b->scheme);
-        const cudaError_t e =
-            L.fwd ? launch_fwd_batched(L.elem_kind, sch, L.nl, L.q1, nullptr, 0, 0, st, false)
-                  : launch_inv_batched(L.elem_kind, sch, L.nl, L.q1, nullptr, 0, 0, st, false);
-        if (e != cudaSuccess) return DWT2D_ERR_CUDA;
     }
-    // the tables go up from the caller's pinned staging buffer when given one
+    // the table goes up from the caller's pinned staging buffer when given one
     // (a copy from pageable memory may wait for the stream to drain)
-    auto upload = [&](size_t dev_off, const std::vector<BatchEntry>& v, size_t stage_off) {
+    auto upload = [&](size_t dev_off, const std::vector<BatchEntry>& v) {
         if (v.empty()) return cudaSuccess;
         const size_t bytes = v.size() * sizeof(BatchEntry);
         const void* srcp = v.data();
-        if (h_staging) {
-            memcpy(static_cast<char*>(h_staging) + stage_off, v.data(), bytes);
-            srcp = static_cast<char*>(h_staging) + stage_off;
-        }
+        if (h_staging) srcp = memcpy(h_staging, v.data(), bytes);
         return cudaMemcpyAsync(wsb + dev_off, srcp, bytes, cudaMemcpyHostToDevice, st);
     };
-    if (upload(b->table_off, b->table, 0) != cudaSuccess) return DWT2D_ERR_CUDA;
+    if (!b->queue && upload(b->table_off, b->table) != cudaSuccess) return DWT2D_ERR_CUDA;
     // queue mode: the same entries queue by queue, numbered within their
     // queue, with their done counters and the group each depends on
     b->qtable.clear();
@@ -1540,15 +1552,8 @@ static dwt2d_status batch_upload(dwt2d_batch_t b, void* d_ws, void* h_staging, s
         }
         q.items = first;
         if (first > (1LL << 30)) return DWT2D_ERR_INVALID;
-        const int sch = base_scheme(b->scheme);
-        const cudaError_t e = q.fwd ? launch_fwd_queue(q.elem_kind, sch, b->q1, nullptr, 0, 0, nullptr,
-                                                       nullptr, nullptr, 0, st)
-                                    : launch_inv_queue(q.elem_kind, sch, b->q1, nullptr, 0, 0, nullptr,
-                                                       nullptr, nullptr, 0, st);
-        if (e != cudaSuccess) return DWT2D_ERR_CUDA;
     }
-    if (upload(b->qtable_off, b->qtable, b->table.size() * sizeof(BatchEntry)) != cudaSuccess)
-        return DWT2D_ERR_CUDA;
+    if (b->queue && upload(b->qtable_off, b->qtable) != cudaSuccess) return DWT2D_ERR_CUDA;
     if (cudaMemsetAsync(d_ws, 0, sizeof(int), st) != cudaSuccess) return DWT2D_ERR_CUDA;
     return DWT2D_OK;
 }

@@ -26,9 +26,7 @@ template <class S, int SCH, int NL, int Q1>
 static cudaError_t launch_one(const CUtensorMap& map, const FusedArgs& a, int grid,
                               cudaStream_t st) {
     auto k = fwd_fused_kernel<S, SCH, NL, Q1>;
-    const size_t smem = fwd_smem_bytes(sizeof(S), NL, Q1);
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+    const size_t smem = fwd_smem_bytes(sizeof(S), NL, Q1);  // below the 48 KB that need an opt-in
     return launch_kernel(k, grid, kFwdWarps * 32, smem, st, a.pdl != 0, map, a);
 }
 

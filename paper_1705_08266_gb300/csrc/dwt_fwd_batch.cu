@@ -81,8 +81,6 @@ static cudaError_t launch_queue_one(const BatchEntry* table, int n, int total, i
                                     int* err, int grid, cudaStream_t st) {
     auto k = fwd_queue_kernel<S, SCH, Q1>;
     const size_t smem = queue_smem(sizeof(S), Q1);
-    if (grid == 0)
-        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return launch_kernel(k, grid, kFwdWarps * 32, smem, st, false, table, n, total, head, done, err);
 }
 
@@ -121,8 +119,6 @@ static cudaError_t launch_batched_one(const BatchEntry* table, int n, int grid, 
                                       bool pdl) {
     auto k = fwd_batched_kernel<S, SCH, NL, Q1>;
     const size_t smem = fwd_smem_bytes(sizeof(S), NL, Q1);
-    if (grid == 0)
-        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return launch_kernel(k, grid, kFwdWarps * 32, smem, st, pdl, table, n);
 }
 

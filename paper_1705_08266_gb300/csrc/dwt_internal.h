@@ -108,8 +108,8 @@ size_t fwd_smem_bytes(int elem_bytes, int nl, int q1);
 // Batched forward / inverse: entries of one element type, scheme, fusion
 // depth (1 or 2) and quadruple columns per lane q1 (2 or 4); `grid` CTAs of
 // kFwdWarps (forward) or kInvTmaWarps (inverse) warps.
-// grid == 0 only sets the kernel's shared-memory attribute (done once, before
-// any stream capture), so a launch itself is a plain kernel launch.
+// Rings stay below the 48 KB of shared memory that need an opt-in, so a launch
+// is a plain kernel launch.
 cudaError_t launch_fwd_batched(int elem, int scheme, int nl, int q1, const BatchEntry* table, int n,
                                int grid, cudaStream_t st, bool pdl);
 cudaError_t launch_inv_batched(int elem, int scheme, int nl, int q1, const BatchEntry* table, int n,

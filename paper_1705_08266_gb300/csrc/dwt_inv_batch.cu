@@ -77,8 +77,6 @@ static cudaError_t inv_queue_one(const BatchEntry* table, int n, int total, int*
                                  int* err, int grid, cudaStream_t st) {
     auto k = inv_queue_kernel<S, SCH, Q1>;
     const size_t smem = inv_queue_smem(sizeof(S), Q1);
-    if (grid == 0)
-        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return launch_kernel(k, grid, kInvWarps * 32, smem, st, false, table, n, total, head, done, err);
 }
 
@@ -117,8 +115,6 @@ static cudaError_t inv_batched_one(const BatchEntry* table, int n, int grid, cud
                                    bool pdl) {
     auto k = inv_batched_kernel<S, SCH, NL, Q1>;
     const size_t smem = inv_tma_smem_bytes(sizeof(S), NL, Q1);
-    if (grid == 0)
-        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return launch_kernel(k, grid, kInvWarps * 32, smem, st, pdl, table, n);
 }
 

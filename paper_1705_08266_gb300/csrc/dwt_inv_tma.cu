@@ -37,9 +37,7 @@ static cudaError_t inv_launch_one(const CUtensorMap& m1, const CUtensorMap& m2,
                                   const CUtensorMap& ml, const FusedArgs& a, int grid,
                                   cudaStream_t st) {
     auto k = inv_tma_kernel<S, SCH, NL, Q1>;
-    const size_t smem = inv_tma_smem_bytes(sizeof(S), NL, Q1);
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+    const size_t smem = inv_tma_smem_bytes(sizeof(S), NL, Q1);  // below the 48 KB that need an opt-in
     return launch_kernel(k, grid, kInvWarps * 32, smem, st, a.pdl != 0, m1, m2, ml, a);
 }
 

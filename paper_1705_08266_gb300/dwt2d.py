@@ -145,9 +145,12 @@ def _check(status: int, what: str):
         raise DwtError(status, what)
 
 
-def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    # the raw handle, where torch offers it without building a Stream object
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
 
 
 def pitch_elems(width: int, dtype: torch.dtype) -> int:
@@ -164,8 +167,8 @@ def empty_image(height: int, width: int, dtype=torch.float32, device="cuda") -> 
 
 def as_pitched(t: torch.Tensor) -> torch.Tensor:
     """t itself if its rows are 16-byte aligned and unit-stride, else a pitched copy."""
-    es = t.element_size()
-    if t.dim() == 2 and t.stride(1) == 1 and (t.stride(0) * es) % 16 == 0 and t.data_ptr() % 16 == 0:
+    st = t.stride()
+    if len(st) == 2 and st[1] == 1 and (st[0] * t.element_size()) % 16 == 0 and t.data_ptr() % 16 == 0:
         return t
     out = empty_image(t.shape[0], t.shape[1], t.dtype, t.device)
     out.copy_(t)
@@ -258,11 +261,10 @@ class Plan:
         if own_ws:
             workspace = self.workspace(src.device, stream)
         es = src.element_size()
-        st = getattr(lib(), name)(self._h, ctypes.c_void_p(src.data_ptr()), src.stride(0) * es,
-                                  ctypes.c_void_p(dst.data_ptr()), dst.stride(0) * es,
-                                  ctypes.c_void_p(workspace.data_ptr()), float(scale),
-                                  _stream_ptr(stream))
-        _check(st, name)
+        st = getattr(_lib, name)(self._h, src.data_ptr(), src.stride(0) * es, dst.data_ptr(),
+                                 dst.stride(0) * es, workspace.data_ptr(), float(scale), _stream_ptr(stream))
+        if st:
+            _check(st, name)
         if own_ws:
             # nobody else can read the status word of a workspace made here:
             # read it now (synchronizes the stream) so kernel errors surface
