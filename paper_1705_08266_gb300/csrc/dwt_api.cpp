@@ -62,6 +62,7 @@ struct dwt2d_plan_s {
     int inv_warps_large4;
     int inv_q1;  // the same for the inverse
     int min_segq;
+    bool fill;  // segments fill whole slots (unless the shortest segment was asked for)
     int pdl;  // device entry points: launches with programmatic stream serialization
     int fwd_short, inv_short;  // short last-wave segments: divisor (0: off)
     int fwd_seg_f;  // forward segment interleave (0: as many groups as waves)
@@ -262,12 +263,27 @@ int resident_per_sm(bool fwd, int nl, int q1, int scheme) {
     return q1 <= 2 ? (scheme == SCH_NONSEP ? 12 : 16) : 12;
 }
 
+// The longest segment that streams as many slots as one of `segq` rows: a
+// segment's halo rows and its own fill whole slots, so that no slot is mostly
+// rows of the next segment (2048 x 2048, two levels: 103 segments of 5 rows
+// and 6 slots became 86 of 6 rows and 6 slots).
+int fill_slots(bool fwd, int nl, int rho, int q1, int segq) {
+    if (nl > 2) return segq;
+    const int sr = fwd ? fwd_slot_rows(nl, q1) / 2 : inv_slot_rows(q1);
+    const int sh = fwd ? nl - 1 : 0;  // log2 of level-1 rows per row of a segment
+    // level-1 halo rows, both sides, with the alignment of the first one
+    const int halo = fwd ? (nl == 1 ? 2 * rho : 6 * rho + (rho & 1)) : 2 * rho + (nl == 2 ? (rho & 1) : 0);
+    const int slots = ((segq << sh) + halo + sr - 1) / sr;
+    const int full = (slots * sr - halo) >> sh;
+    return std::max(segq, full);
+}
+
 // Warp work decomposition of one streaming launch.
 // Rows per warp: enough segments for target_warps warps, or segq_fixed (> 0).
 // With short_div > 1 the rows at the bottom that one wave of resident warps
 // (resident per SM) takes are cut into segments short_div times shorter and
 // taken last: the launch's last warps are short, so it drains quickly.
-void decompose(const dwt2d_plan_s* p, int w_first, int rows, int nl, int rho, int q1,
+void decompose(const dwt2d_plan_s* p, bool fwd, int w_first, int rows, int nl, int rho, int q1,
                int target_warps, FusedArgs* a, int* grid, int warps_per_block, int segq_fixed = 0,
                int resident = 16, int short_div = 0, int seg_f_opt = 0) {
     valid_lanes(nl, rho, q1, &a->lane_lo, &a->lane_hi);
@@ -287,6 +303,8 @@ void decompose(const dwt2d_plan_s* p, int w_first, int rows, int nl, int rho, in
         segq = (rows + nsegs - 1) / nsegs;
     }
     if (segq < p->min_segq) segq = p->min_segq;
+    const bool fill = segq_fixed <= 0 && p->fill;
+    if (fill) segq = fill_slots(fwd, nl, rho, q1, segq);
     if (segq > rows) segq = rows;
     if (segq < 1) segq = 1;
     a->segq = segq;
@@ -295,7 +313,8 @@ void decompose(const dwt2d_plan_s* p, int w_first, int rows, int nl, int rho, in
     a->segq2 = segq;
     const int res_warps = p->sm_count * resident;
     if (short_div > 1 && segq_fixed <= 0) {
-        const int sq2 = std::max(std::max(p->min_segq, 1), segq / short_div);
+        int sq2 = std::max(std::max(p->min_segq, 1), segq / short_div);
+        if (fill) sq2 = fill_slots(fwd, nl, rho, q1, sq2);
         const int nshort = std::max(1, res_warps / a->nstrips);  // one wave of short segments
         const int big = (rows - nshort * sq2) / segq;               // whole long segments above them
         if (sq2 < segq && big >= 1) {
@@ -364,7 +383,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         bool use4 = false;
         if (g.n <= 2 && p->fwd_q1 == 0 && segq_fixed <= 0 && elem_kind != 1 && p->fwd_warps_large4 > 0) {
             big4 = a;
-            decompose(p, a.lv[0].w, rows, g.n, rho, 4, p->fwd_warps_large4, &big4, &grid4, kFwdWarps, 0,
+            decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, p->fwd_warps_large4, &big4, &grid4, kFwdWarps, 0,
                       resident_per_sm(true, g.n, 4, sch), uniform_segments ? 0 : p->fwd_short4,
                       p->fwd_seg_f);
             use4 = big4.segq >= p->large_segq;
@@ -377,12 +396,12 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             const int res = resident_per_sm(true, g.n, q1, sch);
             const int large = q1 == 4 ? p->fwd_warps_large4 : p->fwd_warps_large;
             const int sd = uniform_segments ? 0 : (q1 == 4 ? p->fwd_short4 : p->fwd_short);
-            decompose(p, a.lv[0].w, rows, g.n, rho, q1, fwd_target, &a, &out->grid, kFwdWarps,
+            decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, fwd_target, &a, &out->grid, kFwdWarps,
                       segq_fixed, res, 0, p->fwd_seg_f);
             if (segq_fixed <= 0 && large > fwd_target) {
                 FusedArgs b = a;
                 int grid_b = 0;
-                decompose(p, a.lv[0].w, rows, g.n, rho, q1, large, &b, &grid_b, kFwdWarps, 0, res, sd,
+                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, large, &b, &grid_b, kFwdWarps, 0, res, sd,
                           p->fwd_seg_f);
                 if (b.segq >= p->large_segq) {
                     a = b;
@@ -402,12 +421,12 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         const int large = q1 == 4 ? p->inv_warps_large4 : p->inv_warps_large;
         const int sd = uniform_segments ? 0 : p->inv_short;
         // the inverse measured fastest with its segments top to bottom
-        decompose(p, a.lv[0].w, rows, g.n, rho, q1, inv_target, &a, &out->grid, kInvTmaWarps,
+        decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, inv_target, &a, &out->grid, kInvTmaWarps,
                   segq_fixed, res, 0, p->inv_seg_f);
         if (segq_fixed <= 0 && large > inv_target) {
             FusedArgs b = a;
             int grid_b = 0;
-            decompose(p, a.lv[0].w, rows, g.n, rho, q1, large, &b, &grid_b, kInvTmaWarps, 0, res, sd,
+            decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, large, &b, &grid_b, kInvTmaWarps, 0, res, sd,
                       p->inv_seg_f);
             if (b.segq >= p->large_segq) {
                 a = b;
@@ -417,7 +436,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         out->path = 1;
         out->q1 = q1;
     } else {
-        decompose(p, a.lv[0].w, (a.lv[0].h + 1) / 2, g.n, rho, 4, inv_target, &a, &out->grid, 4, 0,
+        decompose(p, false, a.lv[0].w, (a.lv[0].h + 1) / 2, g.n, rho, 4, inv_target, &a, &out->grid, 4, 0,
                   8, 0, p->inv_seg_f);
         out->path = 2;
         out->q1 = 4;
@@ -791,6 +810,7 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->inv_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.inv_warps_per_sm, 12));
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
+    p->fill = o.min_segment == 0;
     // measured at 8192^2: the first forward launch is fastest at 48 warps
     // per SM (3 waves of 16) for CDF 9/7 and at 44 for LeGall 5/3 (its
     // shorter halo) with 2 columns per lane, at 24 (2 waves of 12) with 4;
@@ -949,7 +969,7 @@ static int seg_input_end(const dwt2d_plan_s* p, const FusedArgs& a, int nl, int 
         }
     }
     const int rows = fwd_slot_rows(nl, q1), sr = rows / 2;  // image / quadruple rows per slot
-    const int qstart = std::max(f, 0) & ~(sr - 1), qend = e + 1;
+    const int qstart = std::max(f, 0) & ~(fwd_row_align(nl) - 1), qend = e + 1;
     const int nslots = (qend - qstart + sr - 1) / sr;
     return std::min(2 * qstart + rows * nslots, p->H);
 }
@@ -1145,7 +1165,7 @@ static dwt2d_status run_host_inv_pipelined(dwt2d_plan_s* p, const void* h_src, i
     auto ready = [&](int seg, int c) {  // rows segment `seg` reads are all in after band c
         if (c == B - 1) return true;
         const int A0 = seg * base.segq, A1 = std::min(A0 + base.segq, ne_r1);
-        const int qstart = std::max(A0 - lag, 0) & ~(sr - 1);
+        const int qstart = std::max(A0 - lag, 0) & ~(inv_row_align(n0) - 1);
         const int nmain = (A1 + lag - qstart + sr - 1) / sr;
         const int end1 = std::min(qstart + sr * nmain, ne_r1);
         if (end1 > std::min((c + 1) * rb, ne_r1)) return false;
@@ -1375,7 +1395,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                     auto strips = [&](const dwt2d_plan_s* p, const Cand& c, int q, int segq, FusedArgs* a) {
                         memset(a, 0, sizeof(*a));
                         int grid = 0;
-                        decompose(p, c.w0, c.rows, nl, c.rho, q, 1, a, &grid, 4, segq);
+                        decompose(p, fwd == 1, c.w0, c.rows, nl, c.rho, q, 1, a, &grid, 4, segq);
                         return (long long)a->nstrips;
                     };
                     for (int i = 0; i < n; ++i) {
@@ -1406,11 +1426,13 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                     }
                     const long long work = L.q1 == 4 ? work4 : work2;
                     auto rows_at = [&](long long w) { return (work + sms * w - 1) / (sms * w); };
-                    const int segq = (int)std::max<long long>(
+                    int segq = (int)std::max<long long>(
                         min_segq, wps > 0 ? rows_at(wps)
                                           : std::max(rows_at(kBatchWarpsLarge),
                                                      std::min<long long>(kBatchSegRows,
                                                                          rows_at(kBatchWarpsSmall))));
+                    if (wps <= 0 && tun.min_segment <= 0)
+                        segq = fill_slots(fwd == 1, nl, cand[0].rho, L.q1, segq);
                     long long warps = 0;
                     for (const Cand& c : cand) {
                         FusedArgs a;

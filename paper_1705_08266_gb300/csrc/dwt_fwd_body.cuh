@@ -223,10 +223,9 @@ struct FwdWarp {
     }
 
     // One slot: level-1 input quadruple rows q0 .. q0+SR-1 (q0 a multiple of
-    // SR) in shared memory (2 SR image rows of BW pixels), pushed as one
-    // block.  With q0 % SR == 0 the rows every level emits, and how LL rows
-    // pair into the next level's quadruple rows, are fixed by the pipeline lag
-    // alone.
+    // fwd_row_align) in shared memory (2 SR image rows of BW pixels), pushed as
+    // one block.  The rows every level emits, and how LL rows pair into the
+    // next level's quadruple rows, are then fixed by the pipeline lag alone.
     // Level-2 input rows of the slot at q0: LL rows q0 - 2 .. q0 + SR - 3
     // paired into quadruple rows q0/2 - 1 .. q0/2 + SR/2 - 2.
     template <int R2>
@@ -361,7 +360,7 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
             e = 2 * e + 1;
         }
     }
-    const int qstart = max(f, 0) & ~(SR - 1);  // slots hold SR quadruple rows, aligned
+    const int qstart = max(f, 0) & ~(fwd_row_align(NL) - 1);
     const int qend = e + 1;
     const int nslots = (qend - qstart + SR - 1) / SR;
 

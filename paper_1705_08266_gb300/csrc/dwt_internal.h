@@ -100,6 +100,14 @@ constexpr int kFwdWarps = 1;
 constexpr int kFwdSlots = 3;        // TMA ring depth per warp
 constexpr int kFwdSlotRows = 8;     // image rows per TMA box (4 quadruple rows) with 2 columns per lane
 
+// First quadruple row of a work item, forward: a multiple of this.  A slot of
+// 1 or 2 fused levels may start at any row or pair of rows (the LL rows of the
+// lag pair up all the same), which saves the halo up to a slot against starts
+// at a multiple of the slot; three levels pair rows across slots.
+__host__ __device__ constexpr int fwd_row_align(int nl) { return nl == 1 ? 1 : (nl == 2 ? 2 : 4); }
+// The same for the inverse (two levels: a whole level-2 row).
+__host__ __device__ constexpr int inv_row_align(int nl) { return nl == 1 ? 1 : 2; }
+
 // Image rows per TMA box of the forward kernel: 8, or 4 with 4 quadruple
 // columns per lane and at most 2 fused levels.
 int fwd_slot_rows(int nl, int q1);

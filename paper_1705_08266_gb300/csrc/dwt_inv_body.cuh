@@ -337,7 +337,7 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
     if constexpr (NL >= 2) w.e2.init();
 
     // level-1 input rows of this item: outputs [A0, A1) need [A0 - RHO, A1 - 1 + LAG]
-    const int qstart = max(w.A0 - RHO, 0) & ~(SR - 1);
+    const int qstart = max(w.A0 - RHO, 0) & ~(inv_row_align(NL) - 1);
     const int nmain = (w.A1 + LAG - qstart + SR - 1) / SR;
     const int nslots = nmain + PRO_SLOTS;
     const int qbase = qstart - SR * PRO_SLOTS;

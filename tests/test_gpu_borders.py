@@ -1,0 +1,99 @@
+"""Image borders by mirrored data, unaligned bands, and where work items start.
+
+Sizes at the edges of strips (a strip whose last column, or whose halo, lies
+outside the image), widths shorter than a halo, odd and even, in both tile
+widths, forward and inverse, against the FP64 oracle; segments of every short
+length; the row decomposition of batches.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import lifting as L
+from paper_1705_08266_gb300 import dwt2d as D
+from tests.parity_util import (assert_forward_matches, assert_inverse_matches, device_image, host,
+                               make_input)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    D.lib()
+
+
+# strips store 104 / 120 columns (2 / 1 fused levels) with 2 columns per lane
+# and 224 / 240 with 4
+EDGE_WIDTHS = [2, 3, 4, 5, 6, 7, 9, 12, 15, 16, 17, 18, 31, 33, 103, 104, 105, 106, 113, 119, 120, 121, 122,
+               207, 208, 209, 210, 223, 224, 225, 226, 239, 240, 241, 242, 447, 448, 449, 450]
+
+
+@pytest.mark.parametrize("cols", [2, 4])
+@pytest.mark.parametrize("wavelet,scheme", [("cdf97", "nonsep_reduced"), ("cdf97", "separable"),
+                                            ("cdf97", "nonsep"), ("legall53", "nonsep_reduced")])
+def test_strip_edges(wavelet, scheme, cols):
+    for w in EDGE_WIDTHS:
+        for h, levels in ((19, 3), (40, 2), (2, 1)):
+            x = make_input(wavelet, h, w, seed=w * 3 + h)
+            plan = D.Plan(h, w, levels, wavelet, scheme,
+                          options=dict(fwd_cols_per_lane=cols, inv_cols_per_lane=cols))
+            ws = plan.workspace()
+            tag = f"{wavelet} {scheme} cols={cols} {h}x{w} L{levels}"
+            c = plan.forward(device_image(x), workspace=ws)
+            assert_forward_matches(host(c), x, levels, wavelet, tag)
+            ref = L.forward(x, levels, wavelet).astype(x.dtype)
+            y = plan.inverse(device_image(ref), workspace=ws)
+            assert_inverse_matches(host(y), ref, levels, wavelet, x, tag)
+            assert plan.status(ws) == 0, tag
+
+
+# rows that leave 1 .. a slot's rows in the last segment, at both fusion depths
+@pytest.mark.parametrize("wavelet", ["cdf97", "legall53"])
+@pytest.mark.parametrize("fuse", [1, 2])
+def test_slot_starts(wavelet, fuse):
+    """Work items start at any row (one fused level) or pair of rows (two):
+    every segment length from 1 up gives the same bits, forward and inverse."""
+    for h in (37, 38, 39, 40, 130):
+        w = 150
+        x = make_input(wavelet, h, w, seed=h)
+        xd = device_image(x)
+        ref = None
+        for seg in (1, 2, 3, 4, 5, 7, 8, 1000, 0):
+            opts = dict(fuse_max=fuse)
+            if seg:
+                opts.update(min_segment=seg, fwd_warps_per_sm=60000, inv_warps_per_sm=60000)
+            plan = D.Plan(h, w, 3, wavelet, options=opts)
+            ws = plan.workspace()
+            c = plan.forward(xd, workspace=ws)
+            y = plan.inverse(c, workspace=ws)
+            torch.cuda.synchronize()
+            assert plan.status(ws) == 0
+            if ref is None:
+                ref = (c.clone(), y.clone())
+                assert_forward_matches(host(c), x, 3, wavelet, f"{h} fuse {fuse}")
+            assert torch.equal(c, ref[0]) and torch.equal(y, ref[1]), (h, fuse, seg)
+
+
+def test_default_batch_rows_equal_tuned_ones():
+    """The default row decomposition of batches (by the size of each launch,
+    4 columns per lane for large ones) gives the bits of a fixed one."""
+    rng = np.random.default_rng(5)
+    jobs = []
+    for _ in range(24):
+        h, w = int(rng.integers(65, 3000)), int(rng.integers(65, 3000))
+        x = D.empty_image(h, w)
+        x.copy_(torch.rand(h, w, device="cuda"))
+        jobs.append((x, D.empty_image(h, w), int(rng.integers(1, 6)), "cdf97", 0))
+    outs = []
+    for tuning in (None, dict(warps_per_sm=24, cols_per_lane=2)):
+        b = D.Batch(jobs, tuning=tuning)
+        ws = b.workspace()
+        b.upload(ws)
+        b.launch(ws)
+        torch.cuda.synchronize()
+        assert b.status(ws) == 0
+        outs.append([d.clone() for _s, d, _l, _w, _i in jobs])
+    for a, c in zip(*outs):
+        assert torch.equal(a, c)
