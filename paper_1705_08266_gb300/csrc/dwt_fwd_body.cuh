@@ -35,35 +35,34 @@ __device__ __forceinline__ void st_fast(S* p, const T (&v)[Q], bool ok, bool kee
     }
 }
 
-// The first n of a lane's Q values at p, whose row starts `al` elements past
-// a vector boundary (al < Q, the same for a whole band): aligned vectors, the
-// widest pieces an unaligned band allows, or the columns left at its edge.
-template <class S, class T, int Q>
-__device__ __forceinline__ void st_any(S* p, const T (&v)[Q], int n, int al, bool keep = false) {
-    if (n <= 0) return;
-    S w[Q];
-#pragma unroll
-    for (int j = 0; j < Q; ++j) w[j] = Storage<S>::st(v[j]);
-    if (!store_ok(p, n * (int)sizeof(S))) return;
-    if (n < Q) {
-#pragma unroll
-        for (int j = 0; j < Q; ++j)
-            if (j < n) p[j] = w[j];
-    } else if (al == 0) {
-        if (keep) st_vec_keep<S, Q>(p, w);
-        else st_vec<S, Q>(p, w);
-    } else if constexpr (Q == 4) {
-        if (al == 2) {
-            st_vec<S, 2>(p, *reinterpret_cast<const S(*)[2]>(w));
-            st_vec<S, 2>(p + 2, *reinterpret_cast<const S(*)[2]>(w + 2));
-        } else {
-            p[0] = w[0];
-            st_vec<S, 2>(p + 1, *reinterpret_cast<const S(*)[2]>(w + 1));
-            p[3] = w[3];
-        }
+// How a strip stores the bands of a level.  kWhole: every storing lane whole
+// aligned vectors; kHalves: the HL / HH bands start half a vector (of 4) off,
+// two halves each; kColumns: column by column, for other starts and for the
+// strips that the right border cuts.  One predicate per store and no branches:
+// a lane-dependent branch per store made border strips, which are most strips
+// of a small image, twice as long.
+enum StoreMode { kWhole = 0, kHalves = 1, kColumns = 2 };
+
+// A lane's Q values at p: whole vectors, or the first n of them.
+template <class S, class T, int Q, int MODE>
+__device__ __forceinline__ void st_band(S* p, const T (&v)[Q], bool ok, int n, bool keep = false) {
+    if constexpr (MODE == kWhole) {
+        st_fast<S, T, Q>(p, v, ok && n > 0, keep);
     } else {
+        S w[Q];
 #pragma unroll
-        for (int j = 0; j < Q; ++j) p[j] = w[j];
+        for (int j = 0; j < Q; ++j) w[j] = Storage<S>::st(v[j]);
+        ok = ok && n > 0 && store_ok(p, n * (int)sizeof(S));
+        if constexpr (MODE == kHalves && Q == 4) {
+            if (ok) {
+                st_vec<S, 2>(p, *reinterpret_cast<const S(*)[2]>(w));
+                st_vec<S, 2>(p + 2, *reinterpret_cast<const S(*)[2]>(w + 2));
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < Q; ++j)
+                if (ok && j < n) p[j] = w[j];
+        }
     }
 }
 
@@ -73,35 +72,26 @@ struct StoreGeo {
     int g0;          // first quadruple column of this lane
     int r_lo, r_hi;  // rows of this level that this work item stores
     int n_e, n_o;    // columns this lane stores of the LL / LH and of the HL / HH bands
-    int al;          // where the HL / HH rows start, in elements past a vector boundary
+    int mode;        // warp-uniform StoreMode
 };
 
-// The bands of rows r .. r + R - 1 whose rows the item owns.  WHOLE: every
-// storing lane stores whole aligned vectors and all rows exist; LAST: the LL
-// leaves the chip too.
-template <class S, class T, int Q, int R, bool WHOLE, bool LAST>
+// The bands of rows r .. r + R - 1 whose rows the item owns (and, with border
+// rows, that exist); LAST: the LL leaves the chip too.
+template <int E, class S, class T, int Q, int R, int MODE, bool LAST>
 __device__ __forceinline__ void store_rows(const Block<T, Q, R>& b, int r, const StoreGeo& g, S* mallat,
                                            long long mpitch, S* ll, long long llpitch, bool keep) {
+    constexpr int ME = MODE == kHalves ? kWhole : MODE;  // LL and LH start on a vector
     S* hl = mallat + (long long)r * mpitch + (g.g0 + g.ne_c);
     S* lh = hl + ((long long)g.ne_r * mpitch - g.ne_c);
     S* lrow = ll + (long long)r * llpitch + g.g0;
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         const bool in = r + k >= g.r_lo && r + k < g.r_hi;
-        if constexpr (WHOLE) {
-            const bool ok = in && g.n_e > 0;
-            st_fast<S, T, Q>(hl, b.r[k].c[1], ok);
-            st_fast<S, T, Q>(lh, b.r[k].c[2], ok);
-            st_fast<S, T, Q>(lh + g.ne_c, b.r[k].c[3], ok);
-            if constexpr (LAST) st_fast<S, T, Q>(lrow, b.r[k].c[0], ok, keep);
-        } else if (in && r + k < g.ne_r) {
-            st_any<S, T, Q>(hl, b.r[k].c[1], g.n_o, g.al);
-            if (r + k < g.no_r) {
-                st_any<S, T, Q>(lh, b.r[k].c[2], g.n_e, 0);
-                st_any<S, T, Q>(lh + g.ne_c, b.r[k].c[3], g.n_o, g.al);
-            }
-            if constexpr (LAST) st_any<S, T, Q>(lrow, b.r[k].c[0], g.n_e, 0, keep);
-        }
+        const bool even = in && (E == kInner || r + k < g.ne_r), odd = in && (E == kInner || r + k < g.no_r);
+        st_band<S, T, Q, MODE>(hl, b.r[k].c[1], even, g.n_o);
+        st_band<S, T, Q, ME>(lh, b.r[k].c[2], odd, g.n_e);
+        st_band<S, T, Q, MODE>(lh + g.ne_c, b.r[k].c[3], odd, g.n_o);
+        if constexpr (LAST) st_band<S, T, Q, ME>(lrow, b.r[k].c[0], even, g.n_e, keep);
         hl += mpitch;
         lh += mpitch;
         if constexpr (LAST) lrow += llpitch;
@@ -119,14 +109,11 @@ __device__ __forceinline__ StoreGeo make_geo(int h, int w, int g0, int Q, int r_
     g.r_hi = r_hi;
     g.n_e = lane_ok ? min(max(g.ne_c - g0, 0), Q) : 0;
     g.n_o = lane_ok ? min(max((w >> 1) - g0, 0), Q) : 0;
-    g.al = g.ne_c & (Q - 1);
+    const int al = g.ne_c & (Q - 1);  // where the HL / HH rows start, past a vector boundary
+    const bool whole = __all_sync(kFull, (g.n_e == 0 || g.n_e == Q) && g.n_o == g.n_e);
+    g.mode = !whole ? kColumns : al == 0 ? kWhole : Q == 4 && al == 2 ? kHalves : kColumns;
     return g;
 }
-// Every lane of the warp stores whole aligned vectors of this level or nothing.
-__device__ __forceinline__ bool geo_whole(const StoreGeo& g, int Q) {
-    return g.al == 0 && __all_sync(kFull, (g.n_e == 0 || g.n_e == Q) && g.n_o == g.n_e);
-}
-
 // Pair two consecutive LL rows (even row e, odd row o) of Q values into a
 // quadruple row of Q/2 columns for the next level.
 template <class T, int Q>
@@ -167,7 +154,6 @@ struct FwdWarp {
     S* mallat;
     S* ll;
     long long mpitch, llpitch;
-    bool whole;    // every lane stores whole aligned vectors (all fused levels)
     bool ll_keep;  // the next launch reads the LL back: store it L2 evict-last
     int lane;
     // border strips: columns outside the image that this lane fills with the
@@ -244,10 +230,12 @@ struct FwdWarp {
     // The rows of level L that a push emitted, from row r on.
     template <int E, int L, int Q, int R>
     __device__ __forceinline__ void store_level(const Block<T, Q, R>& b, int r, const StoreGeo& g) {
-        if (E == kInner && __builtin_expect(whole, 1))
-            store_rows<S, T, Q, R, true, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
+        if (__builtin_expect(g.mode == kWhole, 1))
+            store_rows<E, S, T, Q, R, kWhole, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
+        else if (E == kInner && Q == 4 && g.mode == kHalves)
+            store_rows<E, S, T, Q, R, kHalves, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
         else
-            store_rows<S, T, Q, R, false, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
+            store_rows<E, S, T, Q, R, kColumns, L == NL>(b, r, g, mallat, mpitch, ll, llpitch, ll_keep);
     }
 
     template <int E>
@@ -380,7 +368,6 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
         W.s1 = make_geo(a.lv[0].h, a.lv[0].w, g1, Q1, R0 << (NL - 1), R1 << (NL - 1), lane_ok);
         no_r[0] = a.lv[0].h >> 1;
         active = a.lv[0].w > 1 && a.lv[0].h > 1;
-        W.whole = geo_whole(W.s1, Q1);
     }
     if constexpr (NL >= 2) {
         const int g2 = (xb >> 2) + FW::Q2 * lane;
@@ -388,7 +375,6 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
         W.s2 = make_geo(a.lv[1].h, a.lv[1].w, g2, FW::Q2, R0 << (NL - 2), R1 << (NL - 2), lane_ok);
         no_r[1] = a.lv[1].h >> 1;
         active = active && a.lv[1].w > 1 && a.lv[1].h > 1;
-        W.whole = geo_whole(W.s2, FW::Q2) && W.whole;
     }
     if constexpr (NL >= 3) {
         const int g3 = (xb >> 3) + FW::Q3 * lane;
@@ -396,7 +382,6 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
         W.s3 = make_geo(a.lv[2].h, a.lv[2].w, g3, FW::Q3, R0, R1, lane_ok);
         no_r[2] = a.lv[2].h >> 1;
         active = active && a.lv[2].w > 1 && a.lv[2].h > 1;
-        W.whole = geo_whole(W.s3, FW::Q3) && W.whole;
     }
     // columns outside the image: up to 32 on each side, one per lane (the
     // halo of three fused levels takes 28)
