@@ -132,11 +132,11 @@ typedef struct {
     int32_t inv_warps_per_sm;      /* the same for the inverse (default 12) */
     int32_t fwd_warps_per_sm_large;/* forward launches whose row segments stay at least
                                       large_segment rows long at this many warps per SM take it
-                                      (default 48 for CDF 9/7, 64 for LeGall 5/3 at 2 columns per
-                                      lane, 32 at 4; -1: never) */
-    int32_t inv_warps_per_sm_large;/* the same for the inverse (default 64 for CDF 9/7 in 32 bits,
-                                      32 in 16, 80 for LeGall 5/3 at 2 columns per lane, 24 at 4;
-                                      -1: never) */
+                                      (default 48 for float32, 32 for 16-bit storage, 64 for
+                                      LeGall 5/3 at 2 columns per lane, 32 at 4; -1: never) */
+    int32_t inv_warps_per_sm_large;/* the same for the inverse (default 80 for float32, 48 for
+                                      16-bit storage, 96 for LeGall 5/3 at 2 columns per lane,
+                                      24 at 4; -1: never) */
     int32_t large_segment;         /* that threshold, quadruple rows of the launch's last level
                                       (default 16) */
     int32_t min_segment;           /* shortest row segment of a warp (default 2) */
@@ -144,9 +144,9 @@ typedef struct {
                                       (default: the launch's waves of resident warps; 1: top to
                                       bottom) */
     int32_t inv_seg_interleave;    /* the same for the inverse (default 1; -1: the launch's waves) */
-    int32_t fwd_cols_per_lane;     /* quadruple columns per lane, 2 or 4 (default: 4 for a float
+    int32_t fwd_cols_per_lane;     /* quadruple columns per lane, 2 or 4 (default: 4 for a float32
                                       launch of at most 2 fused levels whose rows give long
-                                      segments at 24 warps per SM, else 2) */
+                                      segments at 32 warps per SM, else 2) */
     int32_t inv_cols_per_lane;     /* the same for the inverse, 2 or 4 (default 2) */
     int32_t programmatic_launch;   /* device entry points launch with programmatic stream
                                       serialization (default on) */
@@ -154,9 +154,9 @@ typedef struct {
     int32_t host_pipeline;         /* *_host entry points overlap copies and transform (default on) */
     int32_t fwd_short_tail;        /* in a large launch, the rows one wave of warps takes last are
                                       cut into segments this many times shorter, 2-64, so that
-                                      the launch drains quickly (default 3 at 2 columns per lane,
-                                      4 at 4; -1: off) */
-    int32_t inv_short_tail;        /* the same for the inverse (default 4; 3 for LeGall 5/3) */
+                                      the launch drains quickly (default 4; 3 for float32 at 2
+                                      columns per lane; -1: off) */
+    int32_t inv_short_tail;        /* the same for the inverse (default 4) */
 } dwt2d_plan_options;
 
 /*

@@ -374,14 +374,14 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         a.ll_keep = k != p->ngroups - 1 && 3 * ll_bytes <= p->l2_bytes;
         const int rows = (hN + 1) / 2;
         // quadruple columns per lane: 4 for three fused levels; with
-        // fwd_q1 == 0 (automatic), 4 for a float launch whose rows still give
-        // long segments at the 4-column wave count (measured faster there:
-        // less halo and shuffle work per pixel), else 2
+        // fwd_q1 == 0 (automatic), 4 for a float32 launch whose rows still give
+        // long segments at the 4-column wave count, else 2 (16-bit storage,
+        // two levels of 8192^2: 89.1 us with 4, 78.6 with 2; 16384^2 268 and 260)
         int q1 = g.n >= 3 ? 4 : (p->fwd_q1 == 4 ? 4 : 2);
         FusedArgs big4;
         int grid4 = 0;
         bool use4 = false;
-        if (g.n <= 2 && p->fwd_q1 == 0 && segq_fixed <= 0 && elem_kind != 1 && p->fwd_warps_large4 > 0) {
+        if (g.n <= 2 && p->fwd_q1 == 0 && segq_fixed <= 0 && elem_kind == 0 && p->fwd_warps_large4 > 0) {
             big4 = a;
             decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, p->fwd_warps_large4, &big4, &grid4, kFwdWarps, 0,
                       resident_per_sm(true, g.n, 4, sch), uniform_segments ? 0 : p->fwd_short4,
@@ -811,17 +811,20 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
                                                                     : opt(o.inv_warps_per_sm, 12));
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
     p->fill = o.min_segment == 0;
-    // measured at 8192^2: the first forward launch is fastest at 48 warps
-    // per SM (3 waves of 16) for CDF 9/7 and at 44 for LeGall 5/3 (its
-    // shorter halo) with 2 columns per lane, at 24 (2 waves of 12) with 4;
-    // the small later ones at one wave
-    const int fwl = opt(o.fwd_warps_per_sm_large, wavelet == DWT2D_CDF97 ? 48 : 64);
+    // Warps per SM of a large launch (segments of at least large_segq rows), in
+    // waves of the resident warps (16 at 128 registers).  More warps: shorter
+    // last segments and a more compact set of rows in flight, but more halo
+    // rows.  Measured two-level launches, us (8192^2): forward float32, 4
+    // columns per lane 24 warps 105, 32 101.6, 48 112; 16-bit, 2 columns per
+    // lane 16 78.0, 32 78.6, 48 82.4 (16384^2: 282, 260, 259); 5/3 48 87.0, 64
+    // 87.1, 80 99.9.  Inverse float32 48 90.5, 64 90.1, 80 88.4, 96 89.9; 16-bit
+    // 32 80.6, 48 81.0 (16384^2: 281, 276); 5/3 64 85.4, 80 83.4, 96 82.5.
+    const int fwl = opt(o.fwd_warps_per_sm_large, half ? 32 : (wavelet == DWT2D_CDF97 ? 48 : 64));
     p->fwd_warps_large = (tuning && tuning->warps_per_sm > 0) || fwl < 0 ? 0 : sms * fwl;
     const int fwl4 = opt(o.fwd_warps_per_sm_large, 32);
     p->fwd_warps_large4 = (tuning && tuning->warps_per_sm > 0) || fwl4 < 0 ? 0 : sms * fwl4;
     p->large_segq = opt(o.large_segment, 16);
-    // the finest inverse launch: 64 warps per SM (4 waves of 16)
-    const int iwl = opt(o.inv_warps_per_sm_large, half ? 32 : (wavelet == DWT2D_CDF97 ? 64 : 80));
+    const int iwl = opt(o.inv_warps_per_sm_large, half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;
     p->fwd_q1 = o.fwd_cols_per_lane;  // 0: automatic
     p->pdl = opt(o.programmatic_launch, 1) > 0;
@@ -829,9 +832,9 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->inv_seg_f = o.inv_seg_interleave < 0 ? 0 : opt(o.inv_seg_interleave, 1);
     // short last-wave segments: measured 3 % (forward, 3 at 2 columns per
     // lane, 4 at 4) and 2 % (inverse, 4) faster at 8192^2
-    p->fwd_short = o.fwd_short_tail < 0 ? 0 : opt(o.fwd_short_tail, 3);
+    p->fwd_short = o.fwd_short_tail < 0 ? 0 : opt(o.fwd_short_tail, half || wavelet == DWT2D_LEGALL53 ? 4 : 3);
     p->fwd_short4 = o.fwd_short_tail < 0 ? 0 : opt(o.fwd_short_tail, 4);
-    p->inv_short = o.inv_short_tail < 0 ? 0 : opt(o.inv_short_tail, wavelet == DWT2D_CDF97 ? 4 : 3);
+    p->inv_short = o.inv_short_tail < 0 ? 0 : opt(o.inv_short_tail, 4);
     p->host_bands = opt(o.host_bands, 8);
     p->host_pipeline = opt(o.host_pipeline, 1) > 0;
     p->inv_q1 = o.inv_cols_per_lane == 4 ? 4 : 2;
