@@ -52,11 +52,13 @@ struct dwt2d_plan_s {
     int sm_count;
     long long l2_bytes;  // L2 cache of the device the plan was made on
     int fwd_warps_target, inv_warps_target;
-    // a forward launch whose rows allow segments of at least large_segq rows
+    // a forward launch whose rows allow segments of at least fwd_large_segq rows
     // at fwd_warps_large warps runs that many (several waves even out the
-    // strips' unequal costs); smaller launches keep fwd_warps_target
-    int fwd_warps_large, large_segq;
-    int inv_warps_large;  // the same rule for inverse launches
+    // strips' unequal costs), else at fwd_large_step less and so on; smaller
+    // launches keep fwd_warps_target
+    int fwd_warps_large, fwd_large_segq, fwd_large_segq1 /* one level */, fwd_large_step;
+    int inv_warps_large, inv_large_segq, inv_large_step;  // the same rule for inverse launches
+    int large_segq4;  // rows for 4 columns per lane without being asked
     int fwd_q1;  // quadruple columns per lane of the forward kernel (2 or 4; 0: automatic)
     int fwd_warps_large4, fwd_short4;  // the large-launch rule at 4 columns per lane
     int inv_warps_large4;
@@ -386,7 +388,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, p->fwd_warps_large4, &big4, &grid4, kFwdWarps, 0,
                       resident_per_sm(true, g.n, 4, sch), uniform_segments ? 0 : p->fwd_short4,
                       p->fwd_seg_f);
-            use4 = big4.segq >= p->large_segq;
+            use4 = big4.segq >= p->large_segq4;
             if (use4) q1 = 4;
         }
         if (use4) {
@@ -398,14 +400,15 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             const int sd = uniform_segments ? 0 : (q1 == 4 ? p->fwd_short4 : p->fwd_short);
             decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, fwd_target, &a, &out->grid, kFwdWarps,
                       segq_fixed, res, 0, p->fwd_seg_f);
-            if (segq_fixed <= 0 && large > fwd_target) {
+            for (int t = large; segq_fixed <= 0 && t > fwd_target; t -= p->fwd_large_step) {
                 FusedArgs b = a;
                 int grid_b = 0;
-                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, large, &b, &grid_b, kFwdWarps, 0, res, sd,
+                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kFwdWarps, 0, res, sd,
                           p->fwd_seg_f);
-                if (b.segq >= p->large_segq) {
+                if (b.segq >= (g.n == 1 ? p->fwd_large_segq1 : p->fwd_large_segq)) {
                     a = b;
                     out->grid = grid_b;
+                    break;
                 }
             }
         }
@@ -423,14 +426,15 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         // the inverse measured fastest with its segments top to bottom
         decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, inv_target, &a, &out->grid, kInvTmaWarps,
                   segq_fixed, res, 0, p->inv_seg_f);
-        if (segq_fixed <= 0 && large > inv_target) {
+        for (int t = large; segq_fixed <= 0 && t > inv_target; t -= p->inv_large_step) {
             FusedArgs b = a;
             int grid_b = 0;
-            decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, large, &b, &grid_b, kInvTmaWarps, 0, res, sd,
+            decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kInvTmaWarps, 0, res, sd,
                       p->inv_seg_f);
-            if (b.segq >= p->large_segq) {
+            if (b.segq >= p->inv_large_segq) {
                 a = b;
                 out->grid = grid_b;
+                break;
             }
         }
         out->path = 1;
@@ -808,10 +812,10 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->fwd_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.fwd_warps_per_sm, 16));
     p->inv_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
-                                                                    : opt(o.inv_warps_per_sm, 12));
+                                                                    : opt(o.inv_warps_per_sm, half ? 16 : 12));
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
     p->fill = o.min_segment == 0;
-    // Warps per SM of a large launch (segments of at least large_segq rows), in
+    // Warps per SM of a large launch (segments of at least *_large_segq rows), in
     // waves of the resident warps (16 at 128 registers).  More warps: shorter
     // last segments and a more compact set of rows in flight, but more halo
     // rows.  Measured two-level launches, us (8192^2): forward float32, 4
@@ -823,7 +827,24 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->fwd_warps_large = (tuning && tuning->warps_per_sm > 0) || fwl < 0 ? 0 : sms * fwl;
     const int fwl4 = opt(o.fwd_warps_per_sm_large, 32);
     p->fwd_warps_large4 = (tuning && tuning->warps_per_sm > 0) || fwl4 < 0 ? 0 : sms * fwl4;
-    p->large_segq = opt(o.large_segment, 16);
+    // A launch whose segments would be shorter than this many rows (level-2
+    // rows forward, level-1 rows inverse) takes a wave less, and so on down to
+    // the count of the small launches: where the halo rows cost more than a
+    // shorter end gives.  Before, it took the small count at once.  Two levels,
+    // us, small count / chosen: forward float32 3000 x 9000 45.9 / 44.1, 8191 x
+    // 4095 55.8 / 53.1, 5/3 50.4 / 46.0; inverse float32 3000 x 9000 49.4 /
+    // 43.3, 5/3 45.2 / 36.9, 8191 x 4095 61.1 / 45.5.  16-bit launches are bound
+    // by their arithmetic and want long segments: forward 3000 x 9000 16 warps
+    // 36.7, 32 warps (14 rows) 42.5; inverse 6000^2 47.7 and 49.2 (33 rows).
+    // Small 16-bit inverses: 16 warps for 12, 1500 x 3000 13.9 -> 12.0, 6 levels
+    // of 4099 x 2051 36.2 -> 31.8.
+    p->fwd_large_segq = opt(o.large_segment, half ? 40 : 13);
+    p->fwd_large_segq1 = opt(o.large_segment, half ? 40 : 20);
+    p->inv_large_segq = opt(o.large_segment, half ? 40 : 20);
+    p->large_segq4 = opt(o.large_segment, 16);
+    // counts that were asked for are taken or left as a whole
+    p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * 16 : 1 << 28;
+    p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * 16 : 1 << 28;
     const int iwl = opt(o.inv_warps_per_sm_large, half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;
     p->fwd_q1 = o.fwd_cols_per_lane;  // 0: automatic

@@ -97,3 +97,23 @@ def test_default_batch_rows_equal_tuned_ones():
         outs.append([d.clone() for _s, d, _l, _w, _i in jobs])
     for a, c in zip(*outs):
         assert torch.equal(a, c)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.int32, torch.float16])
+@pytest.mark.parametrize("h,w,levels", [(2500, 5000, 2), (3001, 4097, 1), (6000, 1500, 3), (3000, 9000, 2)])
+def test_middle_sizes_equal_one_wave(h, w, levels, dtype):
+    """Between the small launches and the large ones the wave count follows the
+    segments' length: the default plan gives the bits of one-wave launches."""
+    wavelet = "legall53" if dtype == torch.int32 else "cdf97"
+    x = D.empty_image(h, w, dtype)
+    x.copy_((torch.rand(h, w, device="cuda") * 100).to(dtype))
+    outs = []
+    for options in (None, dict(fwd_warps_per_sm_large=-1, inv_warps_per_sm_large=-1)):
+        plan = D.Plan(h, w, levels, wavelet, "nonsep_reduced", dtype, options=options)
+        ws = plan.workspace()
+        c = plan.forward(x, workspace=ws)
+        y = plan.inverse(x, workspace=ws)
+        torch.cuda.synchronize()
+        assert plan.status(ws) == 0
+        outs.append((c, y))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
