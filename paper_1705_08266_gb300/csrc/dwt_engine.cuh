@@ -238,6 +238,25 @@ __device__ __forceinline__ int find_entry(const BatchEntry* __restrict__ table, 
     return lo;
 }
 
+// The argument block of a table entry in shared memory: the warp copies it
+// with a load or two per lane, and the body reads its fields from there where
+// the single-image kernels read the constant bank.  In registers they took the
+// place of the lifting state: the queue kernels spilled up to 72 bytes per
+// thread.  A multiple of 128 bytes, so the ring behind it stays aligned for TMA.
+struct alignas(128) SharedArgs {
+    FusedArgs a;
+};
+__device__ __forceinline__ void copy_args(SharedArgs* to, const FusedArgs& from) {
+    static_assert(kFwdWarps == 1 && kInvTmaWarps == 1, "one block of arguments per CTA");
+    static_assert(sizeof(FusedArgs) % 4 == 0, "copied by words");
+    const int* s = reinterpret_cast<const int*>(&from);
+    int* d = reinterpret_cast<int*>(&to->a);
+    __syncwarp();  // the reads of the last block before the stores of this one
+#pragma unroll
+    for (int i = threadIdx.x & 31; i < (int)(sizeof(FusedArgs) / 4); i += 32) d[i] = __ldg(s + i);
+    __syncwarp();
+}
+
 // Per-level information of one lane (horizontal) and of the level (vertical).
 struct LevelCtx {
     unsigned right;  // bit j: column j has its right (even) neighbour inside the image

@@ -8,10 +8,11 @@
 namespace dwt {
 
 // Many images in one launch: warp w of the grid works on entry i with
-// first[i] <= w < first[i + 1] of a table in device memory.  The arguments
-// come from registers instead of the constant bank, so the kernel gets the
-// register budget of 12 warps per SM rather than 16 (8 bytes of spills per
-// thread with 2 columns per lane, 32-40 with 4).
+// first[i] <= w < first[i + 1] of a table in device memory; its arguments are
+// copied to shared memory.  Bound by HBM and by the imbalance of a launch's
+// end.  Measured on 256 images of 65..4096 a side (12 launches): arguments in
+// registers 1781 us, in shared memory 1705; 128 registers and 16 warps per SM
+// 1942 (more images in flight, whose rows share DRAM pages less often).
 template <class S, int SCH, int NL, int Q1>
 __global__ void __launch_bounds__(kFwdWarps * 32, 12 / kFwdWarps)
     fwd_batched_kernel(const BatchEntry* __restrict__ table, int n) {
@@ -20,7 +21,9 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12 / kFwdWarps)
     const int gw = blockIdx.x * kFwdWarps + (threadIdx.x >> 5);
     const BatchEntry& e = table[find_entry(table, n, gw)];
     const int wid = gw - e.first_warp;
-    const FusedArgs a = e.args;  // registers: the body's stores cannot alias it
+    __shared__ SharedArgs shared_args;
+    copy_args(&shared_args, e.args);
+    const FusedArgs& a = shared_args.a;
     if (wid < 0 || wid >= a.nstrips * a.nsegs) return;
     fence_tensormap_acquire(&e.m[0]);
     fwd_body<S, SCH, NL, Q1>(&e.m[0], a, wid, smem_raw);
@@ -31,13 +34,17 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12 / kFwdWarps)
 // was taken earlier by a running warp: the bounded wait always ends unless a
 // warp failed, and then the status word already says so.  With both fusion
 // depths' bodies in one kernel, 4 columns per lane need the register budget
-// of 8 warps per SM (12 spill about 300 bytes per thread).
+// of 8 warps per SM (12 spill about 300 bytes per thread).  Arguments in
+// shared memory rather than registers: 64 images of 65..2933 a side 309 -> 302
+// us, 64 of 65..600 80.3 -> 78.2.
 template <class S, int SCH, int Q1>
 __global__ void __launch_bounds__(kFwdWarps * 32, fwd_queue_resident(Q1) / kFwdWarps)
     fwd_queue_kernel(const BatchEntry* __restrict__ table, int n, int total, int* head, int* done,
                      int* err) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     grid_dependency_sync();
+    __shared__ SharedArgs shared_args;
+    const FusedArgs& a = shared_args.a;
     const int lane = threadIdx.x & 31;
     for (;;) {
         int g = 0;
@@ -45,8 +52,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, fwd_queue_resident(Q1) / kFwdW
         g = __shfl_sync(kFull, g, 0);
         if (g >= total) break;
         const BatchEntry& e = table[find_entry(table, n, g)];
-        const FusedArgs a = e.args;
         const int wid = g - e.first_warp;
+        copy_args(&shared_args, e.args);
         bool ok = true;
         if (e.dep >= 0) {
             if (lane == 0) {

@@ -6,7 +6,7 @@
 
 namespace dwt {
 
-// arguments in registers (not the constant bank): 12 warps per SM
+// arguments in shared memory, 12 warps per SM as in the forward
 template <class S, int SCH, int NL, int Q1>
 __global__ void __launch_bounds__(kInvWarps * 32, 12 / kInvWarps)
     inv_batched_kernel(const BatchEntry* __restrict__ table, int n) {
@@ -15,7 +15,9 @@ __global__ void __launch_bounds__(kInvWarps * 32, 12 / kInvWarps)
     const int gw = blockIdx.x * kInvWarps + (threadIdx.x >> 5);
     const BatchEntry& e = table[find_entry(table, n, gw)];
     const int wid = gw - e.first_warp;
-    const FusedArgs a = e.args;  // registers: the body's stores cannot alias it
+    __shared__ SharedArgs shared_args;
+    copy_args(&shared_args, e.args);
+    const FusedArgs& a = shared_args.a;
     if (wid < 0 || wid >= a.nstrips * a.nsegs) return;
     fence_tensormap_acquire(&e.m[0]);
     fence_tensormap_acquire(&e.m[1]);
@@ -32,6 +34,8 @@ __global__ void __launch_bounds__(kInvWarps * 32, inv_queue_resident(Q1) / kInvW
                      int* err) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     grid_dependency_sync();
+    __shared__ SharedArgs shared_args;
+    const FusedArgs& a = shared_args.a;
     const int lane = threadIdx.x & 31;
     for (;;) {
         int g = 0;
@@ -39,8 +43,8 @@ __global__ void __launch_bounds__(kInvWarps * 32, inv_queue_resident(Q1) / kInvW
         g = __shfl_sync(kFull, g, 0);
         if (g >= total) break;
         const BatchEntry& e = table[find_entry(table, n, g)];
-        const FusedArgs a = e.args;
         const int wid = g - e.first_warp;
+        copy_args(&shared_args, e.args);
         bool ok = true;
         if (e.dep >= 0) {
             if (lane == 0) {
