@@ -127,7 +127,9 @@ dwt2d_status dwt2d_plan(dwt2d_plan_t* out, int32_t height, int32_t width, int32_
 typedef struct {
     int32_t fuse_first;            /* levels fused in the first launch, 1-3 (default 2) */
     int32_t fuse_max;              /* at most per later launch, 1-3 (default 2; 3 runs 4 quadruple
-                                      columns per lane; 16-bit storage caps both at 2) */
+                                      columns per lane; 16-bit storage caps both at 2).  With both
+                                      at 0 a forward float32 level of 512 x 512 to 4 million pixels
+                                      (the first: 7 million) has a launch of its own */
     int32_t fwd_warps_per_sm;      /* warps a forward launch is cut into, per SM (default 16) */
     int32_t inv_warps_per_sm;      /* the same for the inverse (default 16 for 16-bit
                                       storage, else 12) */
@@ -246,7 +248,8 @@ dwt2d_status dwt2d_workspace_status(void* d_workspace, void* stream);
 
 /*
  * dwt2d_plan_info -- kernel launches one forward call makes (for launch
- *   accounting), and the number of levels fused per launch, in launch order.
+ *   accounting; an inverse call may make fewer, see dwt2d_plan_launch_info),
+ *   and the number of levels fused per launch, in launch order.
  *   fused: array of at least 16 entries (may be NULL).
  */
 dwt2d_status dwt2d_plan_info(dwt2d_plan_t plan, int32_t* launches_per_call, int32_t* fused,

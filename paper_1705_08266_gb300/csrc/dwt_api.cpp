@@ -38,6 +38,12 @@ struct GroupLaunch {
 // SM of a large and of a small launch, and the segment rows in between.
 constexpr int kBatchWarpsLarge = 144, kBatchWarpsSmall = 12, kBatchSegRows = 16;
 
+// Forward levels of at most this many pixels (and more than 512 x 512) are not
+// fused in float32 (see plan_create): an image's first level (2048^2 25.0 ->
+// 22.8 us, 2000 x 3000 19.4 -> 17.7, 2500 x 3000 no gain), and one whose input
+// a launch before it has left in L2 (5 levels of 2500 x 5000 35.2 -> 33.2).
+constexpr long long kSingleFirst = 7000000, kSinglePixels = 4000000;
+
 constexpr int kMaxHostBands = 64;  // row bands of the pipelined host-buffer entry points
 
 struct dwt2d_plan_s {
@@ -47,8 +53,9 @@ struct dwt2d_plan_s {
     dwt2d_dtype dtype;
     int elem;         // bytes per element
     int hs[17], ws[17];  // extent transformed by level l (l = 0 .. levels-1)
-    Group groups[16];
-    int ngroups;
+    // level groups, finest first, of the inverse [0] and the forward [1]
+    Group groups[2][16];
+    int ngroups[2];
     int sm_count;
     long long l2_bytes;  // L2 cache of the device the plan was made on
     int fwd_warps_target, inv_warps_target;
@@ -75,7 +82,7 @@ struct dwt2d_plan_s {
     size_t size_a, size_b;  // bytes of the two LL buffers
     long long pitch_a, pitch_b, pitch_x;  // elements
     size_t ws_bytes;
-    // the launches of a forward call (k < ngroups), then those of an inverse
+    // the launches of a forward call (k < ngroups[1]), then those of an inverse
     // call, without buffers: their shapes depend on the plan alone, and
     // deriving them on every call took about as long as a kernel launch (null
     // for the plans of a batch, which shapes its own launches)
@@ -360,7 +367,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
     const int rho = p->wavelet == DWT2D_CDF97 ? 2 : 1;
     FusedArgs& a = out->a;
     memset(&a, 0, sizeof(a));
-    const Group g = p->groups[fwd ? k : p->ngroups - 1 - k];
+    const Group g = p->groups[fwd][fwd ? k : p->ngroups[0] - 1 - k];
     for (int i = 0; i < g.n; ++i) {
         a.lv[i].h = p->hs[g.first + i];
         a.lv[i].w = p->ws[g.first + i];
@@ -373,7 +380,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         // takes at most a third of it: 2-4 % faster at 8192^2 float32 and
         // 16384^2 16-bit, slower once it crowds out the launch's own stream
         const long long ll_bytes = (long long)((hN + 1) / 2) * ((a.lv[g.n - 1].w + 1) / 2) * p->elem;
-        a.ll_keep = k != p->ngroups - 1 && 3 * ll_bytes <= p->l2_bytes;
+        a.ll_keep = k != p->ngroups[1] - 1 && 3 * ll_bytes <= p->l2_bytes;
         const int rows = (hN + 1) / 2;
         // quadruple columns per lane: 4 for three fused levels; with
         // fwd_q1 == 0 (automatic), 4 for a float32 launch whose rows still give
@@ -458,7 +465,7 @@ dwt2d_status bind_group(const dwt2d_plan_s* p, bool fwd, int k, const void* src,
     const long long belems[2] = {(long long)(p->size_a / p->elem), (long long)(p->size_b / p->elem)};
     FusedArgs& a = out->a;
     a.err = err;
-    const bool last = k == p->ngroups - 1;
+    const bool last = k == p->ngroups[fwd] - 1;
     // input: the image (coefficients), else the LL the previous launch wrote
     const void* in = k == 0 ? src : bufs[(k - 1) & 1];
     const long long in_pitch = k == 0 ? src_pe : bpitch[(k - 1) & 1];
@@ -510,9 +517,9 @@ dwt2d_status run_fused(const dwt2d_plan_s* p, bool fwd, const void* src, int64_t
     const int sch = base_scheme(p->scheme);
     char* wsb = reinterpret_cast<char*>(ws);
     int* err = reinterpret_cast<int*>(wsb);
-    for (int k = 0; k < p->ngroups; ++k) {
+    for (int k = 0; k < p->ngroups[fwd]; ++k) {
         GroupLaunch gl;
-        if (p->shapes) gl = p->shapes[fwd ? k : p->ngroups + k];
+        if (p->shapes) gl = p->shapes[fwd ? k : p->ngroups[1] + k];
         else shape_group(p, fwd, k, p->fwd_warps_target, p->inv_warps_target, &gl);
         const dwt2d_status s =
             bind_group(p, fwd, k, src, sp / p->elem, dst, dp / p->elem, wsb, err, &gl);
@@ -797,15 +804,28 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
                                                  : opt(o.fuse_first, maxf < 2 ? maxf : 2);
     if (first < 1) first = 1;
     if (first > maxf) first = maxf;
-    p->ngroups = 0;
-    for (int l = 0; l < levels;) {
-        const int cap = p->ngroups == 0 ? first : maxf;
-        const int n = levels - l < cap ? levels - l : cap;
-        p->groups[p->ngroups].first = l;
-        p->groups[p->ngroups].n = n;
-        ++p->ngroups;
-        l += n;
-    }
+    // A small float32 level takes a launch of its own in the forward: two fused
+    // levels stream 12 halo rows per segment, one 4, and where a launch is one
+    // short wave of warps that is its time (5 levels of 1080 x 1920 21.7 us
+    // with 2 + 2 + 1, 19.4 with 1 + 1 + 2 + 1).  Not below 512 x 512, where the
+    // launches themselves are (15.1 and 15.0 us), nor for 5/3 (8 halo rows: 1080
+    // x 1920 14.5 and 14.9 us) or the inverse (18.5 and 19.6), nor for 16-bit
+    // storage, whose LL between launches is rounded.
+    const bool regroup = !tuning && wavelet == DWT2D_CDF97 && dtype == DWT2D_F32 && o.fuse_first == 0 &&
+                         o.fuse_max == 0 && !multipass(scheme) && !convolution(scheme);
+    auto make_groups = [&](int dir, bool single) {
+        p->ngroups[dir] = 0;
+        for (int l = 0; l < levels;) {
+            const long long px = (long long)p->hs[l] * p->ws[l];
+            int cap = p->ngroups[dir] == 0 ? first : maxf;
+            if (single && px > 512 * 512 && px <= (l == 0 ? kSingleFirst : kSinglePixels)) cap = 1;
+            const int n = levels - l < cap ? levels - l : cap;
+            p->groups[dir][p->ngroups[dir]++] = {l, n};
+            l += n;
+        }
+    };
+    make_groups(0, false);
+    make_groups(1, regroup);
     const int sms = dev.sms;
     p->sm_count = sms;
     p->l2_bytes = dev.l2_bytes;
@@ -879,27 +899,34 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
             ba = bb = (size_t)pa * lh * p->elem;
         }
     } else {
-        for (int gi = 0; gi + 1 < p->ngroups; ++gi) {
-            const Group g = p->groups[gi];
-            const int last = g.first + g.n - 1;
-            const int lh = (p->hs[last] + 1) / 2, lw = (p->ws[last] + 1) / 2;
-            const long long pp = round_pitch(lw, p->elem);
-            const size_t b = (size_t)pp * lh * p->elem;
-            // forward writes group gi's LL to buffer gi & 1; the inverse uses the
-            // same buffers for the LL it produces, which have the same sizes
-            if ((gi & 1) == 0) { if (b > ba) { ba = b; pa = pp; } }
-            else { if (b > bb) { bb = b; pb = pp; } }
-        }
-        // inverse order: launch k writes buffer k & 1; launch k produces the LL
-        // that group (ngroups - 2 - k) produced in the forward direction
-        for (int k = 0; k + 1 < p->ngroups; ++k) {
-            const Group g = p->groups[p->ngroups - 2 - k];
-            const int last = g.first + g.n - 1;
-            const int lh = (p->hs[last] + 1) / 2, lw = (p->ws[last] + 1) / 2;
-            const long long pp = round_pitch(lw, p->elem);
-            const size_t b = (size_t)pp * lh * p->elem;
-            if ((k & 1) == 0) { if (b > ba) { ba = b; pa = pp; } }
-            else { if (b > bb) { bb = b; pb = pp; } }
+        // forward launch gi writes the LL of its group to buffer gi & 1; inverse
+        // launch k (coarse to fine) writes buffer k & 1 with the LL above group
+        // ngroups - 2 - k
+        auto size_buffers = [&] {
+            ba = bb = 0;
+            pa = pb = 1;
+            for (int dir = 0; dir < 2; ++dir) {
+                for (int gi = 0; gi + 1 < p->ngroups[dir]; ++gi) {
+                    const Group g = p->groups[dir][gi];
+                    const int last = g.first + g.n - 1;
+                    const int lh = (p->hs[last] + 1) / 2, lw = (p->ws[last] + 1) / 2;
+                    const long long pp = round_pitch(lw, p->elem);
+                    const size_t b = (size_t)pp * lh * p->elem;
+                    const int k = dir == 1 ? gi : p->ngroups[0] - 2 - gi;
+                    if ((k & 1) == 0) { if (b > ba) { ba = b; pa = pp; } }
+                    else { if (b > bb) { bb = b; pb = pp; } }
+                }
+            }
+            return kHeader + (ba + 255) / 256 * 256 + (bb + 255) / 256 * 256;
+        };
+        // a workspace that fits the allocation-free entry point with the usual
+        // groups stays that small
+        if (size_buffers() > DWT2D_NOALLOC_SCRATCH_BYTES && regroup) {
+            make_groups(1, false);
+            if (size_buffers() > DWT2D_NOALLOC_SCRATCH_BYTES) {
+                make_groups(1, true);
+                size_buffers();
+            }
         }
     }
     p->off_a = take(ba);
@@ -917,9 +944,10 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     }
     p->ws_bytes = off;
     if (!tuning && !multipass(scheme)) {
-        p->shapes = new (std::nothrow) GroupLaunch[2 * p->ngroups]();
-        for (int k = 0; p->shapes && k < 2 * p->ngroups; ++k)
-            shape_group(p, k < p->ngroups, k % p->ngroups, p->fwd_warps_target, p->inv_warps_target,
+        const int nf = p->ngroups[1], n = nf + p->ngroups[0];
+        p->shapes = new (std::nothrow) GroupLaunch[n]();
+        for (int k = 0; p->shapes && k < n; ++k)
+            shape_group(p, k < nf, k < nf ? k : k - nf, p->fwd_warps_target, p->inv_warps_target,
                         &p->shapes[k]);
     }
     *workspace_bytes = off;
@@ -1088,7 +1116,7 @@ static dwt2d_status run_host_fwd_pipelined(dwt2d_plan_s* p, const void* h_src, i
     }
     // every band has arrived before the call returns (the input buffer is free)
     if (cudaStreamWaitEvent(st, ev_in(B - 1), 0) != cudaSuccess) return DWT2D_ERR_CUDA;
-    for (int k = 1; k < p->ngroups; ++k) {
+    for (int k = 1; k < p->ngroups[1]; ++k) {
         GroupLaunch gl;
         s = build_group(p, true, k, d_in, dpitch / es, d_out, dpitch / es, wsb, err, p->fwd_warps_target,
                         p->inv_warps_target, &gl);
@@ -1140,7 +1168,7 @@ static dwt2d_status run_host_inv_pipelined(dwt2d_plan_s* p, const void* h_src, i
     if (cudaEventRecord(ev[0], st) != cudaSuccess || cudaStreamWaitEvent(p->host_in, ev[0], 0) ||
         cudaStreamWaitEvent(p->host_out, ev[0], 0))
         return DWT2D_ERR_CUDA;
-    const int n0 = p->groups[0].n;  // levels of the finest group
+    const int n0 = p->groups[0][0].n;  // levels of the finest group
     const int hN = p->hs[n0 - 1], wN = p->ws[n0 - 1];
     // the coarse region: levels > n0 and the last LL
     if (in_rows(0, (hN + 1) / 2, 0, (wN + 1) / 2) != cudaSuccess) return DWT2D_ERR_CUDA;
@@ -1163,7 +1191,7 @@ static dwt2d_status run_host_inv_pipelined(dwt2d_plan_s* p, const void* h_src, i
     }
     const int elem_kind = elem_kind_of(p->dtype);
     const int sch = base_scheme(p->scheme);
-    const int G = p->ngroups;
+    const int G = p->ngroups[0];
     // coarse groups: their input (the coarse region) went in first
     if (G > 1 && cudaStreamWaitEvent(st, ev_in(0), 0) != cudaSuccess) return DWT2D_ERR_CUDA;
     for (int k = 0; k + 1 < G; ++k) {
@@ -1237,10 +1265,10 @@ static dwt2d_status run_host(dwt2d_plan_t p, bool fwd, const void* h_src, int64_
     cudaStream_t st = as_stream(stream);
     if (fwd && p->H >= 1024 && !multipass(p->scheme) && !convolution(p->scheme) &&
         p->host_pipeline && check_buffers(p, d_in, dpitch, d_out, dpitch, d_ws) == DWT2D_OK &&
-        p->groups[0].n <= 2 && scale_ok(p, scale) && host_resources(p))
+        p->groups[1][0].n <= 2 && scale_ok(p, scale) && host_resources(p))
         return run_host_fwd_pipelined(p, h_src, hsp, h_dst, hdp, d_in, d_out, dpitch, d_ws, st);
     if (!fwd && p->H >= 1024 && !multipass(p->scheme) && p->host_pipeline &&
-        check_buffers(p, d_in, dpitch, d_out, dpitch, d_ws) == DWT2D_OK && p->groups[0].n <= 2 &&
+        check_buffers(p, d_in, dpitch, d_out, dpitch, d_ws) == DWT2D_OK && p->groups[0][0].n <= 2 &&
         scale_ok(p, scale) && host_resources(p))
         return run_host_inv_pipelined(p, h_src, hsp, h_dst, hdp, d_in, d_out, dpitch, d_ws, st);
     // one linear copy when both sides are unpadded (faster than a 2-D copy)
@@ -1311,10 +1339,10 @@ dwt2d_status dwt2d_plan_info(dwt2d_plan_t p, int32_t* launches, int32_t* fused, 
             for (int l = 0; l < p->levels; ++l) fused[l] = 1;
         return DWT2D_OK;
     }
-    if (launches) *launches = p->ngroups;
-    if (n_groups) *n_groups = p->ngroups;
+    if (launches) *launches = p->ngroups[1];
+    if (n_groups) *n_groups = p->ngroups[1];
     if (fused)
-        for (int g = 0; g < p->ngroups; ++g) fused[g] = p->groups[g].n;
+        for (int g = 0; g < p->ngroups[1]; ++g) fused[g] = p->groups[1][g].n;
     return DWT2D_OK;
 }
 
@@ -1322,7 +1350,7 @@ dwt2d_status dwt2d_plan_launch_info(dwt2d_plan_t p, int32_t inverse, int32_t i, 
                                      int32_t* cols_per_lane, int32_t* warps) {
     if (!p || i < 0 || (inverse != 0 && inverse != 1)) return DWT2D_ERR_INVALID;
     if (multipass(p->scheme) || (convolution(p->scheme) && !inverse)) return DWT2D_ERR_UNSUPPORTED;
-    if (i >= p->ngroups) return DWT2D_ERR_INVALID;
+    if (i >= p->ngroups[!inverse]) return DWT2D_ERR_INVALID;
     GroupLaunch gl;
     shape_group(p, !inverse, i, p->fwd_warps_target, p->inv_warps_target, &gl);
     if (fused) *fused = gl.nl;
@@ -1404,7 +1432,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
     // cover its images with fewer pixels than 128-pixel ones.
     const int sms = dev.sms;
     int max_groups = 0;
-    for (auto* p : b->plans) max_groups = std::max(max_groups, p->ngroups);
+    for (auto* p : b->plans) max_groups = std::max(max_groups, p->ngroups[0]);
     b->warps = 0;
     for (int k = 0; k < max_groups; ++k) {
         for (int fwd = 1; fwd >= 0; --fwd) {
@@ -1425,10 +1453,10 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                     for (int i = 0; i < n; ++i) {
                         const dwt2d_plan_s* p = b->plans[i];
                         if ((items[i].inverse == 0) != (fwd == 1) || elem_kind_of(p->dtype) != ek ||
-                            k >= p->ngroups)
+                            k >= p->ngroups[fwd])
                             continue;
-                        const int gi = fwd ? k : p->ngroups - 1 - k;
-                        const Group g = p->groups[gi];
+                        const int gi = fwd ? k : p->ngroups[0] - 1 - k;
+                        const Group g = p->groups[fwd][gi];
                         if (g.n != nl) continue;
                         Cand c;
                         c.i = i;

@@ -176,16 +176,18 @@ def as_pitched(t: torch.Tensor) -> torch.Tensor:
 
 
 def workspace_bytes(height: int, width: int, levels: int, wavelet: str = "cdf97",
-                    scheme: str = "nonsep_reduced", dtype: Optional[torch.dtype] = None) -> int:
-    """Device workspace a default plan of this transform needs (dwt2d_plan,
-    then dwt2d_plan_destroy; no Python plan object)."""
+                    scheme: str = "nonsep_reduced", dtype: Optional[torch.dtype] = None,
+                    options: Optional[dict] = None) -> int:
+    """Device workspace a plan of this transform needs (dwt2d_plan_ex, then
+    dwt2d_plan_destroy; no Python plan object)."""
     L = lib()
     if dtype is None:
         dtype = torch.int32 if wavelet == "legall53" else torch.float32
     h = ctypes.c_void_p()
     ws = ctypes.c_size_t()
-    _check(L.dwt2d_plan(ctypes.byref(h), height, width, levels, WAVELETS[wavelet], SCHEMES[scheme], 0,
-                        DTYPES[dtype], ctypes.byref(ws)), "dwt2d_plan")
+    opts = ctypes.byref(plan_options(**options)) if options else None
+    _check(L.dwt2d_plan_ex(ctypes.byref(h), height, width, levels, WAVELETS[wavelet], SCHEMES[scheme], 0,
+                           DTYPES[dtype], opts, ctypes.byref(ws)), "dwt2d_plan_ex")
     L.dwt2d_plan_destroy(h)
     return ws.value
 
@@ -225,13 +227,18 @@ class Plan:
 
     def launch_info(self, inverse: bool = False):
         """[(levels fused, columns per lane, warps)] of each launch of a call, in launch order."""
+        # the directions may group the levels differently
         out = []
-        n = self.info()[0]
-        for i in range(n):
+        i = 0
+        while True:
             f, q, w = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
-            _check(lib().dwt2d_plan_launch_info(self._h, int(inverse), i, ctypes.byref(f), ctypes.byref(q),
-                                                ctypes.byref(w)), "plan_launch_info")
+            st = lib().dwt2d_plan_launch_info(self._h, int(inverse), i, ctypes.byref(f), ctypes.byref(q),
+                                              ctypes.byref(w))
+            if st == -1 and i > 0:  # past the last launch
+                break
+            _check(st, "plan_launch_info")
             out.append((f.value, q.value, w.value))
+            i += 1
         return out
 
     def set_launch_events(self, events):

@@ -147,8 +147,10 @@ class GpuExecutor:
         key = (req.height, req.width, req.levels, req.wavelet, req.dtype)
         n = self._ws_cache.get(key)
         if n is None:
+            # the groups a batch runs (a plan of one image may group its levels
+            # into more launches, with larger LLs between them)
             n = self.D.workspace_bytes(req.height, req.width, req.levels, req.wavelet, self.scheme,
-                                       req.dtype)
+                                       req.dtype, {"fuse_first": 2, "fuse_max": 2})
             if len(self._ws_cache) > 65536:
                 self._ws_cache.clear()
             self._ws_cache[key] = n

@@ -117,3 +117,25 @@ def test_middle_sizes_equal_one_wave(h, w, levels, dtype):
         assert plan.status(ws) == 0
         outs.append((c, y))
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("h,w,levels", [(513, 512, 3), (1080, 1920, 5), (1601, 2499, 4), (2048, 2049, 6),
+                                        (2700, 5001, 5)])
+@pytest.mark.parametrize("scheme", ["nonsep_reduced", "separable"])
+def test_single_level_launches_equal_fused_ones(h, w, levels, scheme):
+    """Small float32 levels have forward launches of their own: the same bits
+    as fused pairs, and an inverse that takes its own groups."""
+    x = D.empty_image(h, w)
+    x.copy_(torch.rand(h, w, device="cuda") * 255)
+    outs = []
+    for options in (None, dict(fuse_first=2, fuse_max=2)):
+        plan = D.Plan(h, w, levels, "cdf97", scheme, options=options)
+        ws = plan.workspace()
+        c = plan.forward(x, workspace=ws)
+        y = plan.inverse(c, workspace=ws)
+        torch.cuda.synchronize()
+        assert plan.status(ws) == 0
+        fwd, inv = plan.launch_info(), plan.launch_info(inverse=True)
+        assert sum(f for f, _q, _w in fwd) == levels and sum(f for f, _q, _w in inv) == levels
+        outs.append((c, y))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
