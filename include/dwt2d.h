@@ -135,16 +135,17 @@ typedef struct {
                                       storage, else 12) */
     int32_t fwd_warps_per_sm_large;/* forward launches whose row segments stay at least
                                       large_segment rows long at this many warps per SM take it
-                                      (default 48 for float32, 32 for 16-bit storage, 64 for
-                                      LeGall 5/3 at 2 columns per lane, 32 at 4; by default also
-                                      16, 32, ... fewer where only that gives such segments;
-                                      -1: never) */
+                                      (default 36 for float32, 32 for 16-bit storage, 64 for
+                                      LeGall 5/3 at 2 columns per lane, 36 and 32 at 4; by default
+                                      also a wave or more fewer where only that gives such
+                                      segments; -1: never) */
     int32_t inv_warps_per_sm_large;/* the same for the inverse (default 80 for float32, 48 for
                                       16-bit storage, 96 for LeGall 5/3 at 2 columns per lane,
                                       24 at 4; -1: never) */
     int32_t large_segment;         /* that threshold, quadruple rows of the launch's last level
-                                      (default: forward 13, for one level 20, for 4 columns per
-                                      lane 16; inverse 20; 16-bit storage 40) */
+                                      (default: forward 13 for 5/3, 17 for float32, 20 for one
+                                      level, 16 to 19 for 4 columns per lane; inverse 20; 16-bit
+                                      storage 40) */
     int32_t min_segment;           /* shortest row segment of a warp (default 2) */
     int32_t fwd_seg_interleave;    /* forward segment order: taken in this many interleaved groups
                                       (default: the launch's waves of resident warps; 1: top to

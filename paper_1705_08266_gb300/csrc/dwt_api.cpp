@@ -66,6 +66,7 @@ struct dwt2d_plan_s {
     int fwd_warps_large, fwd_large_segq, fwd_large_segq1 /* one level */, fwd_large_step;
     int inv_warps_large, inv_large_segq, inv_large_step;  // the same rule for inverse launches
     int large_segq4;  // rows for 4 columns per lane without being asked
+    int fwd_warps_huge4, huge_segq4;  // the same for the largest launches, 12 warps per SM resident
     int fwd_q1;  // quadruple columns per lane of the forward kernel (2 or 4; 0: automatic)
     int fwd_warps_large4, fwd_short4;  // the large-launch rule at 4 columns per lane
     int inv_warps_large4;
@@ -267,6 +268,19 @@ dwt2d_status check_buffers(const dwt2d_plan_s* p, const void* src, int64_t sp, c
 }
 
 // Warps of a streaming kernel resident per SM (their register budgets).
+// A large float32 forward launch keeps 12 warps per SM in flight instead of the
+// 16 its registers allow: it is bound by HBM, and fewer rows in flight share
+// DRAM pages better.  Each warp asks for more shared memory than its ring
+// takes, so that 12 fit the 228 KB of an SM (1 KB of it per CTA reserved).
+// Two levels, us, 16 / 12 warps: 2 columns per lane 6000^2 57.3 / 54.4, 3000 x
+// 20000 89.8 / 86.5; 4 columns 6000 x 20000 169 / 163.6, 16384^2 367 / 354 (2
+// columns of 8192^2: 98.2 / 94.1, 10 warps 95.9, 8 warps 97.6).  A launch of one
+// wave keeps 16 (4096^2 28.1 and 28.5), and so do the inverse (88.6 and 90.3),
+// 5/3 (86.9 and 86.6) and 16-bit storage, which is bound by its arithmetic (78
+// and 80).
+constexpr int kFwdLargeResident = 12;
+constexpr int kFwdLargeSmem = 17920;
+
 int resident_per_sm(bool fwd, int nl, int q1, int scheme) {
     if (fwd) return nl >= 3 ? 8 : (q1 >= 4 && scheme == SCH_NONSEP ? 12 : 16);
     return q1 <= 2 ? (scheme == SCH_NONSEP ? 12 : 16) : 12;
@@ -391,11 +405,16 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         int grid4 = 0;
         bool use4 = false;
         if (g.n <= 2 && p->fwd_q1 == 0 && segq_fixed <= 0 && elem_kind == 0 && p->fwd_warps_large4 > 0) {
-            big4 = a;
-            decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, p->fwd_warps_large4, &big4, &grid4, kFwdWarps, 0,
-                      resident_per_sm(true, g.n, 4, sch), uniform_segments ? 0 : p->fwd_short4,
-                      p->fwd_seg_f);
-            use4 = big4.segq >= p->large_segq4;
+            const struct { int warps, resident, segq, smem; } tries[2] = {
+                {p->fwd_warps_huge4, kFwdLargeResident, p->huge_segq4, kFwdLargeSmem},
+                {p->fwd_warps_large4, resident_per_sm(true, g.n, 4, sch), p->large_segq4, 0}};
+            for (int i = p->fwd_warps_huge4 > 0 ? 0 : 1; i < 2 && !use4; ++i) {
+                big4 = a;
+                decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, tries[i].warps, &big4, &grid4, kFwdWarps, 0,
+                          tries[i].resident, uniform_segments ? 0 : p->fwd_short4, p->fwd_seg_f);
+                big4.min_smem = tries[i].smem;
+                use4 = big4.segq >= tries[i].segq;
+            }
             if (use4) q1 = 4;
         }
         if (use4) {
@@ -403,6 +422,8 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             out->grid = grid4;
         } else {
             const int res = resident_per_sm(true, g.n, q1, sch);
+            const bool fewer = elem_kind == 0 && q1 == 2;  // kFwdLargeResident warps per SM
+            const int segq_min = q1 == 4 ? p->large_segq4 : (g.n == 1 ? p->fwd_large_segq1 : p->fwd_large_segq);
             const int large = q1 == 4 ? p->fwd_warps_large4 : p->fwd_warps_large;
             const int sd = uniform_segments ? 0 : (q1 == 4 ? p->fwd_short4 : p->fwd_short);
             decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, fwd_target, &a, &out->grid, kFwdWarps,
@@ -410,10 +431,11 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             for (int t = large; segq_fixed <= 0 && t > fwd_target; t -= p->fwd_large_step) {
                 FusedArgs b = a;
                 int grid_b = 0;
-                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kFwdWarps, 0, res, sd,
-                          p->fwd_seg_f);
-                if (b.segq >= (g.n == 1 ? p->fwd_large_segq1 : p->fwd_large_segq)) {
+                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kFwdWarps, 0,
+                          fewer ? kFwdLargeResident : res, sd, p->fwd_seg_f);
+                if (b.segq >= segq_min) {
                     a = b;
+                    if (fewer) a.min_smem = kFwdLargeSmem;
                     out->grid = grid_b;
                     break;
                 }
@@ -836,17 +858,20 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
     p->fill = o.min_segment == 0;
     // Warps per SM of a large launch (segments of at least *_large_segq rows), in
-    // waves of the resident warps (16 at 128 registers).  More warps: shorter
-    // last segments and a more compact set of rows in flight, but more halo
-    // rows.  Measured two-level launches, us (8192^2): forward float32, 4
-    // columns per lane 24 warps 105, 32 101.6, 48 112; 16-bit, 2 columns per
+    // waves of the resident warps (12 for float32 forward, else 16).  More warps:
+    // shorter last segments and a more compact set of rows in flight, but more
+    // halo rows.  Measured two-level launches, us (8192^2): forward float32, 2
+    // columns per lane 24 warps 96.7, 36 94.1, 48 94.6 (6000^2: 54.4, 56.8), 4
+    // columns 32 101.6, 48 112 (16384^2, 12 resident: 36 352.8); 16-bit, 2 columns per
     // lane 16 78.0, 32 78.6, 48 82.4 (16384^2: 282, 260, 259); 5/3 48 87.0, 64
     // 87.1, 80 99.9.  Inverse float32 48 90.5, 64 90.1, 80 88.4, 96 89.9; 16-bit
     // 32 80.6, 48 81.0 (16384^2: 281, 276); 5/3 64 85.4, 80 83.4, 96 82.5.
-    const int fwl = opt(o.fwd_warps_per_sm_large, half ? 32 : (wavelet == DWT2D_CDF97 ? 48 : 64));
+    const bool f32 = dtype == DWT2D_F32;
+    const int fwl = opt(o.fwd_warps_per_sm_large, half ? 32 : (f32 ? 36 : 64));
     p->fwd_warps_large = (tuning && tuning->warps_per_sm > 0) || fwl < 0 ? 0 : sms * fwl;
     const int fwl4 = opt(o.fwd_warps_per_sm_large, 32);
     p->fwd_warps_large4 = (tuning && tuning->warps_per_sm > 0) || fwl4 < 0 ? 0 : sms * fwl4;
+    p->fwd_warps_huge4 = (tuning && tuning->warps_per_sm > 0) || o.fwd_warps_per_sm_large != 0 ? 0 : sms * 36;
     // A launch whose segments would be shorter than this many rows (level-2
     // rows forward, level-1 rows inverse) takes a wave less, and so on down to
     // the count of the small launches: where the halo rows cost more than a
@@ -858,12 +883,17 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     // 36.7, 32 warps (14 rows) 42.5; inverse 6000^2 47.7 and 49.2 (33 rows).
     // Small 16-bit inverses: 16 warps for 12, 1500 x 3000 13.9 -> 12.0, 6 levels
     // of 4099 x 2051 36.2 -> 31.8.
-    p->fwd_large_segq = opt(o.large_segment, half ? 40 : 13);
+    p->fwd_large_segq = opt(o.large_segment, half ? 40 : (f32 ? 17 : 13));
     p->fwd_large_segq1 = opt(o.large_segment, half ? 40 : 20);
     p->inv_large_segq = opt(o.large_segment, half ? 40 : 20);
+    // 4 columns per lane: without being asked from 8192^2 on (one level of
+    // 16384^2 342 us, with 2 columns 355); the largest of them, whose segments
+    // stay longer, with 12 warps per SM (two levels of 16384^2 376 -> 359, three
+    // of 9001 x 12000 165 -> 162; 5 of 8192^2 118.1 and 118.7)
     p->large_segq4 = opt(o.large_segment, 16);
+    p->huge_segq4 = opt(o.large_segment, 19);
     // counts that were asked for are taken or left as a whole
-    p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * 16 : 1 << 28;
+    p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * (f32 ? kFwdLargeResident : 16) : 1 << 28;
     p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * 16 : 1 << 28;
     const int iwl = opt(o.inv_warps_per_sm_large, half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;

@@ -3,6 +3,8 @@
 // quadruple columns per lane).
 #include "dwt_fwd_body.cuh"
 
+#include <algorithm>
+
 namespace dwt {
 
 template <class S, int SCH, int NL, int Q1>
@@ -26,7 +28,9 @@ template <class S, int SCH, int NL, int Q1>
 static cudaError_t launch_one(const CUtensorMap& map, const FusedArgs& a, int grid,
                               cudaStream_t st) {
     auto k = fwd_fused_kernel<S, SCH, NL, Q1>;
-    const size_t smem = fwd_smem_bytes(sizeof(S), NL, Q1);  // below the 48 KB that need an opt-in
+    // below the 48 KB that need an opt-in; more than the ring where the launch
+    // wants fewer resident warps
+    const size_t smem = std::max(fwd_smem_bytes(sizeof(S), NL, Q1), (size_t)a.min_smem);
     return launch_kernel(k, grid, kFwdWarps * 32, smem, st, a.pdl != 0, map, a);
 }
 

@@ -45,6 +45,7 @@ struct FusedArgs {
     int* err;                        // device status word (0 = ok)
     int pdl;                         // host: launch with programmatic stream serialization
     int ll_keep;                     // forward: store the LL with an L2 evict-last policy
+    int min_smem;                    // host: shared memory of a CTA at least (limits the resident warps)
 };
 
 

@@ -100,7 +100,8 @@ def test_default_batch_rows_equal_tuned_ones():
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.int32, torch.float16])
-@pytest.mark.parametrize("h,w,levels", [(2500, 5000, 2), (3001, 4097, 1), (6000, 1500, 3), (3000, 9000, 2)])
+@pytest.mark.parametrize("h,w,levels", [(2500, 5000, 2), (3001, 4097, 1), (6000, 1500, 3), (3000, 9000, 2),
+                                        (9999, 10001, 2)])
 def test_middle_sizes_equal_one_wave(h, w, levels, dtype):
     """Between the small launches and the large ones the wave count follows the
     segments' length: the default plan gives the bits of one-wave launches."""
