@@ -267,7 +267,6 @@ dwt2d_status check_buffers(const dwt2d_plan_s* p, const void* src, int64_t sp, c
     return DWT2D_OK;
 }
 
-// Warps of a streaming kernel resident per SM (their register budgets).
 // A large float32 forward launch keeps 12 warps per SM in flight instead of the
 // 16 its registers allow: it is bound by HBM, and fewer rows in flight share
 // DRAM pages better.  Each warp asks for more shared memory than its ring
@@ -281,6 +280,7 @@ dwt2d_status check_buffers(const dwt2d_plan_s* p, const void* src, int64_t sp, c
 constexpr int kFwdLargeResident = 12;
 constexpr int kFwdLargeSmem = 17920;
 
+// Warps of a streaming kernel resident per SM (their register budgets).
 int resident_per_sm(bool fwd, int nl, int q1, int scheme) {
     if (fwd) return nl >= 3 ? 8 : (q1 >= 4 && scheme == SCH_NONSEP ? 12 : 16);
     return q1 <= 2 ? (scheme == SCH_NONSEP ? 12 : 16) : 12;
