@@ -895,7 +895,10 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     // counts that were asked for are taken or left as a whole
     p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * (f32 ? kFwdLargeResident : 16) : 1 << 28;
     p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * 16 : 1 << 28;
-    const int iwl = opt(o.inv_warps_per_sm_large, half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96));
+    // The plain non-separable 9/7 inverse: 36 (8192^2 122.8, 48 123.7, 64 125.4).
+    const bool plain97 = wavelet == DWT2D_CDF97 && base_scheme(scheme) == SCH_NONSEP;
+    const int iwl = opt(o.inv_warps_per_sm_large,
+                        plain97 ? 36 : (half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96)));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;
     p->fwd_q1 = o.fwd_cols_per_lane;  // 0: automatic
     p->pdl = opt(o.programmatic_launch, 1) > 0;
