@@ -413,7 +413,11 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
             mbar_wait_bounded(bar_s + 8 * (t % kInvSlots), (t / kInvSlots) & 1, kWaitBudget);
         return false;
     }
-    // every copy has landed: the barriers may be initialised again
+    // every copy has landed: the barriers may be initialised again.  The last
+    // kInvSlots slots were not refilled, so no fence has ordered this lane's
+    // accesses to them (mirrored columns are stored there) before the copies
+    // that the warp's next work item issues into the same ring.
+    fence_proxy_async_smem();
     if (lane == 0)
         for (int b = 0; b < kInvSlots; ++b) mbar_inval(bar_s + 8 * b);
     __syncwarp();

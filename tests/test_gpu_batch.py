@@ -362,3 +362,27 @@ def test_c4_batch_full_workload(persistent, cols):
                 assert int(got[r, c]) == int(ref), (i, r, c)
             else:
                 assert abs(float(got[r, c]) - float(ref)) <= TOL_F32 * maxabs, (i, r, c)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.int32, torch.float16])
+def test_persistent_inverse_of_short_border_items(dtype):
+    """Work items of a few ring slots whose columns are all mirrored in the
+    ring: a warp reuses every slot of its ring for its next item without a
+    refill in between, many items in a row."""
+    wavelet = "legall53" if dtype == torch.int32 else "cdf97"
+    rng = np.random.default_rng(53)
+    spec = [(int(rng.integers(2, 25)), int(rng.integers(2, 120)), int(rng.integers(1, 5)), wavelet, dtype, 1)
+            for _ in range(64)]
+    # more items than resident warps: long columns of short segments
+    spec += [(4000 + i, 30 + i, 3, wavelet, dtype, 1) for i in range(8)]
+    jobs, _ = _jobs(spec, 530)
+    batch = D.Batch(jobs, tuning={"persistent": 1, "warps_per_sm": 60000, "min_segment": 2})
+    ws = batch.workspace()
+    batch.upload(ws)
+    for _ in range(3):
+        for _s, dst, _l, _w, _i in jobs:
+            dst.fill_(0)
+        batch.launch(ws)
+        torch.cuda.synchronize()
+        assert batch.status(ws) == 0
+        _assert_same_as_single(jobs, "nonsep_reduced", f"short items {dtype}")
