@@ -112,15 +112,34 @@ struct InvWarpT {
                 if (f[i] >= 0) p[i * REGION + off[i] + r * PITCH + (f[i] & 0xffff)] = v[i][r];
     }
 
+    // A level one column wide has no HL and HH (bands at p and p + 2 REGION):
+    // what their boxes hold there is another level's, and a non-finite value of
+    // it would come through the step's zero coefficient as a NaN.  (The integer
+    // steps select instead of multiplying.)
+    template <int ROWS, int PITCH, int REGION>
+    __device__ __forceinline__ void clear_odd(S* p, const LevelCtx& x) {
+        if constexpr (std::is_same<T, float>::value) {
+            if (x.ha) return;
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+                p[r * PITCH + lane] = p[2 * REGION + r * PITCH + lane] = Storage<S>::st(0.0f);
+        }
+    }
+
     // Columns outside the bands take the mirrored ones, in shared memory,
     // before any lane reads them (a band's box holds its neighbour bands there).
     __device__ __forceinline__ void extend_columns(S* sm, bool level1) {
         if constexpr (NL == 1) {
             fix_bands<4, SR, Lay::W1, Lay::R1>(sm, {o1l, o1h, o1l, o1h}, {fix1e, fix1o, fix1e, fix1o});
+            clear_odd<SR, Lay::W1, Lay::R1>(sm + Lay::R1 + o1h, x1);
         } else {
-            if (level1) fix_bands<3, SR, Lay::W1, Lay::R1>(sm, {o1h, o1l, o1h}, {fix1o, fix1e, fix1o});
+            if (level1) {
+                fix_bands<3, SR, Lay::W1, Lay::R1>(sm, {o1h, o1l, o1h}, {fix1o, fix1e, fix1o});
+                clear_odd<SR, Lay::W1, Lay::R1>(sm + o1h, x1);
+            }
             fix_bands<4, SR2, Lay::W2, Lay::R2>(sm + 3 * Lay::R1, {o2l, o2h, o2l, o2h},
                                                 {fix2e, fix2o, fix2e, fix2o});
+            clear_odd<SR2, Lay::W2, Lay::R2>(sm + 3 * Lay::R1 + Lay::R2 + o2h, x2);
         }
         __syncwarp();
     }

@@ -140,3 +140,29 @@ def test_single_level_launches_equal_fused_ones(h, w, levels, scheme):
         assert sum(f for f, _q, _w in fwd) == levels and sum(f for f, _q, _w in inv) == levels
         outs.append((c, y))
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+@pytest.mark.parametrize("scheme", ["nonsep_reduced", "separable", "nonsep"])
+def test_nonfinite_coefficients_stay_where_they_belong(scheme, dtype):
+    """Levels one column wide have no HL and HH bands, and the columns beside
+    their LL hold another level's details: an infinity or a NaN there may only
+    reach the samples that the oracle's inverse makes non-finite.  Wider images
+    likewise, where a box holds a neighbouring band past the border."""
+    rng = np.random.default_rng(17)
+    for h, w in [(40, 1), (1, 40), (40, 2), (64, 3), (33, 5), (64, 8), (7, 300), (37, 241)]:
+        for levels in (1, 2, 3, 6):
+            for options in (None, dict(fuse_max=1), dict(inv_cols_per_lane=4)):
+                plan = D.Plan(h, w, levels, "cdf97", scheme, dtype, options=options)
+                ws = plan.workspace()
+                for k in range(6):
+                    r, c = int(rng.integers(0, h)), min(k, w - 1) if k < 3 else int(rng.integers(0, w))
+                    x = np.full((h, w), 0.5)
+                    x[r, c] = (np.inf, np.nan)[k % 2]
+                    with np.errstate(invalid="ignore"):
+                        ref = L.inverse(x, levels, "cdf97")
+                    xd = D.empty_image(h, w, dtype)
+                    xd.copy_(torch.from_numpy(x))
+                    y = host(plan.inverse(xd, workspace=ws)).astype(np.float64)
+                    bad = np.isfinite(ref) & ~np.isfinite(y)
+                    assert not bad.any(), (h, w, levels, options, r, c, np.argwhere(bad)[:4].tolist())
