@@ -283,7 +283,7 @@ constexpr int kFwdLargeSmem = 17920;
 // Warps of a streaming kernel resident per SM (their register budgets).
 int resident_per_sm(bool fwd, int nl, int q1, int scheme) {
     if (fwd) return nl >= 3 ? 8 : (q1 >= 4 && scheme == SCH_NONSEP ? 12 : 16);
-    return q1 <= 2 ? (scheme == SCH_NONSEP ? 12 : 16) : 12;
+    return inv_resident(q1, scheme);
 }
 
 // The longest segment that streams as many slots as one of `segq` rows: a
@@ -849,12 +849,13 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     make_groups(0, false);
     make_groups(1, regroup);
     const int sms = dev.sms;
+    const bool plain97 = wavelet == DWT2D_CDF97 && base_scheme(scheme) == SCH_NONSEP;
     p->sm_count = sms;
     p->l2_bytes = dev.l2_bytes;
     p->fwd_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.fwd_warps_per_sm, 16));
     p->inv_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
-                                                                    : opt(o.inv_warps_per_sm, half ? 16 : 12));
+                                                                    : opt(o.inv_warps_per_sm, half && !plain97 ? 16 : 12));
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
     p->fill = o.min_segment == 0;
     // Warps per SM of a large launch (segments of at least *_large_segq rows), in
@@ -885,7 +886,7 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     // of 4099 x 2051 36.2 -> 31.8.
     p->fwd_large_segq = opt(o.large_segment, half ? 40 : (f32 ? 17 : 13));
     p->fwd_large_segq1 = opt(o.large_segment, half ? 40 : 20);
-    p->inv_large_segq = opt(o.large_segment, half ? 40 : 20);
+    p->inv_large_segq = opt(o.large_segment, half ? 40 : (plain97 ? 32 : 20));
     // 4 columns per lane: without being asked from 8192^2 on (one level of
     // 16384^2 342 us, with 2 columns 355); the largest of them, whose segments
     // stay longer, with 12 warps per SM (two levels of 16384^2 376 -> 359, three
@@ -894,11 +895,14 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->huge_segq4 = opt(o.large_segment, 19);
     // counts that were asked for are taken or left as a whole
     p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * (f32 ? kFwdLargeResident : 16) : 1 << 28;
-    p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * 16 : 1 << 28;
-    // The plain non-separable 9/7 inverse: 36 (8192^2 122.8, 48 123.7, 64 125.4).
-    const bool plain97 = wavelet == DWT2D_CDF97 && base_scheme(scheme) == SCH_NONSEP;
+    p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * (plain97 ? 12 : 16) : 1 << 28;
+    // The plain non-separable 9/7 inverse runs waves of its 12 resident warps, of
+    // at least 32 rows.  Float32, 5 levels: 8192^2 36 warps 112.4, 60 117.4;
+    // 4096^2 41.4 (36 of 17 rows 44.7).  16-bit 8192^2 36 115.5, 48 117.2, but
+    // 12000^2 217 and 213; 2160 x 3840 28.1 (at most 16 warps, a wave and a
+    // third, 33.4).
     const int iwl = opt(o.inv_warps_per_sm_large,
-                        plain97 ? 36 : (half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96)));
+                        half ? 48 : (plain97 ? 36 : (wavelet == DWT2D_CDF97 ? 80 : 96)));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;
     p->fwd_q1 = o.fwd_cols_per_lane;  // 0: automatic
     p->pdl = opt(o.programmatic_launch, 1) > 0;

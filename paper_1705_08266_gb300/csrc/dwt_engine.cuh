@@ -910,6 +910,11 @@ struct Pipe<float, Q, SCH_RED, true> {
 // part is scalar and the last one packed.
 template <int Q>
 constexpr int inv_pk() { return Q >= 4 ? 2 : 1; }
+// The plain form's predicts are scalar at 2 columns per lane: packed, the
+// kernel of two levels spills 40 bytes at its 168 registers, and with scalar
+// updates instead it takes the same registers but 1-2 % longer.
+template <int Q>
+constexpr int inv_pk_predict() { return Q >= 4 ? 2 : 0; }
 template <int Q>
 struct Pipe<float, Q, SCH_SEP, false> {
     using type = Chain<float, Q, OpFSV<3, -1, false>, OpFSH<3, -1>, OpFTV<2, -1>, OpFTH<2, -1>,
@@ -917,9 +922,9 @@ struct Pipe<float, Q, SCH_SEP, false> {
 };
 template <int Q>
 struct Pipe<float, Q, SCH_NONSEP, false> {
-    static constexpr int P = inv_pk<Q>();
-    using type = Chain<float, Q, OpFS<3, -1, P>, OpFT<2, -1, P>,
-                       OpFS<1, -1, P>, OpFT<0, -1, P>>;
+    static constexpr int P = inv_pk<Q>(), PT = inv_pk_predict<Q>();
+    using type = Chain<float, Q, OpFS<3, -1, P>, OpFT<2, -1, PT>,
+                       OpFS<1, -1, P>, OpFT<0, -1, PT>>;
 };
 template <int Q>
 struct Pipe<float, Q, SCH_RED, false> {

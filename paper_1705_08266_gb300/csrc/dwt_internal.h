@@ -109,6 +109,16 @@ __host__ __device__ constexpr int fwd_row_align(int nl) { return nl == 1 ? 1 : (
 // The same for the inverse (two levels: a whole level-2 row).
 __host__ __device__ constexpr int inv_row_align(int nl) { return nl == 1 ? 1 : 2; }
 
+// Warps of an inverse launch (1 or 2 fused levels) resident per SM, which its
+// kernel's register budget and the host's waves are sized by: 16 (128
+// registers) with 2 quadruple columns per lane, 12 (168) with 4 (slots of 2
+// quadruple rows) and for the plain non-separable steps (48 multiply-adds per
+// quadruple).  Registers come to an SM's four schedulers in whole warps, so a
+// bound of 9 to 11 warps gives the registers of 12; 8 (204 registers) is slower
+// but for the smallest launches: plain 9/7, 5 levels of 2160 x 3840 30.9 us at
+// 12 and 32.8 at 8.
+constexpr int inv_resident(int q1, int scheme) { return q1 <= 2 && scheme != SCH_NONSEP ? 16 : 12; }
+
 // Image rows per TMA box of the forward kernel: 8, or 4 with 4 quadruple
 // columns per lane and at most 2 fused levels.
 int fwd_slot_rows(int nl, int q1);

@@ -3,20 +3,10 @@
 // quadruple columns per lane).
 #include "dwt_inv_body.cuh"
 
-#include <type_traits>
-
 namespace dwt {
 
-// 16 warps per SM (128 registers) with 2 quadruple columns per lane, 12 with
-// 4 (slots of 2 quadruple rows); the plain non-separable steps (48
-// multiply-adds per quadruple) measured faster with the register budget of 12
-// warps
-// The plain non-separable 9/7 steps take 10 warps per SM (200 registers): at 12
-// they spill 36 bytes (5 levels of 8192^2 float32 123.9 -> 122.8 us, 16-bit
-// 117.4 -> 115.3).
 template <class S, int SCH, int NL, int Q1>
-__global__ void __launch_bounds__(kInvWarps * 32,
-                                  (Q1 <= 2 ? (SCH == SCH_NONSEP ? (std::is_same<S, int>::value ? 12 : 10) : 16) : 12) / kInvWarps)
+__global__ void __launch_bounds__(kInvWarps * 32, inv_resident(Q1, SCH) / kInvWarps)
     inv_tma_kernel(const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2,
                    const __grid_constant__ CUtensorMap ml, const FusedArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];

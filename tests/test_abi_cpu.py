@@ -214,3 +214,15 @@ def test_plan_launch_info_reports_the_chosen_shapes(L):
 def test_workspace_bytes_helper_matches_plan(h, w, lv, wav, dt):
     assert D.workspace_bytes(h, w, lv, wav, "nonsep_reduced", dt) == \
         D.Plan(h, w, lv, wav, "nonsep_reduced", dt).workspace_bytes
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+def test_plain_nonseparable_inverse_waves_are_whole(L, dtype):
+    """The plain non-separable 9/7 inverse has 12 warps per SM resident (the
+    registers of its kernel): a launch too small for several waves is one of
+    them, not one and a third.  (Without a GPU a plan assumes 148 SMs.)"""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+    for h, w in ((1080, 1920), (2048, 2048), (2160, 3840), (3000, 3000)):
+        for levels in (1, 2, 5):
+            for _f, q, warps in D.Plan(h, w, levels, "cdf97", "nonsep", dtype).launch_info(inverse=True):
+                assert q == 2 and warps <= 12 * sms, (h, w, levels, warps / sms)
