@@ -352,8 +352,8 @@ typedef struct {
  * image (1 or 2; default 2), at most per later launch (1 or 2; default 2),
  * warps per SM that the rows of one launch are cut into (the batched kernels
  * keep 12 warps per SM resident, 8 for the persistent form at 4 columns per
- * lane; default 144 while segments keep 16 rows, down to 12 for small
- * launches), the smallest row segment of a warp (quadruple rows of the last
+ * lane; default 144 while segments keep 16 rows, the inverse 96 and 40 rows,
+ * 56 for 16-bit storage, down to 12 for small launches), the smallest row segment of a warp (quadruple rows of the last
  * fused level; default 2), and whether the batch's launches use programmatic stream
  * serialization (1 on, -1 or 0 off: measured neutral to 1 % slower for
  * batches).  Every warp of a launch streams the same number of rows.

@@ -35,8 +35,12 @@ struct GroupLaunch {
 }  // namespace
 
 // Row decomposition of a batched launch (see dwt2d_batch_create): warps per
-// SM of a large and of a small launch, and the segment rows in between.
-constexpr int kBatchWarpsLarge = 144, kBatchWarpsSmall = 12, kBatchSegRows = 16;
+// SM of a large and of a small launch, and the segment rows in between.  The
+// inverse counts rows of its finest level, the forward of its coarsest, so the
+// same rows are shorter segments there.
+constexpr int kBatchWarpsSmall = 12;
+constexpr int batch_warps_large(bool fwd) { return fwd ? 144 : 96; }
+constexpr int batch_seg_rows(bool fwd, bool half) { return fwd ? 16 : (half ? 56 : 40); }
 
 // Forward levels of at most this many pixels (and more than 512 x 512) are not
 // fused in float32 (see plan_create): an image's first level (2048^2 25.0 ->
@@ -1465,6 +1469,9 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
     // third; smaller launches run fewer waves of 16-row segments down to a
     // single one, whose segments shrink.  256 images of 65-4096 pixels a side:
     // 2134 us at a fixed 48, 1820 us; 64 images of 65-600: 150 and 132 us.
+    // The inverse takes 96 warps and 40 rows (16-bit storage 56): 32 images of
+    // 1000-3000, 5/3 331 us at 144 and 16 rows, 267 so; float32 388 and 294,
+    // 16-bit 414 and 268; 8 of 8192^2, 5 levels, float32 830 and 798.
     // 4 columns per lane where the launch is that large and 256-pixel strips
     // cover its images with fewer pixels than 128-pixel ones.
     const int sms = dev.sms;
@@ -1510,15 +1517,15 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                     if (tun.cols_per_lane != 0 || b->queue) {
                         L.q1 = b->q1;
                     } else if (fwd && ek != 1 && 2 * work4 < work2 &&
-                               work4 >= (long long)sms * kBatchWarpsLarge * kBatchSegRows) {
+                               work4 >= (long long)sms * batch_warps_large(true) * batch_seg_rows(true, false)) {
                         L.q1 = 4;
                     }
                     const long long work = L.q1 == 4 ? work4 : work2;
                     auto rows_at = [&](long long w) { return (work + sms * w - 1) / (sms * w); };
                     int segq = (int)std::max<long long>(
                         min_segq, wps > 0 ? rows_at(wps)
-                                          : std::max(rows_at(kBatchWarpsLarge),
-                                                     std::min<long long>(kBatchSegRows,
+                                          : std::max(rows_at(batch_warps_large(fwd == 1)),
+                                                     std::min<long long>(batch_seg_rows(fwd == 1, ek >= 2),
                                                                          rows_at(kBatchWarpsSmall))));
                     if (wps <= 0 && tun.min_segment <= 0)
                         segq = fill_slots(fwd == 1, nl, cand[0].rho, L.q1, segq);

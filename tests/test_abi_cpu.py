@@ -226,3 +226,23 @@ def test_plain_nonseparable_inverse_waves_are_whole(L, dtype):
         for levels in (1, 2, 5):
             for _f, q, warps in D.Plan(h, w, levels, "cdf97", "nonsep", dtype).launch_info(inverse=True):
                 assert q == 2 and warps <= 12 * sms, (h, w, levels, warps / sms)
+
+
+def _batch_warps(L, items, **tuning):
+    st, b, _ws = _batch(L, items, 2, D.Tuning(**tuning) if tuning else None)
+    assert st == 0
+    n, w = ctypes.c_int32(), ctypes.c_int64()
+    assert L.dwt2d_batch_info(b, ctypes.byref(n), ctypes.byref(w)) == 0
+    L.dwt2d_batch_destroy(b)
+    return w.value
+
+
+@pytest.mark.parametrize("wav,dt,rows", [(0, 0, 40), (1, 1, 40), (0, 2, 56), (0, 3, 56)])
+@pytest.mark.parametrize("levels", [1, 2])
+def test_inverse_batch_segments_stay_long(L, wav, dt, rows, levels):
+    """By default a large inverse launch cuts no image into segments shorter
+    than this many level-1 rows, where the halo rows would cost more than the
+    launch's shorter end gives."""
+    h, n = 2000, 300
+    one_strip = [_item(h, 64, levels, inv=1, wav=wav, dt=dt) for _ in range(n)]
+    assert _batch_warps(L, one_strip) <= n * -(-(h // 2) // rows)
