@@ -112,34 +112,15 @@ struct InvWarpT {
                 if (f[i] >= 0) p[i * REGION + off[i] + r * PITCH + (f[i] & 0xffff)] = v[i][r];
     }
 
-    // A level one column wide has no HL and HH (bands at p and p + 2 REGION):
-    // what their boxes hold there is another level's, and a non-finite value of
-    // it would come through the step's zero coefficient as a NaN.  (The integer
-    // steps select instead of multiplying.)
-    template <int ROWS, int PITCH, int REGION>
-    __device__ __forceinline__ void clear_odd(S* p, const LevelCtx& x) {
-        if constexpr (std::is_same<T, float>::value) {
-            if (x.ha) return;
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r)
-                p[r * PITCH + lane] = p[2 * REGION + r * PITCH + lane] = Storage<S>::st(0.0f);
-        }
-    }
-
     // Columns outside the bands take the mirrored ones, in shared memory,
     // before any lane reads them (a band's box holds its neighbour bands there).
     __device__ __forceinline__ void extend_columns(S* sm, bool level1) {
         if constexpr (NL == 1) {
             fix_bands<4, SR, Lay::W1, Lay::R1>(sm, {o1l, o1h, o1l, o1h}, {fix1e, fix1o, fix1e, fix1o});
-            clear_odd<SR, Lay::W1, Lay::R1>(sm + Lay::R1 + o1h, x1);
         } else {
-            if (level1) {
-                fix_bands<3, SR, Lay::W1, Lay::R1>(sm, {o1h, o1l, o1h}, {fix1o, fix1e, fix1o});
-                clear_odd<SR, Lay::W1, Lay::R1>(sm + o1h, x1);
-            }
+            if (level1) fix_bands<3, SR, Lay::W1, Lay::R1>(sm, {o1h, o1l, o1h}, {fix1o, fix1e, fix1o});
             fix_bands<4, SR2, Lay::W2, Lay::R2>(sm + 3 * Lay::R1, {o2l, o2h, o2l, o2h},
                                                 {fix2e, fix2o, fix2e, fix2o});
-            clear_odd<SR2, Lay::W2, Lay::R2>(sm + 3 * Lay::R1 + Lay::R2 + o2h, x2);
         }
         __syncwarp();
     }
@@ -312,9 +293,15 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
     w.x1 = make_ctx(g1w + Q1 * lane, Q1, a.lv[0].h, a.lv[0].w, a.lv[0].s);
     const int xh1 = ne_c1 + g1w, xl1 = g1w;
     constexpr int AM = Lay::A - 1;
-    const int bx1h = xh1 & ~AM, bx1l = xl1 & ~AM;
-    w.o1h = xh1 - bx1h;
-    w.o1l = xl1 - bx1l;
+    w.o1h = xh1 & AM;
+    w.o1l = xl1 & AM;
+    // A level one column wide has no HL and HH.  Their boxes would hold another
+    // level's coefficients, whose infinities and NaNs the steps' zero
+    // coefficients do not stop, so they start left of the array and come as
+    // zeros (clearing the columns in the ring made every border strip 3 % longer).
+    constexpr int kOutside = -4096;
+    static_assert(kOutside % Lay::A == 0 && kOutside + Lay::W1 < 0, "aligned and all of it outside");
+    const int bx1h = a.lv[0].w > 1 ? xh1 - w.o1h : kOutside, bx1l = xl1 - w.o1l;
     w.even = !((w.o1h | w.o1l) & 1);
     bool active = a.lv[0].w > 1 && a.lv[0].h > 1;  // both axes of every fused level
     // the column of a band (parity par of a level of width n) outside it that
@@ -341,10 +328,10 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
         ne_r2 = (a.lv[1].h + 1) >> 1;
         w.x2 = make_ctx(g2w + W::Q2 * lane, W::Q2, a.lv[1].h, a.lv[1].w, a.lv[1].s);
         const int xh2 = ne_c2 + g2w, xl2 = g2w;
-        bx2h = xh2 & ~AM;
-        bx2l = xl2 & ~AM;
-        w.o2h = xh2 - bx2h;
-        w.o2l = xl2 - bx2l;
+        w.o2h = xh2 & AM;
+        w.o2l = xl2 & AM;
+        bx2h = a.lv[1].w > 1 ? xh2 - w.o2h : kOutside;
+        bx2l = xl2 - w.o2l;
         active = active && a.lv[1].w > 1 && a.lv[1].h > 1;
         if (w.fix) {
             w.fix2e = fix_of(g2w, a.lv[1].w, 0, W::Q2);
