@@ -68,7 +68,7 @@ struct dwt2d_plan_s {
     // strips' unequal costs), else at fwd_large_step less and so on; smaller
     // launches keep fwd_warps_target
     int fwd_warps_large, fwd_large_segq, fwd_large_segq1 /* one level */, fwd_large_step;
-    int inv_warps_large, inv_large_segq, inv_large_step;  // the same rule for inverse launches
+    int inv_warps_large, inv_large_segq, inv_large_segq1, inv_large_step;  // the same rule for inverse launches
     int large_segq4;  // rows for 4 columns per lane without being asked
     int fwd_warps_huge4, huge_segq4;  // the same for the largest launches, 12 warps per SM resident
     int fwd_q1;  // quadruple columns per lane of the forward kernel (2 or 4; 0: automatic)
@@ -464,7 +464,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             int grid_b = 0;
             decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kInvTmaWarps, 0, res, sd,
                       p->inv_seg_f);
-            if (b.segq >= p->inv_large_segq) {
+            if (b.segq >= (g.n == 1 ? p->inv_large_segq1 : p->inv_large_segq)) {
                 a = b;
                 out->grid = grid_b;
                 break;
@@ -891,6 +891,7 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->fwd_large_segq = opt(o.large_segment, half ? 40 : (f32 ? 17 : 13));
     p->fwd_large_segq1 = opt(o.large_segment, half ? 40 : 20);
     p->inv_large_segq = opt(o.large_segment, half ? 40 : (plain97 ? 32 : 20));
+    p->inv_large_segq1 = opt(o.large_segment, half ? 40 : 20);
     // 4 columns per lane: without being asked from 8192^2 on (one level of
     // 16384^2 342 us, with 2 columns 355); the largest of them, whose segments
     // stay longer, with 12 warps per SM (two levels of 16384^2 376 -> 359, three
@@ -901,12 +902,12 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * (f32 ? kFwdLargeResident : 16) : 1 << 28;
     p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * (plain97 ? 12 : 16) : 1 << 28;
     // The plain non-separable 9/7 inverse runs waves of its 12 resident warps, of
-    // at least 32 rows.  Float32, 5 levels: 8192^2 36 warps 112.4, 60 117.4;
-    // 4096^2 41.4 (36 of 17 rows 44.7).  16-bit 8192^2 36 115.5, 48 117.2, but
-    // 12000^2 217 and 213; 2160 x 3840 28.1 (at most 16 warps, a wave and a
-    // third, 33.4).
+    // at least 32 rows (one level 20).  Float32, 5 levels: 8192^2 36 warps 112.4,
+    // 60 117.4; 4096^2 41.4 (36 of 17 rows 44.7).  16-bit, two levels: 8192^2 36
+    // 97.6, 48 99.4, 12000^2 194 and 189; 2160 x 3840 17.3 (16 warps, a wave and a
+    // third, 22.2).
     const int iwl = opt(o.inv_warps_per_sm_large,
-                        half ? 48 : (plain97 ? 36 : (wavelet == DWT2D_CDF97 ? 80 : 96)));
+                        plain97 ? 36 : (half ? 48 : (wavelet == DWT2D_CDF97 ? 80 : 96)));
     p->inv_warps_large = (tuning && tuning->warps_per_sm > 0) || iwl < 0 ? 0 : sms * iwl;
     p->fwd_q1 = o.fwd_cols_per_lane;  // 0: automatic
     p->pdl = opt(o.programmatic_launch, 1) > 0;

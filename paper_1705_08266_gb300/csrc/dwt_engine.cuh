@@ -22,6 +22,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "dwt_internal.h"
 #include "dwt_steps.cuh"
 
@@ -910,11 +912,18 @@ struct Pipe<float, Q, SCH_RED, true> {
 // part is scalar and the last one packed.
 template <int Q>
 constexpr int inv_pk() { return Q >= 4 ? 2 : 1; }
-// The plain form's predicts are scalar at 2 columns per lane: packed, the
-// kernel of two levels spills 40 bytes at its 168 registers, and with scalar
-// updates instead it takes the same registers but 1-2 % longer.
-template <int Q>
-constexpr int inv_pk_predict() { return Q >= 4 ? 2 : 0; }
+// The plain form at 2 columns per lane packs all but its last predict; where a
+// level of 16-bit storage is fused with another (WIDE = false), the predicts
+// only.  With everything packed the two-level kernel spills 20 to 40 bytes at
+// its 168 registers, with these patterns none.  Two levels of 8192^2, all
+// packed / so: float32 106.0 / 92.5 us (predicts only 97.1), 16-bit 98.7 / 96.3
+// (all but the last predict 98.1).
+template <int Q, bool WIDE>
+struct PlainInverse {
+    static constexpr int P = inv_pk<Q>();
+    static constexpr int S = Q >= 4 || WIDE ? P : 0, T0 = Q >= 4 || !WIDE ? P : 0;
+    using type = Chain<float, Q, OpFS<3, -1, S>, OpFT<2, -1, P>, OpFS<1, -1, S>, OpFT<0, -1, T0>>;
+};
 template <int Q>
 struct Pipe<float, Q, SCH_SEP, false> {
     using type = Chain<float, Q, OpFSV<3, -1, false>, OpFSH<3, -1>, OpFTV<2, -1>, OpFTH<2, -1>,
@@ -922,9 +931,7 @@ struct Pipe<float, Q, SCH_SEP, false> {
 };
 template <int Q>
 struct Pipe<float, Q, SCH_NONSEP, false> {
-    static constexpr int P = inv_pk<Q>(), PT = inv_pk_predict<Q>();
-    using type = Chain<float, Q, OpFS<3, -1, P>, OpFT<2, -1, PT>,
-                       OpFS<1, -1, P>, OpFT<0, -1, PT>>;
+    using type = typename PlainInverse<Q, true>::type;
 };
 template <int Q>
 struct Pipe<float, Q, SCH_RED, false> {
@@ -966,9 +973,11 @@ constexpr float kScaleLL = (float)(1.0 / (kKd * kKd));
 constexpr float kScaleHH = (float)(kKd * kKd);
 
 // One level of the transform for one warp: the chain plus the 9/7 scaling.
-template <class T, int Q, int SCH, bool FWD>
+// WIDE: see PlainInverse.
+template <class T, int Q, int SCH, bool FWD, bool WIDE = true>
 struct Engine {
-    using ChainT = typename Pipe<T, Q, SCH, FWD>::type;
+    using ChainT = typename std::conditional_t<WIDE || FWD || SCH != SCH_NONSEP, Pipe<T, Q, SCH, FWD>,
+                                               PlainInverse<Q, WIDE>>::type;
     static constexpr int LAG = ChainT::LAG;
     ChainT chain;
     int npush;

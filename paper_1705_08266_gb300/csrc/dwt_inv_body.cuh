@@ -72,7 +72,7 @@ struct InvWarpT {
     using Lay = InvLayout<S, NL, Q1>;
     static constexpr int LAG = std::is_same<T, float>::value ? 2 : 1;
     static constexpr int Q2 = Lay::Q2;
-    Engine<T, Q1, SCH, false> e1;
+    Engine<T, Q1, SCH, false, NL == 1 || sizeof(S) == 4> e1;
     Engine<T, (Q2 > 0 ? Q2 : 1), SCH, false> e2;
     LevelCtx x1, x2;
     // column offsets of lane 0 inside each box (elements)
