@@ -359,7 +359,7 @@ typedef struct {
  * batches).  Every warp of a launch streams the same number of rows.
  * cols_per_lane: quadruple columns per lane at the first level of a launch
  * (2: a 128-pixel strip per warp; 4: a 256-pixel strip with half the strips'
- * halo overlap; 0: 2, but 4 for large forward CDF 9/7 launches of the table
+ * halo overlap; 0: 2, but 4 for large forward float32 launches of the table
  * form that 256-pixel strips cover with fewer pixels; any other value is
  * DWT2D_ERR_INVALID). */
 typedef struct {

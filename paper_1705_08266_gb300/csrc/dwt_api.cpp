@@ -1473,8 +1473,10 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
     // The inverse takes 96 warps and 40 rows (16-bit storage 56): 32 images of
     // 1000-3000, 5/3 331 us at 144 and 16 rows, 267 so; float32 388 and 294,
     // 16-bit 414 and 268; 8 of 8192^2, 5 levels, float32 830 and 798.
-    // 4 columns per lane where the launch is that large and 256-pixel strips
-    // cover its images with fewer pixels than 128-pixel ones.
+    // 4 columns per lane where a float32 launch is that large and 256-pixel
+    // strips cover its images with fewer pixels than 128-pixel ones (8 images of
+    // 8192^2: 824 us with 2, 802 with 4).  Not for 16-bit storage, as for a single
+    // image: 96 images of 65-4096 576 us with 2, 659 with 4.
     const int sms = dev.sms;
     int max_groups = 0;
     for (auto* p : b->plans) max_groups = std::max(max_groups, p->ngroups[0]);
@@ -1517,7 +1519,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                     if (cand.empty()) continue;
                     if (tun.cols_per_lane != 0 || b->queue) {
                         L.q1 = b->q1;
-                    } else if (fwd && ek != 1 && 2 * work4 < work2 &&
+                    } else if (fwd && ek == 0 && 2 * work4 < work2 &&
                                work4 >= (long long)sms * batch_warps_large(true) * batch_seg_rows(true, false)) {
                         L.q1 = 4;
                     }

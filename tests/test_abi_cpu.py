@@ -246,3 +246,13 @@ def test_inverse_batch_segments_stay_long(L, wav, dt, rows, levels):
     h, n = 2000, 300
     one_strip = [_item(h, 64, levels, inv=1, wav=wav, dt=dt) for _ in range(n)]
     assert _batch_warps(L, one_strip) <= n * -(-(h // 2) // rows)
+
+
+@pytest.mark.parametrize("dt,cols", [(0, 4), (2, 2), (3, 2)])
+def test_columns_of_a_large_forward_batch(L, dt, cols):
+    """A batch takes 4 columns per lane by default for large float32 launches
+    only, as single images do."""
+    items = [_item(8192, 8192, 2, dt=dt) for _ in range(8)]
+    both = {c: _batch_warps(L, items, cols_per_lane=c) for c in (2, 4)}
+    assert both[2] != both[4]
+    assert _batch_warps(L, items) == both[cols]

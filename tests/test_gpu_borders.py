@@ -166,3 +166,24 @@ def test_nonfinite_coefficients_stay_where_they_belong(scheme, dtype):
                     y = host(plan.inverse(xd, workspace=ws)).astype(np.float64)
                     bad = np.isfinite(ref) & ~np.isfinite(y)
                     assert not bad.any(), (h, w, levels, options, r, c, np.argwhere(bad)[:4].tolist())
+
+
+def test_default_columns_of_a_large_batch_equal_two():
+    """A float32 batch large enough for 4 columns per lane by default gives the
+    bits of 2 columns per lane."""
+    x = D.empty_image(8192, 8192)
+    x.copy_(torch.rand(8192, 8192, device="cuda"))
+    outs, warps = [], []
+    for tuning in (None, dict(cols_per_lane=2)):
+        jobs = [(x, D.empty_image(8192, 8192), 3, "cdf97", 0) for _ in range(6)]
+        b = D.Batch(jobs, tuning=tuning)
+        ws = b.workspace()
+        b.upload(ws)
+        b.launch(ws)
+        torch.cuda.synchronize()
+        assert b.status(ws) == 0
+        outs.append([d for _s, d, _l, _w, _i in jobs])
+        warps.append(b.info()[1])
+    assert warps[0] != warps[1]
+    for a, c in zip(*outs):
+        assert torch.equal(a, c)
