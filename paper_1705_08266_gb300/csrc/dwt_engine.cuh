@@ -431,7 +431,26 @@ template <int E>
 __device__ __forceinline__ bool vact(const LevelCtx& x) { return E != kInner ? x.va : true; }
 
 // float, separable (Sec. 2 matrices).  The vertical steps run as packed pairs
-// (c0, c1) / (c2, c3) of a quadruple, the horizontal ones scalar.
+// (c0, c1) / (c2, c3) of a quadruple, the horizontal ones scalar.  The inverse
+// at 4 columns per lane runs all of them as pairs of columns, which takes 5 to
+// 17 registers fewer: three fused levels, 5 levels of 3000^2 94.7 -> 85.7 us;
+// two levels of 16-bit storage, 8192^2 105.0 -> 100.0.  (The forward would
+// spill: float32 8192^2 124.9 -> 142.6.)
+template <int Q, int SIGN>
+constexpr bool sep_columns() { return SIGN < 0 && Q >= 4; }
+// f on the columns' (x, y, a, a's neighbour, b, b's neighbour), pair by pair.
+template <int Q, class F>
+__device__ __forceinline__ void column_pairs(float (&x)[Q], float (&y)[Q], const float (&a)[Q], const float (&an)[Q],
+                                             const float (&b)[Q], const float (&bn)[Q], F f) {
+#pragma unroll
+    for (int i = 0; i < Q / 2; ++i) {
+        float2 px = pk<2, Q>(x, i), py = pk<2, Q>(y, i);
+        const float2 pa = pk<2, Q>(a, i), pan = pk<2, Q>(an, i), pb = pk<2, Q>(b, i), pbn = pk<2, Q>(bn, i);
+        f(px, py, pa, pan, pb, pbn);
+        unpk<2, Q>(px, x, i);
+        unpk<2, Q>(py, y, i);
+    }
+}
 template <int ID, int SIGN>
 struct OpFTH {
     static constexpr int kind = K_NONE;
@@ -441,6 +460,9 @@ struct OpFTH {
         right_nb<E>(a.c[0], c0r, x.right);
         right_nb<E>(a.c[2], c2r, x.right);
         const float p = hcoef<E>(Coef<ID, SIGN>::v, x);
+        if constexpr (sep_columns<Q, SIGN>())
+            return column_pairs(a.c[1], a.c[3], a.c[0], c0r, a.c[2], c2r,
+                                [p](auto&... v) { f_TH(v..., p); });
 #pragma unroll
         for (int j = 0; j < Q; ++j) f_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], p);
     }
@@ -454,6 +476,9 @@ struct OpFTV {
                                                  const float (&n1)[Q], float, float,
                                                  const LevelCtx& x) {
         const float p = vcoef<E>(Coef<ID, SIGN>::v, x);
+        if constexpr (sep_columns<Q, SIGN>())
+            return column_pairs(a.c[2], a.c[3], a.c[0], n0, a.c[1], n1,
+                                [p](auto&... v) { f_TV(v..., p); });
 #pragma unroll
         for (int j = 0; j < Q; ++j)
             v_part<true>(a.c[2][j], a.c[3][j], a.c[0][j], a.c[1][j], n0[j], n1[j], p);
@@ -472,6 +497,9 @@ struct OpFSH {
         left_nb<E>(a.c[1], c1l, x.left);
         left_nb<E>(a.c[3], c3l, x.left);
         const float u = hcoef<E>(Coef<ID, SIGN>::v, x);
+        if constexpr (sep_columns<Q, SIGN>())
+            return column_pairs(a.c[0], a.c[2], a.c[1], c1l, a.c[3], c3l,
+                                [u](auto&... v) { f_SH(v..., u); });
 #pragma unroll
         for (int j = 0; j < Q; ++j) f_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], u);
     }
@@ -488,6 +516,9 @@ struct OpFSV {
                                                  const float (&up3)[Q], float, float,
                                                  const LevelCtx& x) {
         const float u = vcoef<E>(Coef<ID, SIGN>::v, x);
+        if constexpr (sep_columns<Q, SIGN>())
+            return column_pairs(a.c[0], a.c[1], a.c[2], up2, a.c[3], up3,
+                                [u](auto&... v) { f_SV(v..., u); });
 #pragma unroll
         for (int j = 0; j < Q; ++j)
             v_part<PACK>(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], up2[j], up3[j], u);
@@ -563,7 +594,10 @@ struct OpFS {
 // float, non-separable, reduced form: one spatial step of 8 multiply-adds per
 // quadruple.  The vertical part runs first, on whole quadruples (pairs); the
 // horizontal part then reads the neighbour's result of it by shuffle instead
-// of recomputing it (the ph pv n0r term of the split P0 + P1).
+// of recomputing it (the ph pv n0r term of the split P0 + P1).  kEdgeAll, whose
+// kernel pushes one row at a time and waits for every exchange, fetches what
+// the neighbour's result is made of beforehand and computes it again, with
+// the same bits.
 template <int ID, int SIGN, bool PACK>
 struct OpRT {
     static constexpr int kind = K_DOWN;
@@ -573,12 +607,15 @@ struct OpRT {
                                                  const float (&n1)[Q], float, float,
                                                  const LevelCtx& x) {
         const float ph = hcoef<E>(Coef<ID, SIGN>::v, x), pv = vcoef<E>(Coef<ID, SIGN>::v, x);
-        float c0r[Q], c2r[Q];
-        right_nb<E>(a.c[0], c0r, x.right);
+        float c0r[Q], c2r[Q], c2n{};
+        const float c0n = shfl_dn(a.c[0][0]);
+        if constexpr (E == kEdgeAll) c2n = vfma(pv, vadd(c0n, shfl_dn(n0[0])), shfl_dn(a.c[2][0]));
+        right_of<E>(a.c[0], c0n, c0r, x.right);
 #pragma unroll
         for (int j = 0; j < Q; ++j)
             v_part<PACK>(a.c[2][j], a.c[3][j], a.c[0][j], a.c[1][j], n0[j], n1[j], pv);
-        right_nb<E>(a.c[2], c2r, x.right);
+        if constexpr (E != kEdgeAll) c2n = shfl_dn(a.c[2][0]);
+        right_of<E>(a.c[2], c2n, c2r, x.right);
 #pragma unroll
         for (int j = 0; j < Q; ++j) f_TH(a.c[1][j], a.c[3][j], a.c[0][j], c0r[j], a.c[2][j], c2r[j], ph);
     }
@@ -593,12 +630,15 @@ struct OpRS {
                                                  const float (&up3)[Q], float, float,
                                                  const LevelCtx& x) {
         const float uh = hcoef<E>(Coef<ID, SIGN>::v, x), uv = vcoef<E>(Coef<ID, SIGN>::v, x);
-        float c1l[Q], c3l[Q];
-        left_nb<E>(a.c[3], c3l, x.left);
+        float c1l[Q], c3l[Q], c1p{};
+        const float c3p = shfl_up(a.c[3][Q - 1]);
+        if constexpr (E == kEdgeAll) c1p = vfma(uv, vadd(c3p, shfl_up(up3[Q - 1])), shfl_up(a.c[1][Q - 1]));
+        left_of<E>(a.c[3], c3p, c3l, x.left);
 #pragma unroll
         for (int j = 0; j < Q; ++j)
             v_part<PACK>(a.c[0][j], a.c[1][j], a.c[2][j], a.c[3][j], up2[j], up3[j], uv);
-        left_nb<E>(a.c[1], c1l, x.left);
+        if constexpr (E != kEdgeAll) c1p = shfl_up(a.c[1][Q - 1]);
+        left_of<E>(a.c[1], c1p, c1l, x.left);
 #pragma unroll
         for (int j = 0; j < Q; ++j) f_SH(a.c[0][j], a.c[2][j], a.c[1][j], c1l[j], a.c[3][j], c3l[j], uh);
     }
