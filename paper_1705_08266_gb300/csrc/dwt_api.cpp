@@ -48,6 +48,8 @@ constexpr int batch_seg_rows(bool fwd, bool half) { return fwd ? 16 : (half ? 56
 // a launch before it has left in L2 (5 levels of 2500 x 5000 35.2 -> 33.2).
 constexpr long long kSingleFirst = 7000000, kSinglePixels = 4000000;
 
+constexpr int kOneStep = 1 << 28;  // a wave count that is taken or left as a whole
+
 constexpr int kMaxHostBands = 64;  // row bands of the pipelined host-buffer entry points
 
 struct dwt2d_plan_s {
@@ -63,6 +65,7 @@ struct dwt2d_plan_s {
     int sm_count;
     long long l2_bytes;  // L2 cache of the device the plan was made on
     int fwd_warps_target, inv_warps_target;
+    bool fwd_small_auto;  // fwd_warps_target was not asked for
     // a forward launch whose rows allow segments of at least fwd_large_segq rows
     // at fwd_warps_large warps runs that many (several waves even out the
     // strips' unequal costs), else at fwd_large_step less and so on; smaller
@@ -285,9 +288,9 @@ constexpr int kFwdLargeResident = 12;
 constexpr int kFwdLargeSmem = 17920;
 
 // Warps of a streaming kernel resident per SM (their register budgets).
-int resident_per_sm(bool fwd, int nl, int q1, int scheme) {
-    if (fwd) return nl >= 3 ? 8 : (q1 >= 4 && scheme == SCH_NONSEP ? 12 : 16);
-    return inv_resident(q1, scheme);
+int resident_per_sm(const dwt2d_plan_s* p, bool fwd, int nl, int q1) {
+    const int sch = base_scheme(p->scheme);
+    return fwd ? fwd_resident(sch, nl, q1, p->dtype == DWT2D_F32) : inv_resident(q1, sch);
 }
 
 // The longest segment that streams as many slots as one of `segq` rows: a
@@ -380,7 +383,6 @@ int elem_kind_of(dwt2d_dtype d) {
 // row decomposition.
 void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv_target, GroupLaunch* out,
                  int segq_fixed = 0, bool uniform_segments = false) {
-    const int sch = base_scheme(p->scheme);
     const int elem_kind = elem_kind_of(p->dtype);
     const int rho = p->wavelet == DWT2D_CDF97 ? 2 : 1;
     FusedArgs& a = out->a;
@@ -411,7 +413,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         if (g.n <= 2 && p->fwd_q1 == 0 && segq_fixed <= 0 && elem_kind == 0 && p->fwd_warps_large4 > 0) {
             const struct { int warps, resident, segq, smem; } tries[2] = {
                 {p->fwd_warps_huge4, kFwdLargeResident, p->huge_segq4, kFwdLargeSmem},
-                {p->fwd_warps_large4, resident_per_sm(true, g.n, 4, sch), p->large_segq4, 0}};
+                {p->fwd_warps_large4, resident_per_sm(p, true, g.n, 4), p->large_segq4, 0}};
             for (int i = p->fwd_warps_huge4 > 0 ? 0 : 1; i < 2 && !use4; ++i) {
                 big4 = a;
                 decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, tries[i].warps, &big4, &grid4, kFwdWarps, 0,
@@ -425,14 +427,21 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             a = big4;
             out->grid = grid4;
         } else {
-            const int res = resident_per_sm(true, g.n, q1, sch);
+            const int res = resident_per_sm(p, true, g.n, q1);
             const bool fewer = elem_kind == 0 && q1 == 2;  // kFwdLargeResident warps per SM
             const int segq_min = q1 == 4 ? p->large_segq4 : (g.n == 1 ? p->fwd_large_segq1 : p->fwd_large_segq);
             const int large = q1 == 4 ? p->fwd_warps_large4 : p->fwd_warps_large;
             const int sd = uniform_segments ? 0 : (q1 == 4 ? p->fwd_short4 : p->fwd_short);
+            // 4 columns per lane run waves of their own resident warps (two levels
+            // of 3000^2 float32: 16 warps, a wave and a third, 26.1 us, 12 19.9)
+            int step = p->fwd_large_step;
+            if (q1 == 4 && g.n <= 2) {
+                if (p->fwd_small_auto) fwd_target = std::min(fwd_target, p->sm_count * res);
+                if (step < kOneStep) step = p->sm_count * res;
+            }
             decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, fwd_target, &a, &out->grid, kFwdWarps,
                       segq_fixed, res, 0, p->fwd_seg_f);
-            for (int t = large; segq_fixed <= 0 && t > fwd_target; t -= p->fwd_large_step) {
+            for (int t = large; segq_fixed <= 0 && t > fwd_target; t -= step) {
                 FusedArgs b = a;
                 int grid_b = 0;
                 decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kFwdWarps, 0,
@@ -453,7 +462,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         // 2 columns per lane unless 4 are asked for
         const int rows = (a.lv[0].h + 1) / 2;
         const int q1 = p->inv_q1 == 4 ? 4 : 2;
-        const int res = resident_per_sm(false, g.n, q1, sch);
+        const int res = resident_per_sm(p, false, g.n, q1);
         const int large = q1 == 4 ? p->inv_warps_large4 : p->inv_warps_large;
         const int sd = uniform_segments ? 0 : p->inv_short;
         // the inverse measured fastest with its segments top to bottom
@@ -858,6 +867,7 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->l2_bytes = dev.l2_bytes;
     p->fwd_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.fwd_warps_per_sm, 16));
+    p->fwd_small_auto = !(tuning && tuning->warps_per_sm > 0) && o.fwd_warps_per_sm == 0;
     p->inv_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.inv_warps_per_sm, half && !plain97 ? 16 : 12));
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
@@ -899,8 +909,8 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->large_segq4 = opt(o.large_segment, 16);
     p->huge_segq4 = opt(o.large_segment, 19);
     // counts that were asked for are taken or left as a whole
-    p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * (f32 ? kFwdLargeResident : 16) : 1 << 28;
-    p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * (plain97 ? 12 : 16) : 1 << 28;
+    p->fwd_large_step = o.fwd_warps_per_sm_large == 0 ? sms * (f32 ? kFwdLargeResident : 16) : kOneStep;
+    p->inv_large_step = o.inv_warps_per_sm_large == 0 ? sms * (plain97 ? 12 : 16) : kOneStep;
     // The plain non-separable 9/7 inverse runs waves of its 12 resident warps, of
     // at least 32 rows (one level 20).  Float32, 5 levels: 8192^2 36 warps 112.4,
     // 60 117.4; 4096^2 41.4 (36 of 17 rows 44.7).  16-bit, two levels: 8192^2 36

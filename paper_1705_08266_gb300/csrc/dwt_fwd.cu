@@ -4,11 +4,12 @@
 #include "dwt_fwd_body.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace dwt {
 
 template <class S, int SCH, int NL, int Q1>
-__global__ void __launch_bounds__(kFwdWarps * 32, fwd_min_blocks<SCH, NL, Q1>())
+__global__ void __launch_bounds__(kFwdWarps * 32, fwd_resident(SCH, NL, Q1, std::is_same<S, float>::value) / kFwdWarps)
     fwd_fused_kernel(const __grid_constant__ CUtensorMap map, const FusedArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     grid_dependents_launch();  // the body waits for the previous grid after its setup

@@ -300,14 +300,6 @@ __device__ __forceinline__ bool rows_interior(int q0, int sr, int nl, int lag, c
     return true;
 }
 
-// CTAs per SM the register budget is sized for: 16 warps (128 registers), or
-// 12 (168) for the plain non-separable steps at 4 quadruple columns per lane,
-// 8 for three fused levels.
-template <int SCH, int NL, int Q1>
-__host__ __device__ constexpr int fwd_min_blocks() {
-    return (NL >= 3 ? 8 : (Q1 >= 4 && SCH == SCH_NONSEP ? 12 : 16)) / kFwdWarps;
-}
-
 // One warp's work item `wid` of a launch described by `a` (input through the
 // tensor map at `mapp`).
 // Returns false if a bounded wait gave up (the status word is set).

@@ -109,6 +109,16 @@ __host__ __device__ constexpr int fwd_row_align(int nl) { return nl == 1 ? 1 : (
 // The same for the inverse (two levels: a whole level-2 row).
 __host__ __device__ constexpr int inv_row_align(int nl) { return nl == 1 ? 1 : 2; }
 
+// Warps of a forward launch resident per SM, which its kernel's register budget
+// and the host's waves are sized by: 16 (128 registers); 12 (168) at 4 quadruple
+// columns per lane for two levels, and for one of float32 or in plain
+// non-separable steps; 8 for three fused levels.  Two levels at 4 columns, 16
+// and 12 warps: float32 8192^2 101.7 and 99.2 us, 1080 x 1920 12.7 and 11.1; 5/3
+// 8192^2 103.8 and 92.9; 16-bit 5 levels of 1080 x 1920 34.0 and 29.0.
+constexpr int fwd_resident(int scheme, int nl, int q1, bool f32) {
+    return nl >= 3 ? 8 : (q1 >= 4 && (nl == 2 || f32 || scheme == SCH_NONSEP) ? 12 : 16);
+}
+
 // Warps of an inverse launch (1 or 2 fused levels) resident per SM, which its
 // kernel's register budget and the host's waves are sized by: 16 (128
 // registers) with 2 quadruple columns per lane, 12 (168) with 4 (slots of 2

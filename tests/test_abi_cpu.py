@@ -256,3 +256,20 @@ def test_columns_of_a_large_forward_batch(L, dt, cols):
     both = {c: _batch_warps(L, items, cols_per_lane=c) for c in (2, 4)}
     assert both[2] != both[4]
     assert _batch_warps(L, items) == both[cols]
+
+
+@pytest.mark.parametrize("wav,scheme,dtype", [("cdf97", "nonsep_reduced", torch.float32),
+                                              ("cdf97", "separable", torch.float16),
+                                              ("cdf97", "nonsep", torch.float32),
+                                              ("legall53", "separable", torch.int32)])
+def test_forward_waves_at_four_columns_are_whole(L, wav, scheme, dtype):
+    """Two fused levels at 4 columns per lane have 12 warps per SM resident: a
+    launch too small for several waves is one of them.  A count that was asked
+    for is taken."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+    cols = dict(fwd_cols_per_lane=4, fuse_first=2, fuse_max=2)
+    for h, w in ((1080, 1920), (2048, 2048), (3000, 3000)):
+        p = D.Plan(h, w, 2, wav, scheme, dtype, options=cols)
+        assert all(n <= 12 * sms for _f, _q, n in p.launch_info()), (h, w)
+    asked = D.Plan(3000, 3000, 2, wav, scheme, dtype, options=dict(cols, fwd_warps_per_sm=16)).launch_info()
+    assert asked[0][2] > 12 * sms
