@@ -187,3 +187,27 @@ def test_default_columns_of_a_large_batch_equal_two():
     assert warps[0] != warps[1]
     for a, c in zip(*outs):
         assert torch.equal(a, c)
+
+
+@pytest.mark.parametrize("scheme", ["nonsep_reduced", "separable", "nonsep"])
+def test_nonfinite_pixels_stay_where_they_belong(scheme):
+    """Forward, up to three fused levels: an infinity or a NaN of the image only
+    reaches the coefficients that the oracle makes non-finite, also where a
+    level is one row or one column."""
+    rng = np.random.default_rng(19)
+    for h, w in [(1, 40), (2, 40), (3, 64), (40, 2), (64, 3), (5, 33), (7, 300), (37, 241)]:
+        for levels in (1, 2, 3, 6):
+            for options in (None, dict(fuse_max=1), dict(fwd_cols_per_lane=4), dict(fuse_first=3, fuse_max=3)):
+                plan = D.Plan(h, w, levels, "cdf97", scheme, options=options)
+                ws = plan.workspace()
+                for k in range(6):
+                    r, c = int(rng.integers(0, h)), int(rng.integers(0, w))
+                    x = np.full((h, w), 0.5)
+                    x[r, c] = (np.inf, np.nan)[k % 2]
+                    with np.errstate(invalid="ignore"):
+                        ref = L.forward(x, levels, "cdf97")
+                    xd = D.empty_image(h, w)
+                    xd.copy_(torch.from_numpy(x))
+                    y = host(plan.forward(xd, workspace=ws))
+                    bad = np.isfinite(ref) & ~np.isfinite(y)
+                    assert not bad.any(), (h, w, levels, options, r, c, np.argwhere(bad)[:4].tolist())
