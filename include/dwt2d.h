@@ -130,7 +130,10 @@ typedef struct {
                                       columns per lane; 16-bit storage caps both at 2).  With both
                                       at 0 a forward float32 level of 512 x 512 to 4 million pixels
                                       (the first: 7 million) has a launch of its own */
-    int32_t fwd_warps_per_sm;      /* warps a forward launch is cut into, per SM (default 16) */
+    int32_t fwd_warps_per_sm;      /* warps a forward launch is cut into, per SM (default 16, 12 where
+                                      the kernel has 12 resident; a count that is asked for here or
+                                      below is cut as asked, by default segments are made longer to
+                                      fill the warps' slots) */
     int32_t inv_warps_per_sm;      /* the same for the inverse (default 16 for 16-bit
                                       storage, else 12) */
     int32_t fwd_warps_per_sm_large;/* forward launches whose row segments stay at least

@@ -79,7 +79,8 @@ struct dwt2d_plan_s {
     int inv_warps_large4;
     int inv_q1;  // the same for the inverse
     int min_segq;
-    bool fill;  // segments fill whole slots (unless the shortest segment was asked for)
+    // segments fill whole slots, inverse [0] and forward [1] (unless their number was asked for)
+    bool fill_small[2], fill_large[2];
     int pdl;  // device entry points: launches with programmatic stream serialization
     int fwd_short, inv_short;  // short last-wave segments: divisor (0: off)
     int fwd_seg_f;  // forward segment interleave (0: as many groups as waves)
@@ -296,7 +297,8 @@ int resident_per_sm(const dwt2d_plan_s* p, bool fwd, int nl, int q1) {
 // The longest segment that streams as many slots as one of `segq` rows: a
 // segment's halo rows and its own fill whole slots, so that no slot is mostly
 // rows of the next segment (2048 x 2048, two levels: 103 segments of 5 rows
-// and 6 slots became 86 of 6 rows and 6 slots).
+// and 6 slots became 86 of 6 rows and 6 slots).  Counts of warps that a caller
+// asks for are cut as asked.
 int fill_slots(bool fwd, int nl, int rho, int q1, int segq) {
     if (nl > 2) return segq;
     const int sr = fwd ? fwd_slot_rows(nl, q1) / 2 : inv_slot_rows(q1);
@@ -309,12 +311,13 @@ int fill_slots(bool fwd, int nl, int rho, int q1, int segq) {
 }
 
 // Warp work decomposition of one streaming launch.
-// Rows per warp: enough segments for target_warps warps, or segq_fixed (> 0).
+// Rows per warp: enough segments for target_warps warps, made longer to fill
+// their slots (fill), or segq_fixed (> 0).
 // With short_div > 1 the rows at the bottom that one wave of resident warps
 // (resident per SM) takes are cut into segments short_div times shorter and
 // taken last: the launch's last warps are short, so it drains quickly.
 void decompose(const dwt2d_plan_s* p, bool fwd, int w_first, int rows, int nl, int rho, int q1,
-               int target_warps, FusedArgs* a, int* grid, int warps_per_block, int segq_fixed = 0,
+               int target_warps, bool fill, FusedArgs* a, int* grid, int warps_per_block, int segq_fixed = 0,
                int resident = 16, int short_div = 0, int seg_f_opt = 0) {
     valid_lanes(nl, rho, q1, &a->lane_lo, &a->lane_hi);
     const int qn = q1 >> (nl - 1);
@@ -333,7 +336,7 @@ void decompose(const dwt2d_plan_s* p, bool fwd, int w_first, int rows, int nl, i
         segq = (rows + nsegs - 1) / nsegs;
     }
     if (segq < p->min_segq) segq = p->min_segq;
-    const bool fill = segq_fixed <= 0 && p->fill;
+    fill = fill && segq_fixed <= 0;
     if (fill) segq = fill_slots(fwd, nl, rho, q1, segq);
     if (segq > rows) segq = rows;
     if (segq < 1) segq = 1;
@@ -416,7 +419,8 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
                 {p->fwd_warps_large4, resident_per_sm(p, true, g.n, 4), p->large_segq4, 0}};
             for (int i = p->fwd_warps_huge4 > 0 ? 0 : 1; i < 2 && !use4; ++i) {
                 big4 = a;
-                decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, tries[i].warps, &big4, &grid4, kFwdWarps, 0,
+                decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, tries[i].warps, p->fill_large[1], &big4, &grid4,
+                          kFwdWarps, 0,
                           tries[i].resident, uniform_segments ? 0 : p->fwd_short4, p->fwd_seg_f);
                 big4.min_smem = tries[i].smem;
                 use4 = big4.segq >= tries[i].segq;
@@ -439,12 +443,12 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
                 if (p->fwd_small_auto) fwd_target = std::min(fwd_target, p->sm_count * res);
                 if (step < kOneStep) step = p->sm_count * res;
             }
-            decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, fwd_target, &a, &out->grid, kFwdWarps,
+            decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, fwd_target, p->fill_small[1], &a, &out->grid, kFwdWarps,
                       segq_fixed, res, 0, p->fwd_seg_f);
             for (int t = large; segq_fixed <= 0 && t > fwd_target; t -= step) {
                 FusedArgs b = a;
                 int grid_b = 0;
-                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kFwdWarps, 0,
+                decompose(p, true, a.lv[0].w, rows, g.n, rho, q1, t, p->fill_large[1], &b, &grid_b, kFwdWarps, 0,
                           fewer ? kFwdLargeResident : res, sd, p->fwd_seg_f);
                 if (b.segq >= segq_min) {
                     a = b;
@@ -466,12 +470,12 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         const int large = q1 == 4 ? p->inv_warps_large4 : p->inv_warps_large;
         const int sd = uniform_segments ? 0 : p->inv_short;
         // the inverse measured fastest with its segments top to bottom
-        decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, inv_target, &a, &out->grid, kInvTmaWarps,
+        decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, inv_target, p->fill_small[0], &a, &out->grid, kInvTmaWarps,
                   segq_fixed, res, 0, p->inv_seg_f);
         for (int t = large; segq_fixed <= 0 && t > inv_target; t -= p->inv_large_step) {
             FusedArgs b = a;
             int grid_b = 0;
-            decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, t, &b, &grid_b, kInvTmaWarps, 0, res, sd,
+            decompose(p, false, a.lv[0].w, rows, g.n, rho, q1, t, p->fill_large[0], &b, &grid_b, kInvTmaWarps, 0, res, sd,
                       p->inv_seg_f);
             if (b.segq >= (g.n == 1 ? p->inv_large_segq1 : p->inv_large_segq)) {
                 a = b;
@@ -482,7 +486,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         out->path = 1;
         out->q1 = q1;
     } else {
-        decompose(p, false, a.lv[0].w, (a.lv[0].h + 1) / 2, g.n, rho, 4, inv_target, &a, &out->grid, 4, 0,
+        decompose(p, false, a.lv[0].w, (a.lv[0].h + 1) / 2, g.n, rho, 4, inv_target, p->fill_small[0], &a, &out->grid, 4, 0,
                   8, 0, p->inv_seg_f);
         out->path = 2;
         out->q1 = 4;
@@ -871,7 +875,10 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->inv_warps_target = sms * (tuning && tuning->warps_per_sm > 0 ? tuning->warps_per_sm
                                                                     : opt(o.inv_warps_per_sm, half && !plain97 ? 16 : 12));
     p->min_segq = tuning && tuning->min_segment > 0 ? tuning->min_segment : opt(o.min_segment, 2);
-    p->fill = o.min_segment == 0;
+    p->fill_small[0] = o.inv_warps_per_sm == 0;
+    p->fill_small[1] = o.fwd_warps_per_sm == 0;
+    p->fill_large[0] = o.inv_warps_per_sm_large == 0;
+    p->fill_large[1] = o.fwd_warps_per_sm_large == 0;
     // Warps per SM of a large launch (segments of at least *_large_segq rows), in
     // waves of the resident warps (12 for float32 forward, else 16).  More warps:
     // shorter last segments and a more compact set of rows in flight, but more
@@ -1504,7 +1511,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                     auto strips = [&](const dwt2d_plan_s* p, const Cand& c, int q, int segq, FusedArgs* a) {
                         memset(a, 0, sizeof(*a));
                         int grid = 0;
-                        decompose(p, fwd == 1, c.w0, c.rows, nl, c.rho, q, 1, a, &grid, 4, segq);
+                        decompose(p, fwd == 1, c.w0, c.rows, nl, c.rho, q, 1, false, a, &grid, 4, segq);
                         return (long long)a->nstrips;
                     };
                     for (int i = 0; i < n; ++i) {
@@ -1540,7 +1547,7 @@ dwt2d_status dwt2d_batch_create(dwt2d_batch_t* out, const dwt2d_batch_item* item
                                           : std::max(rows_at(batch_warps_large(fwd == 1)),
                                                      std::min<long long>(batch_seg_rows(fwd == 1, ek >= 2),
                                                                          rows_at(kBatchWarpsSmall))));
-                    if (wps <= 0 && tun.min_segment <= 0)
+                    if (wps <= 0)
                         segq = fill_slots(fwd == 1, nl, cand[0].rho, L.q1, segq);
                     long long warps = 0;
                     for (const Cand& c : cand) {

@@ -273,3 +273,21 @@ def test_forward_waves_at_four_columns_are_whole(L, wav, scheme, dtype):
         assert all(n <= 12 * sms for _f, _q, n in p.launch_info()), (h, w)
     asked = D.Plan(3000, 3000, 2, wav, scheme, dtype, options=dict(cols, fwd_warps_per_sm=16)).launch_info()
     assert asked[0][2] > 12 * sms
+
+
+def test_asked_for_decompositions_are_taken(L):
+    """min_segment = 2 is the default, and a number of warps that was asked for
+    is not changed to fill the warps' slots."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+    for h, w, levels in ((2048, 2048, 2), (3000, 9000, 5), (777, 3001, 2), (8192, 8192, 5)):
+        default, two = D.Plan(h, w, levels), D.Plan(h, w, levels, options=dict(min_segment=2))
+        for inverse in (False, True):
+            assert default.launch_info(inverse) == two.launch_info(inverse), (h, w, levels, inverse)
+    items = [_item(700, 900, 3), _item(2000, 1300, 2, inv=1), _item(900, 4000, 1, dt=2)]
+    assert _batch_warps(L, items) == _batch_warps(L, items, min_segment=2)
+    strips, rows = -(-2048 // 120), 1024  # one level, 2 columns per lane
+    for n in range(2, 17):
+        segq = max(2, -(-rows // (n * sms // strips)))
+        for key, inverse in (("fwd_warps_per_sm", False), ("inv_warps_per_sm", True)):
+            p = D.Plan(2048, 2048, 1, options={key: n, key + "_large": -1})
+            assert p.launch_info(inverse)[0][2] == strips * -(-rows // segq), (key, n)
