@@ -25,6 +25,10 @@ from typing import Callable, Iterable, Optional
 
 KNOBS = ("fuse_first", "fuse_max", "warps_per_sm", "min_segment", "persistent", "cols_per_lane")
 
+# The library's own choice (rows by the size of each launch, columns per lane
+# by launch), which no list of fixed settings contains.
+LIBRARY_DEFAULT = dict.fromkeys(KNOBS, 0)
+
 CANDIDATES = [
     {"fuse_first": ff, "fuse_max": 2, "warps_per_sm": w, "min_segment": m, "persistent": 0,
      "cols_per_lane": 2}
@@ -111,7 +115,9 @@ def pick(sig: str, measure: Callable[[dict], float], candidates=None, cache_path
 def tune(jobs, scheme: str = "nonsep_reduced", cache_path: Optional[str] = None, iters: int = 5,
          warmup: int = 2, stream=None, candidates=None) -> dict:
     """Time the candidates on `jobs` (as for dwt2d.Batch) and return the best
-    tuning dict.  Overwrites the jobs' outputs."""
+    tuning dict.  Overwrites the jobs' outputs.  Unless the caller names the
+    candidates, the library's default is the first of them: tuning never
+    settles for less than not tuning."""
     import torch
 
     from . import dwt2d as D
@@ -146,4 +152,5 @@ def tune(jobs, scheme: str = "nonsep_reduced", cache_path: Optional[str] = None,
     props = torch.cuda.get_device_properties(dev)
     st_lib = os.stat(D.LIB_PATH)
     context = f"{props.name}/{props.multi_processor_count}sm/lib{st_lib.st_size}.{st_lib.st_mtime_ns}"
-    return pick(signature(descs), measure, candidates, cache_path, scheme, context)
+    return pick(signature(descs), measure, candidates or [LIBRARY_DEFAULT] + CANDIDATES, cache_path, scheme,
+                context)

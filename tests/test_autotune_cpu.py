@@ -70,3 +70,30 @@ def test_context_separates_cache_entries(tmp_path):
     A.pick("sig", measure, cache_path=path, context="GPU-B/132sm/lib1")
     assert len(calls) == 2 * n  # measured again
     assert len(json.load(open(path))) == 2
+
+
+def test_tune_times_the_library_default_first(monkeypatch):
+    """Unless told otherwise, tune() offers no tuning at all beside the fixed
+    settings; candidates a caller names are taken as they are."""
+    from types import SimpleNamespace
+
+    import torch
+
+    from paper_1705_08266_gb300 import dwt2d as D
+
+    seen = {}
+
+    def pick(sig, measure, candidates, cache_path, scheme, context):
+        seen["candidates"] = candidates
+        return dict(candidates[0])
+
+    monkeypatch.setattr(A, "pick", pick)
+    monkeypatch.setattr(torch.cuda, "get_device_properties",
+                        lambda dev: SimpleNamespace(name="stand-in", multi_processor_count=1))
+    jobs = [(torch.zeros(8, 8), torch.zeros(8, 8), 1, "cdf97", 0)]
+    best = A.tune(jobs, stream=object())
+    assert set(best) == set(A.KNOBS) and not any(best.values())
+    D.Tuning(**best)  # every knob of it is one of the library's
+    assert seen["candidates"][1:] == A.CANDIDATES
+    A.tune(jobs, stream=object(), candidates=A.CANDIDATES[:2])
+    assert seen["candidates"] == A.CANDIDATES[:2]
