@@ -275,19 +275,6 @@ dwt2d_status check_buffers(const dwt2d_plan_s* p, const void* src, int64_t sp, c
     return DWT2D_OK;
 }
 
-// A large float32 forward launch keeps 12 warps per SM in flight instead of the
-// 16 its registers allow: it is bound by HBM, and fewer rows in flight share
-// DRAM pages better.  Each warp asks for more shared memory than its ring
-// takes, so that 12 fit the 228 KB of an SM (1 KB of it per CTA reserved).
-// Two levels, us, 16 / 12 warps: 2 columns per lane 6000^2 57.3 / 54.4, 3000 x
-// 20000 89.8 / 86.5; 4 columns 6000 x 20000 169 / 163.6, 16384^2 367 / 354 (2
-// columns of 8192^2: 98.2 / 94.1, 10 warps 95.9, 8 warps 97.6).  A launch of one
-// wave keeps 16 (4096^2 28.1 and 28.5), and so do the inverse (88.6 and 90.3),
-// 5/3 (86.9 and 86.6) and 16-bit storage, which is bound by its arithmetic (78
-// and 80).
-constexpr int kFwdLargeResident = 12;
-constexpr int kFwdLargeSmem = 17920;
-
 // Warps of a streaming kernel resident per SM (their register budgets).
 int resident_per_sm(const dwt2d_plan_s* p, bool fwd, int nl, int q1) {
     const int sch = base_scheme(p->scheme);
@@ -849,7 +836,9 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     // with 2 + 2 + 1, 19.4 with 1 + 1 + 2 + 1).  Not below 512 x 512, where the
     // launches themselves are (15.1 and 15.0 us), nor for 5/3 (8 halo rows: 1080
     // x 1920 14.5 and 14.9 us) or the inverse (18.5 and 19.6), nor for 16-bit
-    // storage, whose LL between launches is rounded.
+    // storage, whose LL between launches is rounded; nor where only that takes
+    // the workspace past the scratch of dwt2d_forward_noalloc, which such a
+    // plan would lose (below).
     const bool regroup = !tuning && wavelet == DWT2D_CDF97 && dtype == DWT2D_F32 && o.fuse_first == 0 &&
                          o.fuse_max == 0 && !multipass(scheme) && !convolution(scheme);
     auto make_groups = [&](int dir, bool single) {
@@ -979,7 +968,9 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
             return kHeader + (ba + 255) / 256 * 256 + (bb + 255) / 256 * 256;
         };
         // a workspace that fits the allocation-free entry point with the usual
-        // groups stays that small
+        // groups stays that small (with 3 or more levels this keeps the usual
+        // groups for first levels above 6.7 million pixels, and for images of 26.8
+        // to 33.5 million)
         if (size_buffers() > DWT2D_NOALLOC_SCRATCH_BYTES && regroup) {
             make_groups(1, false);
             if (size_buffers() > DWT2D_NOALLOC_SCRATCH_BYTES) {

@@ -259,6 +259,12 @@ __device__ __forceinline__ void copy_args(SharedArgs* to, const FusedArgs& from)
     __syncwarp();
 }
 
+// Shared memory that a kernel may use without an opt-in, which no launch asks
+// for, less what is static: a batched kernel's arguments and the store windows
+// of a bounds-checked build.
+constexpr size_t kSmemBytes = 48 * 1024 - sizeof(SharedArgs) - 32 * sizeof(StoreWindows);
+static_assert(kFwdLargeSmem <= kSmemBytes, "a large forward launch's request");
+
 // Per-level information of one lane (horizontal) and of the level (vertical).
 struct LevelCtx {
     unsigned right;  // bit j: column j has its right (even) neighbour inside the image

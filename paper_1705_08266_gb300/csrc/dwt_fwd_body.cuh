@@ -318,6 +318,7 @@ __device__ __forceinline__ bool fwd_body(const CUtensorMap* mapp, const FusedArg
     const int warp = threadIdx.x >> 5;
 
     constexpr int kSlotElems = SLOT_ROWS * BW;
+    static_assert(kFwdWarps * kFwdSlots * (kSlotElems * sizeof(S) + 8) <= kSmemBytes, "rings need an opt-in");
     S* ring = reinterpret_cast<S*>(smem_raw) + (size_t)warp * kFwdSlots * kSlotElems;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + (size_t)kFwdWarps * kFwdSlots *
                                                               kSlotElems * sizeof(S)) +

@@ -119,6 +119,20 @@ constexpr int fwd_resident(int scheme, int nl, int q1, bool f32) {
     return nl >= 3 ? 8 : (q1 >= 4 && (nl == 2 || f32 || scheme == SCH_NONSEP) ? 12 : 16);
 }
 
+// A large float32 forward launch keeps 12 warps per SM in flight instead of the
+// 16 its registers allow: it is bound by HBM, and fewer rows in flight share
+// DRAM pages better.  Each warp asks for more shared memory than its ring
+// takes, so that 12 fit the 228 KB of an SM (1 KB of it per CTA reserved; at 4
+// columns per lane the registers allow no more either).
+// Two levels, us, 16 / 12 warps: 2 columns per lane 6000^2 57.3 / 54.4, 3000 x
+// 20000 89.8 / 86.5; 4 columns 6000 x 20000 169 / 163.6, 16384^2 367 / 354 (2
+// columns of 8192^2: 98.2 / 94.1, 10 warps 95.9, 8 warps 97.6).  A launch of one
+// wave keeps 16 (4096^2 28.1 and 28.5), and so do the inverse (88.6 and 90.3),
+// 5/3 (86.9 and 86.6) and 16-bit storage, which is bound by its arithmetic (78
+// and 80).
+constexpr int kFwdLargeResident = 12;
+constexpr int kFwdLargeSmem = 17920;
+
 // Warps of an inverse launch (1 or 2 fused levels) resident per SM, which its
 // kernel's register budget and the host's waves are sized by: 16 (128
 // registers) with 2 quadruple columns per lane, 12 (168) with 4 (slots of 2

@@ -267,6 +267,7 @@ __device__ __forceinline__ bool inv_body(const CUtensorMap* m1p, const CUtensorM
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
 
+    static_assert(kInvWarps * kInvSlots * (Lay::SLOT * sizeof(S) + 8) <= kSmemBytes, "rings need an opt-in");
     S* ring = reinterpret_cast<S*>(smem_raw) + (size_t)warp * kInvSlots * Lay::SLOT;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + (size_t)kInvWarps * kInvSlots *
                                                               Lay::SLOT * sizeof(S)) +
