@@ -20,7 +20,11 @@
  * scheme runs T_P^H, T_P^V, S_U^H, S_U^V (four barrier steps); the
  * non-separable scheme (Sec. 3) runs the spatial predict T_P and the spatial
  * update S_U (two steps); the reduced form (Sec. 3, P = P0 + P1, U = U0 + U1)
- * computes the same two steps with fewer multiply-accumulates.  CDF 9/7 uses
+ * computes the same two steps with fewer multiply-accumulates.  Where a level
+ * stays on chip the float reduced form goes one further: a neighbour's part of
+ * a spatial step is that neighbour's own result of its vertical half, which is
+ * exchanged instead of computed again (8 multiply-adds per step and quadruple
+ * against 9; the multipass form keeps the paper's split).  CDF 9/7 uses
  * two pairs and a final scaling low / K, high * K per axis
  * (K = 1.230174104914001); reversible LeGall 5/3 uses one integer pair
  * d = x_odd - floor((e_i + e_{i+1})/2), s = x_even + floor((d_{i-1} + d_i + 2)/4),
@@ -102,8 +106,12 @@ typedef enum {
  *   height, width   image size, >= 1 each, at most 65536 each.
  *   levels          1 .. 16.
  *   workspace_bytes receives the size of the device workspace that every
- *                   forward / inverse call on this plan needs (>= 256).  The
- *                   workspace must be zeroed once before first use
+ *                   forward / inverse call on this plan needs (>= 256).  It
+ *                   holds the LL between launches, up to the first level's
+ *                   where that has a launch of its own (dwt2d_plan_options,
+ *                   fuse_max), also if only the inverse is called: 2.5 MiB for
+ *                   1080 x 1920 float32 and 5 levels, 1.0 with fuse_first =
+ *                   fuse_max = 2.  The workspace must be zeroed once before first use
  *                   (dwt2d_workspace_init); one workspace must not be used by
  *                   two calls that run at the same time.
  *   Errors: DWT2D_ERR_INVALID, DWT2D_ERR_UNSUPPORTED, DWT2D_ERR_NOMEM.
@@ -128,14 +136,17 @@ typedef struct {
     int32_t fuse_first;            /* levels fused in the first launch, 1-3 (default 2) */
     int32_t fuse_max;              /* at most per later launch, 1-3 (default 2; 3 runs 4 quadruple
                                       columns per lane; 16-bit storage caps both at 2).  With both
-                                      at 0 a forward float32 level of 512 x 512 to 4 million pixels
-                                      (the first: 7 million) has a launch of its own */
+                                      at 0 a forward float32 CDF 9/7 level of more than 512 x 512 and
+                                      at most 4 million pixels (the first: 7 million) has a launch of
+                                      its own, unless only that takes the workspace past
+                                      DWT2D_NOALLOC_SCRATCH_BYTES (3 levels and more: first levels
+                                      above 6.7 million pixels, images of 26.8 to 33.5 million) */
     int32_t fwd_warps_per_sm;      /* warps a forward launch is cut into, per SM (default 16, 12 where
                                       the kernel has 12 resident; a count that is asked for here or
                                       below is cut as asked, by default segments are made longer to
                                       fill the warps' slots) */
     int32_t inv_warps_per_sm;      /* the same for the inverse (default 16 for 16-bit
-                                      storage, else 12) */
+                                      storage but in plain non-separable steps, else 12) */
     int32_t fwd_warps_per_sm_large;/* forward launches whose row segments stay at least
                                       large_segment rows long at this many warps per SM take it
                                       (default 36 for float32, 32 for 16-bit storage, 64 for
@@ -143,13 +154,14 @@ typedef struct {
                                       also a wave or more fewer where only that gives such
                                       segments; -1: never) */
     int32_t inv_warps_per_sm_large;/* the same for the inverse (default 80 for float32, 48 for
-                                      16-bit storage, 96 for LeGall 5/3 at 2 columns per lane,
-                                      24 at 4; -1: never) */
+                                      16-bit storage, 96 for LeGall 5/3, 36 for the plain
+                                      non-separable CDF 9/7 at 2 columns per lane, 24 at 4; -1:
+                                      never) */
     int32_t large_segment;         /* that threshold, quadruple rows of the launch's last level
                                       (default: forward 13 for 5/3, 17 for float32, 20 for one
-                                      level, 16 to 19 for 4 columns per lane; inverse 20; 16-bit
-                                      storage 40) */
-    int32_t min_segment;           /* shortest row segment of a warp (default 2) */
+                                      level, 16 to 19 for 4 columns per lane; inverse 20, two plain
+                                      non-separable CDF 9/7 levels 32; 16-bit storage 40) */
+    int32_t min_segment;           /* shortest row segment of a warp (default 2; a minimum only) */
     int32_t fwd_seg_interleave;    /* forward segment order: taken in this many interleaved groups
                                       (default: the launch's waves of resident warps; 1: top to
                                       bottom) */

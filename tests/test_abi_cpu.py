@@ -291,3 +291,24 @@ def test_asked_for_decompositions_are_taken(L):
         for key, inverse in (("fwd_warps_per_sm", False), ("inv_warps_per_sm", True)):
             p = D.Plan(2048, 2048, 1, options={key: n, key + "_large": -1})
             assert p.launch_info(inverse)[0][2] == strips * -(-rows // segq), (key, n)
+
+
+@pytest.mark.parametrize("h,w,levels,groups", [
+    (512, 512, 5, [2, 2, 1]), (513, 512, 5, [1, 2, 2]),           # more than 512 x 512 pixels
+    (2640, 2650, 2, [1, 1]), (2646, 2646, 2, [2]),                # the first level: 7 million
+    (8000, 8000, 5, [2, 1, 1, 1]), (8010, 8010, 5, [2, 2, 1]),    # a later one: 4 million
+    # a workspace that only single levels would take past 8 MiB
+    (2500, 2680, 5, [1, 1, 1, 2]), (2500, 2690, 5, [2, 2, 1]),
+    (5000, 5350, 4, [2, 1, 1]), (5000, 5500, 4, [2, 2]), (5790, 5790, 4, [2, 2]),
+    (5800, 5800, 4, [2, 1, 1]),
+])
+def test_which_forward_levels_have_their_own_launch(L, h, w, levels, groups):
+    """Both sides of each limit of the default float32 grouping; the inverse and
+    plans that name their groups keep pairs."""
+    p = D.Plan(h, w, levels)
+    assert [f for f, _q, _w in p.launch_info()] == groups
+    assert max(f for f, _q, _w in p.launch_info(inverse=True)) == 2
+    pairs = D.Plan(h, w, levels, options=dict(fuse_first=2, fuse_max=2))
+    assert [f for f, _q, _w in pairs.launch_info()] == [2] * (levels // 2) + [1] * (levels % 2)
+    if pairs.workspace_bytes <= 8 << 20:
+        assert p.workspace_bytes <= 8 << 20
