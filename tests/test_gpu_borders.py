@@ -211,3 +211,51 @@ def test_nonfinite_pixels_stay_where_they_belong(scheme):
                     y = host(plan.forward(xd, workspace=ws))
                     bad = np.isfinite(ref) & ~np.isfinite(y)
                     assert not bad.any(), (h, w, levels, options, r, c, np.argwhere(bad)[:4].tolist())
+
+
+# 16-bit strips start on 8 elements: 96 / 112 columns (2 / 1 fused levels) with
+# 2 columns per lane, 224 / 240 with 4.  Tolerances of 16-bit storage: a stored
+# value's rounding times the largest gain it passes through.
+TOL_16 = {torch.float16: 2e-3, torch.bfloat16: 1.6e-2}
+
+
+@pytest.mark.parametrize("cols", [2, 4])
+@pytest.mark.parametrize("scheme", ["nonsep_reduced", "separable", "nonsep"])
+@pytest.mark.parametrize("dtype", list(TOL_16))
+def test_strip_edges_of_16bit_storage(dtype, scheme, cols):
+    for w in [2, 3, 5, 8, 9, 17, 95, 96, 97, 98, 111, 112, 113, 114, 191, 192, 193, 194, 223, 224, 225, 226,
+              239, 240, 241]:
+        for h, levels in ((19, 3), (2, 1)):
+            x = make_input("cdf97", h, w, seed=w * 3 + h)
+            xq = torch.from_numpy(x / float(np.max(np.abs(x)))).to(dtype)
+            plan = D.Plan(h, w, levels, "cdf97", scheme, dtype,
+                          options=dict(fwd_cols_per_lane=cols, inv_cols_per_lane=cols))
+            ws = plan.workspace()
+            src = D.empty_image(h, w, dtype)
+            src.copy_(xq)
+            ref = L.forward(xq.to(torch.float64).numpy(), levels, "cdf97")
+            got = host(plan.forward(src, workspace=ws).to(torch.float64))
+            assert float(np.max(np.abs(got - ref))) <= TOL_16[dtype], (h, w, levels)
+            cq = torch.from_numpy(ref).to(dtype)
+            src.copy_(cq)
+            back = L.inverse(cq.to(torch.float64).numpy(), levels, "cdf97")
+            got = host(plan.inverse(src, workspace=ws).to(torch.float64))
+            assert float(np.max(np.abs(got - back))) <= TOL_16[dtype], (h, w, levels, "inverse")
+            assert plan.status(ws) == 0
+
+
+@pytest.mark.parametrize("wavelet,scheme", [("cdf97", "nonsep_reduced"), ("cdf97", "separable"),
+                                            ("cdf97", "nonsep"), ("legall53", "nonsep_reduced")])
+def test_strip_edges_of_three_fused_levels(wavelet, scheme):
+    """Strips of 192 (CDF 9/7) and 224 (5/3) columns, whose halo is 28 and 14."""
+    for w in EDGE_WIDTHS + [27, 28, 29, 57, 191, 192, 193, 194, 219, 220, 221, 383, 384, 385]:
+        for h, levels in ((23, 3), (40, 5)):
+            x = make_input(wavelet, h, w, seed=w * 5 + h)
+            plan = D.Plan(h, w, levels, wavelet, scheme, options=dict(fuse_first=3, fuse_max=3))
+            ws = plan.workspace()
+            tag = f"{wavelet} {scheme} {h}x{w} L{levels}"
+            assert_forward_matches(host(plan.forward(device_image(x), workspace=ws)), x, levels, wavelet, tag)
+            ref = L.forward(x, levels, wavelet).astype(x.dtype)
+            y = plan.inverse(device_image(ref), workspace=ws)
+            assert_inverse_matches(host(y), ref, levels, wavelet, x, tag)
+            assert plan.status(ws) == 0, tag
