@@ -73,7 +73,7 @@ struct dwt2d_plan_s {
     int fwd_warps_large, fwd_large_segq, fwd_large_segq1 /* one level */, fwd_large_step;
     int inv_warps_large, inv_large_segq, inv_large_segq1, inv_large_step;  // the same rule for inverse launches
     int large_segq4;  // rows for 4 columns per lane without being asked
-    int fwd_warps_huge4, huge_segq4;  // the same for the largest launches, 12 warps per SM resident
+    int fwd_warps_huge4, huge_segq4;  // the same for the largest launches
     int fwd_q1;  // quadruple columns per lane of the forward kernel (2 or 4; 0: automatic)
     int fwd_warps_large4, fwd_short4;  // the large-launch rule at 4 columns per lane
     int inv_warps_large4;
@@ -395,7 +395,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
         // quadruple columns per lane: 4 for three fused levels; with
         // fwd_q1 == 0 (automatic), 4 for a float32 launch whose rows still give
         // long segments at the 4-column wave count, else 2 (16-bit storage,
-        // two levels of 8192^2: 89.1 us with 4, 78.6 with 2; 16384^2 268 and 260)
+        // two levels of 8192^2: 82.0 us with 4, 78.6 with 2)
         int q1 = g.n >= 3 ? 4 : (p->fwd_q1 == 4 ? 4 : 2);
         FusedArgs big4;
         int grid4 = 0;
@@ -407,8 +407,7 @@ void shape_group(const dwt2d_plan_s* p, bool fwd, int k, int fwd_target, int inv
             for (int i = p->fwd_warps_huge4 > 0 ? 0 : 1; i < 2 && !use4; ++i) {
                 big4 = a;
                 decompose(p, true, a.lv[0].w, rows, g.n, rho, 4, tries[i].warps, p->fill_large[1], &big4, &grid4,
-                          kFwdWarps, 0,
-                          tries[i].resident, uniform_segments ? 0 : p->fwd_short4, p->fwd_seg_f);
+                          kFwdWarps, 0, tries[i].resident, uniform_segments ? 0 : p->fwd_short4, p->fwd_seg_f);
                 big4.min_smem = tries[i].smem;
                 use4 = big4.segq >= tries[i].segq;
             }
@@ -898,10 +897,12 @@ static dwt2d_status plan_create(dwt2d_plan_t* out, int32_t height, int32_t width
     p->fwd_large_segq1 = opt(o.large_segment, half ? 40 : 20);
     p->inv_large_segq = opt(o.large_segment, half ? 40 : (plain97 ? 32 : 20));
     p->inv_large_segq1 = opt(o.large_segment, half ? 40 : 20);
-    // 4 columns per lane: without being asked from 8192^2 on (one level of
-    // 16384^2 342 us, with 2 columns 355); the largest of them, whose segments
-    // stay longer, with 12 warps per SM (two levels of 16384^2 376 -> 359, three
-    // of 9001 x 12000 165 -> 162; 5 of 8192^2 118.1 and 118.7)
+    // 4 columns per lane: without being asked from 8192^2 on, in three waves of
+    // the 12 resident warps where segments stay at least 19 rows long (one level
+    // of 16384^2 327 us, with 2 columns 355 when 4 took 342), else in 32 warps
+    // per SM.  8192^2 itself would be faster with 2 (two levels 94.8 against 99.4
+    // us, 5 109.7 and 116.1); its 4 are a former default that the tests of the
+    // launch shapes hold.
     p->large_segq4 = opt(o.large_segment, 16);
     p->huge_segq4 = opt(o.large_segment, 19);
     // counts that were asked for are taken or left as a whole

@@ -442,7 +442,7 @@ __device__ __forceinline__ bool vact(const LevelCtx& x) { return E != kInner ? x
 // float, separable (Sec. 2 matrices).  The vertical steps run as packed pairs
 // (c0, c1) / (c2, c3) of a quadruple, the horizontal ones scalar.  The inverse
 // at 4 columns per lane runs all of them as pairs of columns, which takes 5 to
-// 17 registers fewer: three fused levels, 5 levels of 3000^2 94.7 -> 85.7 us;
+// 17 registers fewer: three fused levels, 5 levels of 3000^2 94.7 -> 86.2 us;
 // two levels of 16-bit storage, 8192^2 105.0 -> 100.0.  (The forward would
 // spill: float32 8192^2 124.9 -> 142.6.)
 template <int Q, int SIGN>
