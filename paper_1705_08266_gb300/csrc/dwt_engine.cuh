@@ -271,7 +271,7 @@ struct LevelCtx {
     unsigned left;   // bit j: column j is not column 0
     unsigned odd;    // bit j: column j has odd samples (c1, c3)
     bool need_hsub;  // warp-uniform: some column of this warp lacks its odd samples
-    int ne_r, no_r;  // quadruple rows with an even / an odd image row (no_r: none for one row)
+    int ne_r, no_r;  // quadruple rows with an even / an odd image row
     bool ha, va;     // horizontal / vertical axis longer than 1
     float hf, vf;    // 1.0f if the axis is active, else 0.0f
     float s[4];      // scale of LL, HL, LH, HH (forward) or its inverse (inverse)
@@ -292,10 +292,7 @@ __device__ __forceinline__ LevelCtx make_ctx(int g0, int Q, int h, int w, const 
     const int gw1 = __shfl_sync(kFull, g0, 31) + Q;
     x.need_hsub = (w & 1) && no_c >= gw0 && no_c < gw1;
     x.ne_r = (h + 1) >> 1;
-    // (one row: no quadruple row has an odd one, nor do the rows above it that a
-    // launch of several levels computes before the image, whose odd components
-    // a zero coefficient would not keep out if they were not finite)
-    x.no_r = h > 1 ? h >> 1 : -(1 << 30);
+    x.no_r = h >> 1;
     x.ha = w > 1;
     x.va = h > 1;
     x.hf = x.ha ? 1.0f : 0.0f;
